@@ -1,7 +1,6 @@
-// Memory-bound kernels of the LR-QAT layer: range setting, downcast (Eq. 6/7),
-// merge into integer weights (Sec. 3, after Eq. 8), the per-tensor int8
-// activation quantizer, operand re-layouts for the fused GEMMs, and the
-// deterministic reduction of per-tile gradient partials.
+// Memory-bound kernels of the LR-QAT layer: merge into integer weights (Sec. 3,
+// after Eq. 8), the int8 activation quantizers, operand re-layouts for the fused
+// GEMMs, and the deterministic reduction of per-tile gradient partials.
 #include <cuda_runtime.h>
 #include <cstdint>
 
@@ -16,170 +15,6 @@ constexpr int kThreads = 256;
 inline int blocks_for(int64_t n, int per_block) {
   int64_t b = (n + per_block - 1) / per_block;
   return static_cast<int>(b > 0x7FFFFFFF ? 0x7FFFFFFF : b);
-}
-
-// ------------------------------------------------------------ range setting --
-// One block per (row, group): s0 = max|W0| / p over the segment (1 if all zero).
-__global__ void range_minmax_kernel(const float* __restrict__ W0, int64_t k, int seg, int ngroups, float p,
-                                    float* __restrict__ s0) {
-  const int64_t row = blockIdx.x / ngroups;
-  const int g = blockIdx.x % ngroups;
-  const float* src = W0 + row * k + static_cast<int64_t>(g) * seg;
-  float amax = 0.0f;
-  for (int j = threadIdx.x; j < seg; j += blockDim.x) amax = fmaxf(amax, fabsf(src[j]));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-  __shared__ float warp_max[kThreads / 32];
-  if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = amax;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float a = 0.0f;
-    for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) a = fmaxf(a, warp_max[w]);
-    s0[blockIdx.x] = a > 0.0f ? __fdiv_rn(a, p) : 1.0f;
-  }
-}
-
-// Asymmetric min-max range setting (zero offsets, Eq. 1): per (row, group)
-// s0 = (max - min) / (2^b - 1) in fp32 (1 if max == min) and
-// z0 = clip(round(n - min / s0), n, p), min / s0 one fp32 division, the rest exact.
-__global__ void range_minmax_asym_kernel(const float* __restrict__ W0, int64_t k, int seg, int ngroups, int bits,
-                                         float* __restrict__ s0, float* __restrict__ z0) {
-  const int64_t row = blockIdx.x / ngroups;
-  const int g = blockIdx.x % ngroups;
-  const float* src = W0 + row * k + static_cast<int64_t>(g) * seg;
-  float lo = INFINITY, hi = -INFINITY;
-  for (int j = threadIdx.x; j < seg; j += blockDim.x) {
-    const float v = src[j];
-    lo = fminf(lo, v);
-    hi = fmaxf(hi, v);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-  }
-  __shared__ float warp_lo[kThreads / 32], warp_hi[kThreads / 32];
-  if ((threadIdx.x & 31) == 0) {
-    warp_lo[threadIdx.x >> 5] = lo;
-    warp_hi[threadIdx.x >> 5] = hi;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) {
-      lo = fminf(lo, warp_lo[w]);
-      hi = fmaxf(hi, warp_hi[w]);
-    }
-    const float span = __fsub_rn(hi, lo);
-    const float s = span > 0.0f ? __fdiv_rn(span, static_cast<float>((1 << bits) - 1)) : 1.0f;
-    const double n = -static_cast<double>(1 << (bits - 1)), p = static_cast<double>((1 << (bits - 1)) - 1);
-    const double z = fmin(fmax(rint(n - static_cast<double>(__fdiv_rn(lo, s))), n), p);
-    s0[blockIdx.x] = s;
-    z0[blockIdx.x] = static_cast<float>(z);
-  }
-}
-
-// ----------------------------------------------------------------- downcast --
-// Q-fixed (Eq. 7): round(2^f clip(W0/s0, n, p)) -> int8; 4 elements per thread.
-// With zero offsets z0 (nullable): round(2^f clip(W0/s0 + z0, n, p)), the integer
-// offset added exactly in double precision.
-__global__ void downcast_qfixed_kernel(const float4* __restrict__ W0, const float* __restrict__ s0,
-                                       const float* __restrict__ z0, int64_t k, int group_size, int ngroups,
-                                       float n, float p, float two_f, char4* __restrict__ out, int64_t n4) {
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n4;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t row = (e * 4) / k;
-    const int64_t col = (e * 4) % k;
-    const int64_t sidx = group_size ? row * ngroups + col / group_size : row;
-    const float s = s0[sidx];
-    const float4 w = W0[e];
-    const float x[4] = {w.x, w.y, w.z, w.w};
-    int q[4];
-    if (z0 == nullptr) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float y = fminf(fmaxf(__fdiv_rn(x[i], s), n), p) * two_f;   // exact scaling by 2^f
-        q[i] = __float2int_rn(y);
-      }
-    } else {
-      const double z = z0[sidx];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const double y = fmin(fmax(static_cast<double>(__fdiv_rn(x[i], s)) + z, static_cast<double>(n)),
-                              static_cast<double>(p)) * two_f;
-        q[i] = __double2int_rn(y);
-      }
-    }
-    out[e] = make_char4(static_cast<signed char>(q[0]), static_cast<signed char>(q[1]),
-                        static_cast<signed char>(q[2]), static_cast<signed char>(q[3]));
-  }
-}
-
-// INT-b, double packed: clip(round(W0/s0), n, p), two nibbles per byte; 8 elements per thread.
-// With zero offsets z0 (nullable): clip(round(W0/s0 + z0), n, p).
-__global__ void downcast_packed_kernel(const float4* __restrict__ W0, const float* __restrict__ s0,
-                                       const float* __restrict__ z0, int64_t k, int group_size, int ngroups, int n,
-                                       int p, uint32_t* __restrict__ out, int64_t n8) {
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n8;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t row = (e * 8) / k;
-    const int64_t col = (e * 8) % k;
-    const int64_t sidx = group_size ? row * ngroups + col / group_size : row;
-    const float s = s0[sidx];
-    const double z = z0 != nullptr ? static_cast<double>(z0[sidx]) : 0.0;
-    const float4 w0 = W0[2 * e];
-    const float4 w1 = W0[2 * e + 1];
-    const float x[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-    uint32_t word = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      int c = z0 == nullptr ? __float2int_rn(__fdiv_rn(x[i], s))
-                            : __double2int_rn(static_cast<double>(__fdiv_rn(x[i], s)) + z);
-      c = c < n ? n : (c > p ? p : c);
-      word |= (static_cast<uint32_t>(c) & 0xFu) << (4 * i);
-    }
-    out[e] = word;
-  }
-}
-
-// Floating-point storage (Sec. 3, the cast choices of phi): Phi0 = cast(fl32(W0 / s0))
-// with round-to-nearest-even, no clipping inside phi, FP16 and FP8 saturating at their
-// largest finite value; 4 elements per thread.
-template <int FMT>
-__device__ __forceinline__ uint32_t pack_fp8x2(float lo, float hi) {
-  unsigned short r;
-  if (FMT == FMT_E4M3) asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
-  else asm("cvt.rn.satfinite.e5m2x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-
-// Saturating: values beyond 65504 (which round-to-nearest would turn into infinities)
-// are clamped to it first.
-__device__ __forceinline__ uint32_t pack_sat_f16x2(float lo, float hi) {
-  uint32_t r;
-  lo = fminf(fmaxf(lo, -65504.0f), 65504.0f);
-  hi = fminf(fmaxf(hi, -65504.0f), 65504.0f);
-  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-
-template <int FMT>
-__global__ void downcast_float_kernel(const float4* __restrict__ W0, const float* __restrict__ s0, int64_t k,
-                                      int group_size, int ngroups, void* __restrict__ out, int64_t n4) {
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n4;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t row = (e * 4) / k;
-    const int64_t col = (e * 4) % k;
-    const float s = s0[group_size ? row * ngroups + col / group_size : row];
-    const float4 w = W0[e];
-    const float x0 = __fdiv_rn(w.x, s), x1 = __fdiv_rn(w.y, s), x2 = __fdiv_rn(w.z, s), x3 = __fdiv_rn(w.w, s);
-    if (FMT == FMT_BF16) {
-      static_cast<uint2*>(out)[e] = make_uint2(pack_rn_bf16x2(x0, x1), pack_rn_bf16x2(x2, x3));
-    } else if (FMT == FMT_F16) {
-      static_cast<uint2*>(out)[e] = make_uint2(pack_sat_f16x2(x0, x1), pack_sat_f16x2(x2, x3));
-    } else {
-      static_cast<uint32_t*>(out)[e] = pack_fp8x2<FMT>(x0, x1) | (pack_fp8x2<FMT>(x2, x3) << 16);
-    }
-  }
 }
 
 // 4 stored values of a row -> phi^{-1}(Phi0) in the units of u_f (Eq. 7 / Eq. 8).
@@ -303,18 +138,6 @@ __global__ void __launch_bounds__(kMergeThreads) merge_kernel(const void* __rest
     }
     *reinterpret_cast<uint32_t*>(wz + i * k + j) = out;
   }
-}
-
-// round(fl(x / s)) with fl the IEEE fp32 division, without dividing in the common
-// case: y = x * r with r = fl(1 / s) is within |y| 2^-22 of x / s, and fl(x / s) within
-// |y| 2^-24, so unless y lies within |y| 2^-20 (+ a tiny absolute margin) of a
-// half-integer both round to the same integer; near a half-integer the exact
-// division decides.
-__device__ __forceinline__ float div_round(float x, float s, float r) {
-  const float y = x * r;
-  const float q = rintf(y);
-  if (fabsf(fabsf(y - q) - 0.5f) > fmaxf(fabsf(y), 1.0f) * 9.5367431640625e-07f) return q;   // 2^-20
-  return rintf(__fdiv_rn(x, s));
 }
 
 // --------------------------------------------------------- activation quant --
@@ -514,76 +337,6 @@ __global__ void __launch_bounds__(kThreads) act_quant_token_wide_kernel(const ui
     }
     out[t * k8 + j] = make_uint4(o[0], o[1], o[2], o[3]);
   }
-}
-
-// L^p range setting (symmetric), one block per (row, group): the segment is staged in
-// shared memory, s_max = max|w| / p as in min-max, and thread j < N evaluates the
-// candidate s_j = fl32(s_max (j + 1) / N): loss_j = sum |w - s_j clip(round(w / s_j), n, p)|^p
-// (w / s_j decided as one fp32 division, the error formed with one fused multiply-add,
-// |err|^p by multiplication for integer p).  The smallest loss wins, the smaller j on
-// a tie.
-__global__ void __launch_bounds__(kThreads) range_lp_kernel(const float* __restrict__ W0, int64_t k, int seg,
-                                                            int ngroups, int bits, float p_norm, int n_cand,
-                                                            float* __restrict__ s0) {
-  extern __shared__ float segw[];
-  const int64_t row = blockIdx.x / ngroups;
-  const int g = blockIdx.x % ngroups;
-  const float* src = W0 + row * k + static_cast<int64_t>(g) * seg;
-  float amax = 0.0f;
-  for (int j = threadIdx.x; j < seg; j += blockDim.x) {
-    const float v = src[j];
-    segw[j] = v;
-    amax = fmaxf(amax, fabsf(v));
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-  __shared__ float warp_max[kThreads / 32];
-  __shared__ float best_loss[kThreads];
-  __shared__ int best_j[kThreads];
-  if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = amax;
-  __syncthreads();
-  float a = 0.0f;
-  for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) a = fmaxf(a, warp_max[w]);
-  const float pmax = static_cast<float>((1 << (bits - 1)) - 1), nmin = -static_cast<float>(1 << (bits - 1));
-  const float s_max = a > 0.0f ? __fdiv_rn(a, pmax) : 1.0f;
-  const int j = threadIdx.x;
-  float loss = INFINITY;
-  if (j < n_cand) {
-    const float s = static_cast<float>(static_cast<double>(s_max) * (j + 1) / n_cand);
-    const float r = __frcp_rn(s);
-    const int ip = static_cast<int>(p_norm);
-    const bool int_p = static_cast<float>(ip) == p_norm && ip >= 1 && ip <= 8;
-    float acc0 = 0.0f, acc1 = 0.0f;
-    for (int e = 0; e < seg; ++e) {
-      const float w = segw[e];
-      const float q = fminf(fmaxf(div_round(w, s, r), nmin), pmax);
-      const float err = fabsf(fmaf(-s, q, w));
-      float t;
-      if (int_p) {
-        t = err;
-        for (int i = 1; i < ip; ++i) t *= err;
-      } else {
-        t = err > 0.0f ? powf(err, p_norm) : 0.0f;
-      }
-      if (e & 1) acc1 += t; else acc0 += t;
-    }
-    loss = acc0 + acc1;
-  }
-  best_loss[threadIdx.x] = loss;
-  best_j[threadIdx.x] = j;
-  __syncthreads();
-  for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-    if (static_cast<int>(threadIdx.x) < h) {
-      const float lo = best_loss[threadIdx.x + h];
-      const int jo = best_j[threadIdx.x + h];
-      if (lo < best_loss[threadIdx.x] || (lo == best_loss[threadIdx.x] && jo < best_j[threadIdx.x])) {
-        best_loss[threadIdx.x] = lo;
-        best_j[threadIdx.x] = jo;
-      }
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) s0[blockIdx.x] = static_cast<float>(static_cast<double>(s_max) * (best_j[0] + 1) / n_cand);
 }
 
 // ---------------------------------------------------------------- re-layouts --
@@ -987,65 +740,6 @@ __global__ void __launch_bounds__(kThreads) reduce_grads_kernel(RedJob ja, RedJo
 }
 
 }  // namespace
-
-cudaError_t launch_range_minmax(const float* W0, int64_t m, int64_t k, int group_size, int bits, float* s0,
-                                float* z0, cudaStream_t stream) {
-  const int ngroups = group_size ? static_cast<int>(k / group_size) : 1;
-  const int seg = group_size ? group_size : static_cast<int>(k);
-  const unsigned grid = static_cast<unsigned>(m * ngroups);
-  if (z0 == nullptr) {
-    range_minmax_kernel<<<grid, kThreads, 0, stream>>>(W0, k, seg, ngroups,
-                                                       static_cast<float>((1 << (bits - 1)) - 1), s0);
-  } else {
-    range_minmax_asym_kernel<<<grid, kThreads, 0, stream>>>(W0, k, seg, ngroups, bits, s0, z0);
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_range_lp(const float* W0, int64_t m, int64_t k, int group_size, int bits, float p_norm, int n_cand,
-                            float* s0, cudaStream_t stream) {
-  const int ngroups = group_size ? static_cast<int>(k / group_size) : 1;
-  const int seg = group_size ? group_size : static_cast<int>(k);
-  const size_t smem = static_cast<size_t>(seg) * 4;
-  if (n_cand < 1 || n_cand > kThreads || smem > 200 * 1024) return cudaErrorInvalidValue;
-  if (smem > 48 * 1024) {
-    // the largest row or group any call may need (200 KB), set once per device
-    static bool configured[kMaxDevices] = {};
-    const cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(range_lp_kernel), 200 * 1024, configured);
-    if (e != cudaSuccess) return e;
-  }
-  range_lp_kernel<<<static_cast<unsigned>(m * ngroups), kThreads, smem, stream>>>(W0, k, seg, ngroups, bits, p_norm,
-                                                                                 n_cand, s0);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_downcast(const float* W0, const float* s0, const float* z0, int64_t m, int64_t k, int group_size,
-                            int bits, int fmt, void* phi0, cudaStream_t stream) {
-  const int ngroups = group_size ? static_cast<int>(k / group_size) : 1;
-  const int n = -(1 << (bits - 1)), p = (1 << (bits - 1)) - 1;
-  if (fmt_float(fmt)) {
-    if (z0 != nullptr) return cudaErrorInvalidValue;
-    const int64_t n4 = m * k / 4;
-    const unsigned grid = blocks_for(n4, kThreads);
-    const float4* w4 = reinterpret_cast<const float4*>(W0);
-    auto kernel = fmt == FMT_BF16   ? downcast_float_kernel<FMT_BF16>
-                  : fmt == FMT_F16  ? downcast_float_kernel<FMT_F16>
-                  : fmt == FMT_E4M3 ? downcast_float_kernel<FMT_E4M3>
-                                    : downcast_float_kernel<FMT_E5M2>;
-    kernel<<<grid, kThreads, 0, stream>>>(w4, s0, k, group_size, ngroups, phi0, n4);
-  } else if (fmt == FMT_Q8) {
-    const int64_t n4 = m * k / 4;
-    downcast_qfixed_kernel<<<blocks_for(n4, kThreads), kThreads, 0, stream>>>(
-        reinterpret_cast<const float4*>(W0), s0, z0, k, group_size, ngroups, static_cast<float>(n),
-        static_cast<float>(p), static_cast<float>(1 << (8 - bits)), static_cast<char4*>(phi0), n4);
-  } else {
-    const int64_t n8 = m * k / 8;
-    downcast_packed_kernel<<<blocks_for(n8, kThreads), kThreads, 0, stream>>>(
-        reinterpret_cast<const float4*>(W0), s0, z0, k, group_size, ngroups, n, p, static_cast<uint32_t*>(phi0),
-        n8);
-  }
-  return cudaGetLastError();
-}
 
 cudaError_t launch_merge(const void* phi0, const uint16_t* A, const uint16_t* B, int64_t m, int64_t k, int r,
                          int fmt, int u_bf16, const QuantParams& q, int8_t* wz, cudaStream_t stream) {

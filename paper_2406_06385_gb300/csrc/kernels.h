@@ -29,16 +29,18 @@ inline cudaError_t ensure_smem_attr(const void* kernel, int bytes, bool* done) {
   return cudaSuccess;
 }
 
-// ---- elementwise.cu --------------------------------------------------------
+// ---- range.cu --------------------------------------------------------------
 // z0 == nullptr: symmetric range setting (s0 only); else asymmetric (s0 and zero offsets z0).
 cudaError_t launch_range_minmax(const float* W0, int64_t m, int64_t k, int group_size, int bits, float* s0,
                                 float* z0, cudaStream_t stream);
 // L^p range setting over N scaled min-max candidates (symmetric grids).
 cudaError_t launch_range_lp(const float* W0, int64_t m, int64_t k, int group_size, int bits, float p_norm, int n_cand,
-                            float* s0, cudaStream_t stream);
+                            float* s0, int sms, cudaStream_t stream);
 // fmt: a PhiFmt value (quant.cuh); zero offsets z0 only with the integer formats.
 cudaError_t launch_downcast(const float* W0, const float* s0, const float* z0, int64_t m, int64_t k, int group_size,
                             int bits, int fmt, void* phi0, cudaStream_t stream);
+
+// ---- elementwise.cu --------------------------------------------------------
 cudaError_t launch_merge(const void* phi0, const uint16_t* A, const uint16_t* B, int64_t m, int64_t k, int r,
                          int fmt, int u_bf16, const QuantParams& q, int8_t* wz, cudaStream_t stream);
 // codes = clip(round(X / s_x), -128, 127) as bf16; optional mask bits [k][ceil(T/32)].

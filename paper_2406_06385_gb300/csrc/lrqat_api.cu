@@ -648,8 +648,10 @@ int lrqat_range_lp(const lrqat_layer* layer, const float* W0, float p_norm, int3
     return fail(LRQAT_ERR_INVALID_ARG, "n_candidates must be in [1, 256] (got %d)", n_candidates);
   const int64_t seg = L.group_size ? L.group_size : L.k;
   if (seg * 4 > 200 * 1024) return fail(LRQAT_ERR_UNSUPPORTED, "row or group of %lld values too long", (long long)seg);
+  DeviceInfo* dev = nullptr;
+  LRQAT_TRY(device_info(&dev));
   LRQAT_LAUNCH("range_lp", 1, stream,
-               launch_range_lp(W0, L.m, L.k, L.group_size, L.bits, p_norm, n_candidates, s0, stream),
+               launch_range_lp(W0, L.m, L.k, L.group_size, L.bits, p_norm, n_candidates, s0, dev->sms, stream),
                "range_lp launch");
   return LRQAT_OK;
 }
