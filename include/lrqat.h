@@ -33,9 +33,8 @@
  *     low-rank tile (alpha/r) A B next to the main product; otherwise one
  *     tensor-core pass per call first writes one byte per weight into the
  *     workspace, the clipped code c = clip(round(u), n, p) biased by 64 (128 for
- *     8-bit weights) where only the forward and dX GEMMs read it, or the
- *     unclipped round(u) saturated to [-128, 127] (which keeps the clip mask)
- *     where the weight-gradient kernel needs the mask too (ranks above 64); the
+ *     8-bit weights), which for the weight-gradient kernel carries the clip mask in
+ *     its top bit (weights of up to 7 bits); the
  *     GEMMs then turn those bytes into W_hat on chip.  The results are the same
  *     codes, gradients and outputs.
  */
@@ -336,8 +335,9 @@ int lrqat_set_gemm_variant(int variant);
  * GEMMs read those bytes as their base, with no low-rank work in the stage; 0 (the default)
  * = codes from 3072 tokens
  * on, the tile below (the pass costs two bytes of HBM traffic per weight, the tile a low-rank
- * MMA chain per stage).  Ranks above 64 always take the codes pass.  dW is unaffected: it
- * computes its own low-rank tile for ranks up to 64.  All settings give the same codes up to
+ * MMA chain per stage).  Ranks above 64 always take the codes pass.  dW reads the codes where
+ * the pair kernels take it (m and k multiples of 256, up to 7 bits) and computes its own
+ * low-rank tile elsewhere.  All settings give the same codes up to
  * fp32 summation order of A B.  Process-wide; the environment variable LRQAT_LOWRANK_PATH
  * ("auto", "tile" or "codes") gives the start value, read once when the library is loaded.
  * Returns LRQAT_ERR_INVALID_ARG for other values. */

@@ -19,8 +19,8 @@
 // stages with TMA.  Work units (row block, column tile, token split) are
 // distributed persistently over the CTAs.
 //
-// Ranks above 64 (NL): the base holds the unclipped codes round(u), low-rank term
-// included (the tensor-core code pass writes them once per call), so no low-rank tile
+// Ranks above 64 (NL; shapes or schedules that the pair kernel dw_codes.cu does not take): the
+// base holds the code bytes of the codes pass (c + 64, bit 7 the clip mask), so no low-rank tile
 // is computed, and the tiles are 128 columns wide.  The adapter contractions run in
 // rounds of 64 rank indices: per round the slices A^T[64 ranks, 128 rows] and B[64
 // ranks, 128 columns] land in the epilogue buffers, tcgen05 computes that round's 64
@@ -173,7 +173,7 @@ __device__ __forceinline__ bool work_next(WorkIter& it, const DwArgs& a, Unit& x
 }
 
 // UB: pre-round value in bf16 (u_bf16x2) instead of one fp32 FMA.
-// NL: the base holds the unclipped codes (FMT_Q8, 0 fraction bits), no low-rank tile,
+// NL: the base holds the code bytes (FMT_Q8), no low-rank tile,
 // 128-column tiles, adapter contractions in rounds of 64 ranks.
 template <int FMT, bool ZP, bool UB, bool NL>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
@@ -512,16 +512,31 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             const uint4 r1 = ld_shared_v4(smem + OFF_PHI + swz_offset(row, jl / 16 + 1, 128));
             raw[0] = r0.x, raw[1] = r0.y, raw[2] = r0.z, raw[3] = r0.w;
             raw[4] = r1.x, raw[5] = r1.y, raw[6] = r1.z, raw[7] = r1.w;
-            decode16<FMT>(raw, v);
-            decode16<FMT>(raw + 4, v + 16);
+            if (NL) {
+#pragma unroll
+              for (int e = 0; e < 8; ++e) {
+                float2 c01, c23;
+                decode_codes4(raw[e], c01, c23);
+                v[4 * e] = c01.x, v[4 * e + 1] = c01.y, v[4 * e + 2] = c23.x, v[4 * e + 3] = c23.y;
+              }
+            } else {
+              decode16<FMT>(raw, v);
+              decode16<FMT>(raw + 4, v + 16);
+            }
           }
           uint32_t du[16];
 #pragma unroll
           for (int e = 0; e < 16; ++e) {
             const float2 g2 = make_float2(G[2 * e], G[2 * e + 1]);
+            if (NL) {   // the code and its mask come from the code byte
+              const float2 c2 = make_float2(v[2 * e], v[2 * e + 1]);
+              ds2 = __ffma2_rn(g2, ZP ? __fadd2_rn(c2, make_float2(-z_i, -z_i)) : c2, ds2);
+              const float2 gs = __fmul2_rn(g2, make_float2(gs_i, gs_i));
+              du[e] = pack_rn_bf16x2(gs.x, gs.y) & ((e & 1) ? code_masks2<1>(raw[e >> 1]) : code_masks2<0>(raw[e >> 1]));
+              continue;
+            }
             const float2 v2 = make_float2(v[2 * e], v[2 * e + 1]);
-            const float2 u2 = NL   ? v2
-                              : UB ? u_bf16x2(Lv[2 * e], Lv[2 * e + 1], v2.x, v2.y, lr2)
+            const float2 u2 = UB ? u_bf16x2(Lv[2 * e], Lv[2 * e + 1], v2.x, v2.y, lr2)
                                    : __ffma2_rn(make_float2(Lv[2 * e], Lv[2 * e + 1]),
                                                 make_float2(qp.lr_scale, qp.lr_scale), v2);
             const float2 t2 = __fadd2_rn(u2, make_float2(qp.magic, qp.magic));

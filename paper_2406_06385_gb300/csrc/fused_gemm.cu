@@ -29,9 +29,8 @@
 // Large 128-byte-row boxes matter: an SM's TMA throughput falls with the number
 // of boxes it processes, and loads issued by one warp are handled one at a time,
 // hence one loader warp per ring slot of the token operand.
-// Ranks above 64 (NL): the base operand already holds the codes round(u) of Eq. 8,
-// low-rank term included (written once per call by the tensor-core code pass), so no
-// factor is loaded and no low-rank tile is computed; the producers clip, (scale) and
+// On the codes (NL): the base operand holds the biased codes of Eq. 8 that the codes pass
+// wrote, so no factor is loaded and no low-rank tile is computed; the producers (scale and)
 // store W_hat from the base alone.
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -120,7 +119,7 @@ __device__ __forceinline__ void drain_wait(uint32_t bar, uint32_t parity, uint64
 // even number of slices, so stage gg uses token slot gg % 2 for the (gg / 2)-th
 // time and factor slot gg % NF for the (gg / NF)-th time.
 // UB: pre-round value in bf16 (u_bf16x2) instead of one fp32 FMA.
-// NL: no low-rank term (the base holds the unclipped codes, FMT_Q8 with 0 fraction bits).
+// NL: no low-rank term (the base holds the biased codes of the codes pass).
 template <int MODE, int FMT, bool ZP, bool UB, bool NL>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     fused_gemm_kernel(const __grid_constant__ CUtensorMap tm_tok, const __grid_constant__ CUtensorMap tm_phi,
@@ -403,7 +402,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         if (b64) {
 #pragma unroll
           for (int i = 0; i < 4; ++i) decode_b64_bf16x4(raw[i], c8[2 * i], c8[2 * i + 1]);
-        } else if (NL && args.codes_bias == 128) {
+        } else if (NL) {
           decode_ob16(raw, v);
         } else {
           decode16<FMT>(raw, v);
@@ -424,9 +423,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         for (int e = 0; e < 8; ++e) {
           uint32_t cw;
           if (NL) {
-            cw = b64                         ? c8[e]
-                 : args.codes_bias == 128    ? pack_int_bf16x2(v[2 * e], v[2 * e + 1])
-                                             : int_codes_bf16x2(v[2 * e], v[2 * e + 1], qp);
+            cw = b64 ? c8[e] : pack_int_bf16x2(v[2 * e], v[2 * e + 1]);
           } else {
             const float2 u = UB ? u_bf16x2(Lv[2 * e], Lv[2 * e + 1], v[2 * e], v[2 * e + 1], lr2)
                                 : __ffma2_rn(make_float2(Lv[2 * e], Lv[2 * e + 1]),

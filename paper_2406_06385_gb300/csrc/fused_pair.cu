@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           if (b64) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) decode_b64_bf16x4(raw[j][i], c8[2 * i], c8[2 * i + 1]);
-          } else if (NL && args.codes_bias == 128) {
+          } else if (NL) {
             decode_ob16(raw[j], v);
           } else {
             decode16<FMT>(raw[j], v);
@@ -473,9 +473,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           for (int e = 0; e < 8; ++e) {
             uint32_t cw;
             if (NL) {
-              cw = b64                         ? c8[e]
-                   : args.codes_bias == 128    ? pack_int_bf16x2(v[2 * e], v[2 * e + 1])
-                                               : int_codes_bf16x2(v[2 * e], v[2 * e + 1], qp);
+              cw = b64 ? c8[e] : pack_int_bf16x2(v[2 * e], v[2 * e + 1]);
             } else {
               const float2 u = UB ? u_bf16x2(Lv[2 * e], Lv[2 * e + 1], v[2 * e], v[2 * e + 1], lr2)
                                   : __ffma2_rn(make_float2(Lv[2 * e], Lv[2 * e + 1]),

@@ -58,11 +58,10 @@ cudaError_t launch_adapter_layouts(const uint16_t* A, const uint16_t* B, int64_t
 // The backward's preparation in one launch: the adapter layouts (as launch_adapter_layouts)
 // and phi_t[j][i] = stored value of Phi0[i][j]: the raw byte (Q-fixed, FP8), the
 // sign-extended nibble as an int8 (packed INT-b), or the raw 16-bit pattern (BF16, FP16);
-// phi_t [k, m].  clip_bits > 0 (int8 codes only): each value is clamped to the signed
-// clip_bits-bit grid and biased by 64 on the way (the GEMMs' clip(c) + 64 codes).
+// phi_t [k, m].
 cudaError_t launch_bwd_prep(const uint16_t* A, const uint16_t* B, int64_t m, int64_t k, int r, int r16,
                             uint16_t* A_pad, uint16_t* Bt_pad, uint16_t* At, uint16_t* B_pad, const void* phi0,
-                            int fmt, void* phi_t, cudaStream_t stream, int clip_bits = 0);
+                            int fmt, void* phi_t, cudaStream_t stream);
 // Schedule of the dW work over its persistent CTAs.  The work is ni x nj tiles (128 rows i x
 // 128 * nchunks columns j; tile = ib + ni * jt) of tsteps 32-token stages each; G and the
 // gradients it feeds (dU, dA, dB, ds) are linear in the tokens, so any token range of a tile
@@ -144,7 +143,7 @@ struct FusedArgs {
   int32_t kdim;          // contraction length (k for fwd, m for dX)
   int32_t T;             // tokens
   int32_t r16;           // adapter rank rounded up to 16; 0: no low-rank term (the base holds
-                         // the unclipped int8 codes round(u), written for ranks above 64)
+                         // the biased codes of the codes pass)
   int32_t sf_cols;       // columns of the second factor loaded per stage (16, 32 or 64)
   int32_t num_rb;        // rows / 128
   int32_t num_tb;        // ceil(T / 448)
@@ -166,8 +165,8 @@ struct FusedArgs {
   // Forward only: the second factor's slice read straight from B as one MN-major box
   // of 64 columns x r16 rank rows (no padded B^T copy).
   int32_t sf_mn;
-  // Codes base (r16 == 0): 0: saturated int8 codes (the producers clamp them); 64 or 128: the
-  // codes clipped to [n, p] and stored as the unsigned byte c + 64 (b <= 7) or c + 128 (b = 8).
+  // Codes base (r16 == 0): the codes are stored as the unsigned byte c + codes_bias, 64 (b <= 7)
+  // or 128 (b = 8).
   int32_t codes_bias;
   // dX only: the scales (and zero offsets, or nullptr) as bf16 rows along the contraction,
   // [groups][kdim] (one row per channel scale), written by launch_dx_scales.
@@ -207,8 +206,8 @@ struct DwArgs {
   int32_t u_bf16;        // pre-round value in bf16 (lrqat_layer.u_bf16)
   DwSched sched;         // kept last (argument layout)
   int32_t* tile_segs;    // tail schedule: [ni * nj] slots written per tile
-  // Ranks above 64: the base (tm_phi) holds the unclipped int8 codes round(u), low-rank
-  // term included; no low-rank tile, nchunks == 1, tm_at / tm_b boxes of 64 rank rows.
+  // Ranks above 64: the base (tm_phi) holds the code bytes (c + 64, bit 7 the clip mask); no
+  // low-rank tile, nchunks == 1, tm_at / tm_b boxes of 64 rank rows.
   int32_t codes_base;
 };
 int dw_smem_bytes(int r16, int fmt);
@@ -219,6 +218,11 @@ int dw_smem_bytes(int r16, int fmt);
 cudaError_t launch_dw_pair(int fmt, const CUtensorMap& tm_dy, const CUtensorMap& tm_x, const CUtensorMap& tm_at,
                            const CUtensorMap& tm_ath, const CUtensorMap& tm_phi, const CUtensorMap& tm_b,
                            const CUtensorMap& tm_bh, const DwArgs& args, int npairs, cudaStream_t stream);
+// The pair kernel on the codes (dw_codes.cu), any rank up to 256: args.phi holds the code bytes
+// [m, k] (c + 64, bit 7 the clip mask); tm_at boxes of min(r16, 64) rank rows, tm_b of half as many;
+// ranks above 64 take equal token splits only.
+cudaError_t launch_dw_codes(const CUtensorMap& tm_dy, const CUtensorMap& tm_x, const CUtensorMap& tm_at,
+                            const CUtensorMap& tm_b, const DwArgs& args, int npairs, cudaStream_t stream);
 // Clusters of two of the pair dW kernel that can be resident at once on the current device
 // (0 when the query fails).
 int dw_pair_max_pairs();

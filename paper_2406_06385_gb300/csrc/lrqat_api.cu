@@ -109,6 +109,9 @@ CUtensorMapSwizzle sf_swizzle(int r16) {
   return c == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : c == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
 }
 
+// Rank columns of the codes pass's K-major A boxes (merge.cu): r16 for 16 and 32, else 64.
+uint32_t a_cols(int r16) { return r16 <= 32 ? static_cast<uint32_t>(r16) : 64u; }
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // The fused GEMMs read the factors straight from the caller's A [m, r] and B [r, k] when
@@ -123,9 +126,8 @@ int frac_bits(const lrqat_layer& L) { return L.phi_format == LRQAT_PHI_QFIXED ? 
 
 // Where the forward and dX GEMMs take the low-rank term from (lrqat_set_lowrank_path):
 // 1 = the tile that each GEMM stage computes next to the main product (ranks up to 64);
-// 2 = the codes pass: one tensor-core pass per call writes the unclipped codes round(u) of every
-// weight (int8, saturated) into the workspace, and the GEMMs read them as their base with the
-// low-rank term switched off.  In the pair GEMM the in-stage tile is a chain of small MMAs
+// 2 = the codes pass: one tensor-core pass per call writes the code of every weight as a byte into
+// the workspace, and the GEMMs read those as their base with the low-rank term switched off.  In the pair GEMM the in-stage tile is a chain of small MMAs
 // whose TMEM buffer holds one stage, so it paces the stage (measured on a 4096 x 4096 layer at
 // T = 8192: forward 218 -> 191 us, dX 254 -> 210 us with the codes, for a pass of 18 us), while
 // the pass moves ~2 bytes per weight through HBM whatever T is.  Measured fwd + bwd per call,
@@ -142,7 +144,6 @@ int lowrank_path_from_env() {
 }
 std::atomic<int> g_lowrank_path{lowrank_path_from_env()};
 constexpr int64_t kCodesMinTokens = 3072;
-bool codes_dw(const lrqat_layer& L) { return L.r > 64; }
 bool codes_gemm(const lrqat_layer& L, int64_t T) {
   if (L.r > 64) return true;
   const int v = g_lowrank_path.load(std::memory_order_relaxed);
@@ -179,7 +180,7 @@ int validate_layer(const lrqat_layer* L) {
   if (L->group_size > 0 && (L->group_size % 128 || L->k % L->group_size))
     return fail(LRQAT_ERR_UNSUPPORTED, "group_size %d must be a multiple of 128 dividing k", L->group_size);
   if (L->r > 64 && L->bits > 7)
-    return fail(LRQAT_ERR_UNSUPPORTED, "ranks above 64 need bits <= 7 (the unclipped codes are kept as int8)");
+    return fail(LRQAT_ERR_UNSUPPORTED, "ranks above 64 need bits <= 7 (the code byte holds the clip mask)");
   if (L->act_bits != 0 && L->act_bits != 8)
     return fail(LRQAT_ERR_UNSUPPORTED, "act_bits must be 0 or 8 (got %d)", L->act_bits);
   if (L->zero && !aligned16(L->zero)) return fail(LRQAT_ERR_ALIGNMENT, "zero (offsets) is not 16-byte aligned");
@@ -324,9 +325,10 @@ constexpr int kPairTokens = 448;   // tokens per pair tile (two accumulators of 
 constexpr int kDwPairTokensPerStage = 64;   // the pair dW kernel's stage (dw_pair.cu)
 // dW on CTA pairs (dw_pair.cu): 256 x 256 tiles, ranks up to 64, by the same setting as the
 // forward and dX GEMMs (lrqat_set_gemm_variant: not with 1, the one-SM kernels).
-bool use_pair_dw(const lrqat_layer& L) {
-  return L.m % 256 == 0 && L.k % 256 == 0 && !codes_dw(L) && g_gemm_variant.load(std::memory_order_relaxed) != 1;
+bool pair_dw_shape(const lrqat_layer& L) {
+  return L.m % 256 == 0 && L.k % 256 == 0 && g_gemm_variant.load(std::memory_order_relaxed) != 1;
 }
+bool use_pair_dw(const lrqat_layer& L) { return pair_dw_shape(L) && L.r <= 64; }
 
 struct DwPlan {
   int nchunks, ni, nj, nsplit, tchunk, units;
@@ -341,7 +343,7 @@ struct DwPlan {
 DwPlan plan_dw(const lrqat_layer& L, int64_t T, int sms, bool pair) {
   DwPlan p;
   p.pair = pair;
-  p.nchunks = (L.k % 256 == 0 && !codes_dw(L)) ? 2 : 1;
+  p.nchunks = (L.k % 256 == 0 && L.r <= 64) ? 2 : 1;
   p.ni128 = static_cast<int>(L.m / 128);
   p.ni = static_cast<int>(pair ? L.m / 256 : L.m / 128);
   p.nj = static_cast<int>(L.k / (128 * p.nchunks));
@@ -397,6 +399,27 @@ DwPlan plan_dw(const lrqat_layer& L, int64_t T, int sms, bool pair) {
   return p;
 }
 
+// The plan of a layer's dW on the current device (pairs: the pair kernels' resident clusters).
+// Ranks above 64 are planned as 128 x 128 tiles of 32-token stages over the SMs; where that plan
+// has equal token splits and the shape allows, the pair kernel on the codes takes the same splits
+// in 256 x 256 tiles, so every G has the same tokens in the same order.  A pair tile's stage costs
+// about as much as a 128 x 128 tile's, so pairs are taken when their rounds are no more.
+DwPlan plan_layer_dw(const lrqat_layer& L, int64_t T, int sms, int pairs) {
+  if (use_pair_dw(L)) return plan_dw(L, T, pairs, true);
+  DwPlan p = plan_dw(L, T, sms, false);
+  if (L.r <= 64 || p.sched.tail || !pair_dw_shape(L) || pairs < 1) return p;
+  const int64_t tiles = (L.m / 256) * (L.k / 256), units = tiles * p.nsplit;
+  if ((units + pairs - 1) / pairs > (p.units + sms - 1) / sms) return p;
+  p.pair = true;
+  p.nchunks = 2;
+  p.ni = static_cast<int>(L.m / 256);
+  p.nj = static_cast<int>(L.k / 256);
+  p.bkt = kDwPairTokensPerStage;
+  p.units = static_cast<int>(units);
+  p.sched = DwSched{0, static_cast<int32_t>(units < pairs ? units : pairs), (T + p.bkt - 1) / p.bkt, 0, 0, 0};
+  return p;
+}
+
 struct FwdWs {
   uint16_t* a_pad;
   uint16_t* bt_pad;
@@ -444,7 +467,7 @@ struct BwdWs {
   float* dB_part;
   float* ds_part;
   int32_t* tile_segs;
-  int8_t* codes;       // codes path: the unclipped codes [m, k] (phit then holds their transpose)
+  int8_t* codes;       // codes path: dW's code bytes [m, k] (phit then holds the transposed codes)
   uint16_t* s_bf16;    // dX: the scales (and zero offsets) as bf16 rows [groups][m]
   uint16_t* z_bf16;
 };
@@ -493,29 +516,28 @@ int phi_map(CUtensorMap* map, const lrqat_layer& L, const void* phi0, uint32_t b
                    dw ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B, "Phi0 (packed)");
 }
 
-// Quantizer constants of the codes written for ranks above 64: the clamp bounds are the int8
-// range instead of [n, p] (the GEMMs clip and mask from the unclipped code).
 // The bias of the clipped codes the GEMMs read (merge.h, FusedArgs::codes_bias): c + 64 fits a
 // byte's low seven bits for b <= 7 (the GEMM producers then turn four codes into bf16 with two
 // byte permutes and two bf16 subtractions), c + 128 for b = 8.
 uint32_t codes_bias(const lrqat_layer& L) { return L.bits <= 7 ? 64u : 128u; }
 
-QuantParams saturating_params(const lrqat_layer& L) {
-  QuantParams q = make_quant_params(L.bits, frac_bits(L), L.alpha, L.r);
-  const QuantParams wide = make_quant_params(8, frac_bits(L), L.alpha, L.r);
-  q.lo = wide.lo;
-  q.hi = wide.hi;
-  return q;
-}
+// What the codes pass writes besides the codes themselves (merge.h).
+struct CodesOut {
+  int8_t* row_major;   // [m, k], or nullptr
+  bool mask;           // row_major: the clip mask in bit 7 (dW)
+  int8_t* transposed;  // [k, m], or nullptr
+  const float* s;      // bf16 scale rows [groups][m] into s_bf16 (and z_bf16), or s_bf16 == nullptr
+  uint16_t* s_bf16;
+  uint16_t* z_bf16;
+  uint16_t* at;        // A^T [r16, m] (direct factors only), or nullptr
+};
 
-// The codes pass: codes[i, j] = sat8(round(phi^{-1}(Phi0[i, j]) + (alpha/r) (A B)[i, j])) on the
-// tensor cores (any rank up to 256), from A [m, r] and B [r, k] themselves when the factors are
-// direct (rank a multiple of 8, 16-byte aligned: TMA boxes past r read as zeros), else from the
-// zero-padded A^T [r16, m] and B [r16, k].  clipped: the codes clip(round(u), n, p) plus the bias
-// (codes_bias) instead, for when only the forward and dX GEMMs read them (dW of ranks above 64
-// needs the unclipped codes for its mask).
+// The codes pass: clip(round(phi^{-1}(Phi0) + (alpha/r) A B), n, p) plus the bias (codes_bias) of
+// every weight on the tensor cores (any rank up to 256), from A [m, r] and B [r, k] themselves when
+// the factors are direct (rank a multiple of 8, 16-byte aligned: TMA boxes past r read as zeros),
+// else from the zero-padded A^T [r16, m] and B [r16, k].
 int run_codes_pass(const lrqat_layer& L, const void* Phi0, const uint16_t* A, const uint16_t* B, const uint16_t* At,
-                   const uint16_t* B_pad, int8_t* codes, bool clipped, const DeviceInfo* dev, cudaStream_t stream);
+                   const uint16_t* B_pad, const CodesOut& out, const DeviceInfo* dev, cudaStream_t stream);
 
 }  // namespace
 }  // namespace lrqat
@@ -556,13 +578,13 @@ int noalloc_scratch(void** out) {
 
 namespace {
 int run_codes_pass(const lrqat_layer& L, const void* Phi0, const uint16_t* A, const uint16_t* B, const uint16_t* At,
-                   const uint16_t* B_pad, int8_t* codes, bool clipped, const DeviceInfo* dev, cudaStream_t stream) {
+                   const uint16_t* B_pad, const CodesOut& out, const DeviceInfo* dev, cudaStream_t stream) {
   const int r16 = round16(L.r);
   const bool direct = direct_factors(L, A, B);
   CUtensorMap tm_a, tm_b;
   if (direct) {
-    LRQAT_TRY(encode_2d(&tm_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, A, L.r, L.m, L.r * 2, 64, 128,
-                        CU_TENSOR_MAP_SWIZZLE_128B, "A"));
+    LRQAT_TRY(encode_2d(&tm_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, A, L.r, L.m, L.r * 2, a_cols(r16), 128,
+                        sf_swizzle(r16), "A"));
     LRQAT_TRY(encode_2d(&tm_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, B, L.k, L.r, L.k * 2, 64,
                         static_cast<uint32_t>(r16), CU_TENSOR_MAP_SWIZZLE_128B, "B"));
   } else {
@@ -574,12 +596,27 @@ int run_codes_pass(const lrqat_layer& L, const void* Phi0, const uint16_t* A, co
   CUtensorMap tm_phi;
   LRQAT_TRY(phi_map(&tm_phi, L, Phi0, 128, true));
   MergeArgs a{};
-  a.wz = codes;
+  a.wz = out.row_major;
+  a.wt = out.transposed;
   a.m = L.m;
   a.k = L.k;
   a.r16 = r16;
-  a.q = clipped ? make_quant_params(L.bits, frac_bits(L), L.alpha, L.r) : saturating_params(L);
-  a.code_bias = clipped ? codes_bias(L) : 0u;
+  a.q = make_quant_params(L.bits, frac_bits(L), L.alpha, L.r);
+  a.code_bias = codes_bias(L);
+  a.bits = L.bits;
+  a.mask_bit = out.mask ? 1 : 0;
+  if (out.s_bf16) {
+    a.s = out.s;
+    a.z = L.zero;
+    a.s_out = out.s_bf16;
+    a.z_out = L.zero ? out.z_bf16 : nullptr;
+    a.s_groups = L.group_size ? static_cast<int32_t>(L.k / L.group_size) : 1;
+  }
+  if (out.at) {
+    a.A = A;
+    a.at_out = out.at;
+    a.r = L.r;
+  }
   a.status = dev->status;
   a.timeout_ns = kWaitTimeoutNs;
   LRQAT_LAUNCH("lowrank_codes", 1, stream,
@@ -733,7 +770,14 @@ static int linear_fwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
       LRQAT_LAUNCH("adapter_layouts", 1, stream,
                    launch_adapter_layouts(A, B, L.m, L.k, L.r, r16, nullptr, nullptr, ws.at, ws.b_pad, stream),
                    "adapter layouts");
-    LRQAT_TRY(run_codes_pass(L, Phi0, A, B, ws.at, ws.b_pad, ws.codes, true, dev, stream));
+    CodesOut out{};
+    out.row_major = ws.codes;
+    if (pair && L.group_size) {
+      out.s = s;
+      out.s_bf16 = ws.s_bf16;
+      out.z_bf16 = ws.z_bf16;
+    }
+    LRQAT_TRY(run_codes_pass(L, Phi0, A, B, ws.at, ws.b_pad, out, dev, stream));
   } else if (!direct) {
     LRQAT_LAUNCH("adapter_layouts", 1, stream,
                  launch_adapter_layouts(A, B, L.m, L.k, L.r, r16, ws.a_pad, ws.bt_pad, nullptr, nullptr, stream),
@@ -804,9 +848,11 @@ static int linear_fwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
   const int ffmt = cb ? LRQAT_PHI_QFIXED : L.phi_format;
   if (pair && L.group_size) {
     // the pair kernel's producers read the group scales as bf16 rows [groups][m], staged per stage
+    // (on the codes path the codes pass wrote them)
     const int groups = static_cast<int>(L.k / L.group_size);
-    LRQAT_LAUNCH("scale_rows", 1, stream,
-                 launch_dx_scales(s, L.zero, L.m, groups, groups, ws.s_bf16, ws.z_bf16, stream), "scale rows");
+    if (!cb)
+      LRQAT_LAUNCH("scale_rows", 1, stream,
+                   launch_dx_scales(s, L.zero, L.m, groups, groups, ws.s_bf16, ws.z_bf16, stream), "scale rows");
     a.s_bf16 = ws.s_bf16;
     a.z_bf16 = ws.z_bf16;
   }
@@ -840,11 +886,9 @@ size_t lrqat_bwd_workspace_bytes(const lrqat_layer* layer, int64_t T) {
   DeviceInfo* dev = nullptr;
   int sms = 152;
   if (device_info(&dev) == LRQAT_OK) sms = dev->sms;
-  const bool pair = use_pair_dw(*layer);
-  int pairs = sms / 2;
-  if (pair && dev) pairs = dw_pair_max_pairs();
-  if (pair && pairs < 1) return 0;
-  return bwd_ws_layout(*layer, T, plan_dw(*layer, T, pair ? pairs : sms, pair), nullptr, nullptr);
+  const int pairs = dev ? dw_pair_max_pairs() : sms / 2;
+  if (pairs < 1 && use_pair_dw(*layer)) return 0;
+  return bwd_ws_layout(*layer, T, plan_layer_dw(*layer, T, sms, pairs), nullptr, nullptr);
 }
 
 // quantized: X is already the activation quantizer's output (as for linear_fwd_impl) and
@@ -881,10 +925,9 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
     return fail(LRQAT_ERR_INVALID_ARG, "s_x is required when act_bits == 8 (per-tensor scale)");
   DeviceInfo* dev = nullptr;
   LRQAT_TRY(device_info(&dev));
-  const bool dw_pair = use_pair_dw(L);
-  const int dw_pairs = dw_pair ? dw_pair_max_pairs() : 0;
-  if (dw_pair && dw_pairs < 1) return fail(LRQAT_ERR_CUDA, "no cluster of two fits the dW kernel");
-  const DwPlan plan = plan_dw(L, T, dw_pair ? dw_pairs : dev->sms, dw_pair);
+  const int dw_pairs = dw_pair_max_pairs();
+  if (dw_pairs < 1 && use_pair_dw(L)) return fail(LRQAT_ERR_CUDA, "no cluster of two fits the dW kernel");
+  const DwPlan plan = plan_layer_dw(L, T, dev->sms, dw_pairs);
   const size_t need = bwd_ws_layout(L, T, plan, nullptr, nullptr);
   if (!workspace || workspace_bytes < need)
     return fail(LRQAT_ERR_WORKSPACE, "backward workspace of %zu bytes required, %zu given", need,
@@ -896,31 +939,31 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
   const int r16 = round16(L.r);
   // the transposed base of a packed layer holds one int8 code per byte
   const int fmt_t = L.phi_format == LRQAT_PHI_INT_PACKED ? LRQAT_PHI_QFIXED : L.phi_format;
-  // with direct factors the dX GEMM reads its A slices from A itself; its row factor stays the
-  // padded B^T, and dW takes A^T and B padded
-  // cb: the dX GEMM reads the codes (lrqat_set_lowrank_path); cbw: so does dW (ranks above 64)
+  // cb: the dX GEMM reads the codes (lrqat_set_lowrank_path); cbw: so does dW, with the clip mask in
+  // the byte's top bit (needs codes of 7 bits; the pair kernel, and every rank above 64)
   const bool cb = codes_gemm(L, T);
-  const bool cbw = codes_dw(L);
-  const bool direct = !cb && direct_factors(L, A, B);
-  if (cb && direct_factors(L, A, B)) {
-    // the codes of every weight from A and B themselves, then one launch for A^T and B padded
-    // (dW's operands) and the transposed codes (the dX GEMM's base)
-    LRQAT_TRY(run_codes_pass(L, Phi0, A, B, ws.at, ws.b_pad, ws.codes, !cbw, dev, stream));
-    LRQAT_LAUNCH("bwd_prep", 1, stream,
-                 launch_bwd_prep(A, B, L.m, L.k, L.r, r16, nullptr, nullptr, ws.at, ws.b_pad, ws.codes,
-                                 LRQAT_PHI_QFIXED, ws.phit, stream, cbw ? L.bits : 0),
-                 "adapter layouts and transposed codes");
-  } else if (cb) {
-    // the codes of every weight, then their transpose for the dX GEMM; A^T and B padded serve
-    // the code pass and dW
-    LRQAT_LAUNCH("adapter_layouts", 1, stream,
-                 launch_adapter_layouts(A, B, L.m, L.k, L.r, r16, nullptr, nullptr, ws.at, ws.b_pad, stream),
-                 "adapter layouts");
-    LRQAT_TRY(run_codes_pass(L, Phi0, A, B, ws.at, ws.b_pad, ws.codes, !cbw, dev, stream));
-    LRQAT_LAUNCH("bwd_prep", 1, stream,
-                 launch_bwd_prep(A, B, L.m, L.k, L.r, r16, nullptr, nullptr, nullptr, nullptr, ws.codes,
-                                 LRQAT_PHI_QFIXED, ws.phit, stream, cbw ? L.bits : 0),
-                 "transposed codes");
+  const bool cbw = L.r > 64 || (cb && plan.pair && L.bits <= 7);
+  const bool direct_ab = direct_factors(L, A, B);
+  // with direct factors the dX GEMM reads its A slices from A itself (its row factor stays the
+  // padded B^T), and dW its B slices from B
+  const bool direct = !cb && direct_ab;
+  const uint16_t* b_rows = cb && direct_ab ? B : ws.b_pad;
+  if (cb) {
+    // one pass: the transposed codes (the dX GEMM's base), dW's code bytes, the scale rows of dX and,
+    // from direct factors, A^T
+    if (!direct_ab)
+      LRQAT_LAUNCH("adapter_layouts", 1, stream,
+                   launch_adapter_layouts(A, B, L.m, L.k, L.r, r16, nullptr, nullptr, ws.at, ws.b_pad, stream),
+                   "adapter layouts");
+    CodesOut out{};
+    out.row_major = cbw ? ws.codes : nullptr;
+    out.mask = cbw;
+    out.transposed = ws.phit;
+    out.s = s;
+    out.s_bf16 = ws.s_bf16;
+    out.z_bf16 = ws.z_bf16;
+    out.at = direct_ab ? ws.at : nullptr;
+    LRQAT_TRY(run_codes_pass(L, Phi0, A, B, ws.at, ws.b_pad, out, dev, stream));
   } else {
     LRQAT_LAUNCH("bwd_prep", 1, stream,
                  launch_bwd_prep(A, B, L.m, L.k, L.r, r16, direct ? nullptr : ws.a_pad, ws.bt_pad, ws.at, ws.b_pad,
@@ -944,14 +987,15 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
   }
   // the codes base has no fraction bits
   const QuantParams q = make_quant_params(L.bits, cb ? 0 : frac_bits(L), L.alpha, L.r);
-  const QuantParams qw = make_quant_params(L.bits, cbw ? 0 : frac_bits(L), L.alpha, L.r);
+  const QuantParams qw = make_quant_params(L.bits, frac_bits(L), L.alpha, L.r);
 
   // dX = dY W_hat (W_hat^T produced on chip from Phi0^T, B^T and A).
   {
     const int groups = L.group_size ? static_cast<int>(L.k / L.group_size) : 1;
-    LRQAT_LAUNCH("dx_scales", 1, stream,
-                 launch_dx_scales(s, L.zero, L.m, groups, L.group_size ? groups : 0, ws.s_bf16, ws.z_bf16, stream),
-                 "dX scale rows");
+    if (!cb)
+      LRQAT_LAUNCH("dx_scales", 1, stream,
+                   launch_dx_scales(s, L.zero, L.m, groups, L.group_size ? groups : 0, ws.s_bf16, ws.z_bf16, stream),
+                   "dX scale rows");
     const bool pair = use_pair(L.k);
     CUtensorMap tm_tok, tm_phi, tm_rf, tm_sf;
     LRQAT_TRY(encode_2d(&tm_tok, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, dY, L.m, T, L.m * 2, 64, pair ? 112 : 224,
@@ -989,7 +1033,7 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
     a.zero = L.zero;
     a.u_bf16 = cb ? 0 : L.u_bf16;
     a.sf_mn = 0;
-    a.codes_bias = cb ? static_cast<int32_t>(codes_bias(L)) : 0;   // ranks above 64: clipped and biased in the transpose
+    a.codes_bias = cb ? static_cast<int32_t>(codes_bias(L)) : 0;
     a.s_bf16 = ws.s_bf16;
     a.z_bf16 = ws.z_bf16;
     a.s_ld = L.group_size ? static_cast<int32_t>(L.k / L.group_size) : 0;
@@ -1021,8 +1065,8 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
                         static_cast<uint32_t>(plan.bkt), CU_TENSOR_MAP_SWIZZLE_128B, "dY (dW)"));
     LRQAT_TRY(encode_2d(&tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, xop, L.k, T, L.k * 2, 64,
                         static_cast<uint32_t>(plan.bkt), CU_TENSOR_MAP_SWIZZLE_128B, "X (dW)"));
-    // the codes base: boxes of 64 rank rows (one round of the adapter contractions)
-    const uint32_t rbox_rows = cbw ? 64u : static_cast<uint32_t>(r16);
+    // ranks above 64: boxes of 64 rank rows (one round of the adapter contractions)
+    const uint32_t rbox_rows = r16 > 64 ? 64u : static_cast<uint32_t>(r16);
     LRQAT_TRY(encode_2d(&tm_at, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ws.at, L.m, r16, L.m * 2, 64, rbox_rows,
                         CU_TENSOR_MAP_SWIZZLE_128B, "A^T"));
     if (cbw)
@@ -1030,8 +1074,10 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
                           CU_TENSOR_MAP_SWIZZLE_128B, "codes"));
     else
       LRQAT_TRY(phi_map(&tm_phi, L, Phi0, 128, true));
-    LRQAT_TRY(encode_2d(&tm_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ws.b_pad, L.k, r16, L.k * 2, 64, rbox_rows,
-                        CU_TENSOR_MAP_SWIZZLE_128B, "B (padded)"));
+    // B's rows past r (direct factors) read as zeros, as the padded copy's do
+    const int64_t b_ranks = b_rows == B ? L.r : r16;
+    LRQAT_TRY(encode_2d(&tm_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, b_rows, L.k, b_ranks, L.k * 2, 64, rbox_rows,
+                        CU_TENSOR_MAP_SWIZZLE_128B, "B (dW)"));
     DwArgs a{};
     a.m = static_cast<int32_t>(L.m);
     a.k = static_cast<int32_t>(L.k);
@@ -1061,12 +1107,19 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
     a.tile_segs = ws.tile_segs;
     a.codes_base = cbw ? 1 : 0;
     const int grid = plan.sched.grid;
-    if (plan.pair) {
+    if (plan.pair && cbw) {
+      // each CTA of a pair loads half of a round's ranks of B
+      CUtensorMap tm_bh;
+      LRQAT_TRY(encode_2d(&tm_bh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, b_rows, L.k, b_ranks, L.k * 2, 64, rbox_rows / 2,
+                          CU_TENSOR_MAP_SWIZZLE_128B, "B (rank halves)"));
+      LRQAT_LAUNCH("fused_dw", 1, stream, launch_dw_codes(tm_dy, tm_x, tm_at, tm_bh, a, grid, stream),
+                   "fused dW launch (CTA pairs on the codes)");
+    } else if (plan.pair) {
       // each CTA of a pair loads half of the ranks of the slices that serve as N-split B operands
       CUtensorMap tm_ath, tm_bh;
       LRQAT_TRY(encode_2d(&tm_ath, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ws.at, L.m, r16, L.m * 2, 64,
                           static_cast<uint32_t>(r16 / 2), CU_TENSOR_MAP_SWIZZLE_128B, "A^T (rank halves)"));
-      LRQAT_TRY(encode_2d(&tm_bh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ws.b_pad, L.k, r16, L.k * 2, 64,
+      LRQAT_TRY(encode_2d(&tm_bh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, b_rows, L.k, b_ranks, L.k * 2, 64,
                           static_cast<uint32_t>(r16 / 2), CU_TENSOR_MAP_SWIZZLE_128B, "B (rank halves)"));
       LRQAT_LAUNCH("fused_dw", 1, stream,
                    launch_dw_pair(L.phi_format, tm_dy, tm_x, tm_at, tm_ath, tm_phi, tm_b, tm_bh, a, grid, stream),
@@ -1134,8 +1187,8 @@ int lrqat_merge(const lrqat_layer* layer, const void* Phi0, const uint16_t* A, c
     LRQAT_TRY(device_info(&dev));
     const int r16 = round16(L.r);
     CUtensorMap tm_a, tm_b;
-    LRQAT_TRY(encode_2d(&tm_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, A, L.r, L.m, L.r * 2, 64, 128,
-                        CU_TENSOR_MAP_SWIZZLE_128B, "A"));
+    LRQAT_TRY(encode_2d(&tm_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, A, L.r, L.m, L.r * 2, a_cols(r16), 128,
+                        sf_swizzle(r16), "A"));
     LRQAT_TRY(encode_2d(&tm_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, B, L.k, L.r, L.k * 2, 64,
                         static_cast<uint32_t>(r16), CU_TENSOR_MAP_SWIZZLE_128B, "B"));
     CUtensorMap tm_phi;
@@ -1146,6 +1199,7 @@ int lrqat_merge(const lrqat_layer* layer, const void* Phi0, const uint16_t* A, c
     a.k = L.k;
     a.r16 = r16;
     a.q = q;
+    a.bits = L.bits;
     a.status = dev->status;
     a.timeout_ns = kWaitTimeoutNs;
     LRQAT_LAUNCH("merge", 1, stream, launch_merge_tc(L.phi_format, L.u_bf16, 0, tm_a, tm_b, tm_phi, a, stream),

@@ -193,15 +193,6 @@ __device__ __forceinline__ uint32_t pack_int_bf16x2(float c0, float c1) {
   return __byte_perm(__float_as_uint(c0), __float_as_uint(c1), 0x7632u);
 }
 
-// The same for two stored integer codes (the codes base: already rounded, 0 fraction bits):
-// their floats are exact, so their top halves are their bf16 values.
-__device__ __forceinline__ uint32_t int_codes_bf16x2(float c0, float c1, const QuantParams& q) {
-  uint32_t w = __byte_perm(__float_as_uint(c0), __float_as_uint(c1), 0x7632u);
-  asm("max.bf16x2 %0, %0, %1;" : "+r"(w) : "r"(q.n_bf16x2));
-  asm("min.bf16x2 %0, %0, %1;" : "+r"(w) : "r"(q.p_bf16x2));
-  return w;
-}
-
 // t = round-half-even(u_f / 2^f) in the magic domain, unclipped.
 __device__ __forceinline__ float magic_round(float L, float v, const QuantParams& q) {
   const float u = __fmaf_rn(L, q.lr_scale, v);
@@ -275,6 +266,26 @@ __device__ __forceinline__ uint32_t sub_bf16x2(uint32_t a, uint32_t b) {
 __device__ __forceinline__ void decode_b64_bf16x4(uint32_t w, uint32_t& w01, uint32_t& w23) {
   w01 = sub_bf16x2(__byte_perm(w, 0x43u, 0x4140u), 0x43404340u);
   w23 = sub_bf16x2(__byte_perm(w, 0x43u, 0x4342u), 0x43404340u);
+}
+
+// Code bytes of the weight-gradient kernels (c + 64, bit 7 the clip mask M): four of them -> the
+// codes as floats, and the masks of codes 0, 1 (HI = 0) or 2, 3 (HI = 1) as all-ones or zero
+// halves of a word.
+__device__ __forceinline__ void decode_codes4(uint32_t w, float2& c01, float2& c23) {
+  const uint32_t x = w & 0x7f7f7f7fu;
+  constexpr float off = 8388608.0f + 64.0f;   // 2^23 + 64
+  c01 = __fadd2_rn(make_float2(__uint_as_float(__byte_perm(x, 0x4B000000u, 0x7540u)),
+                               __uint_as_float(__byte_perm(x, 0x4B000000u, 0x7541u))),
+                   make_float2(-off, -off));
+  c23 = __fadd2_rn(make_float2(__uint_as_float(__byte_perm(x, 0x4B000000u, 0x7542u)),
+                               __uint_as_float(__byte_perm(x, 0x4B000000u, 0x7543u))),
+                   make_float2(-off, -off));
+}
+template <int HI>
+__device__ __forceinline__ uint32_t code_masks2(uint32_t w) {
+  uint32_t r;   // selector values 8 .. 11 replicate the sign bit of bytes 0 .. 3
+  asm("prmt.b32 %0, %1, %1, %2;" : "=r"(r) : "r"(w), "n"(HI ? 0xBBAA : 0x9988));
+  return r;
 }
 
 // Elementwise bf16x2 product, rounded to nearest even.

@@ -1,0 +1,73 @@
+"""The weight gradients from the code bytes of the codes pass (clip mask in the top bit) against the
+kernels that recompute the low-rank tile: the same G, code and mask per weight, so dA, dB and ds
+agree bit for bit, over both work schedules, ragged token counts, ranks of one to four K steps,
+clipping grids, groups, zero offsets and several tiles per persistent CTA."""
+import pytest
+
+from paper_2406_06385_gb300 import lrqat as LQ
+from paper_2406_06385_gb300 import workloads as WL
+
+from gpu_util import DeviceLayer, to_dev, torch
+
+pytestmark = pytest.mark.gpu
+
+
+def _spec(m, k, r, bits=4, group=0, phi=WL.PHI_QFIXED, act=0, asym=False, ub=False, std=0.2):
+    return WL.LayerSpec("c", m, k, r, float(r), bits, group, phi, act, a_std=std, b_std=std, asym=asym,
+                        w_row_shift=0.03 if asym else 0.0, u_bf16=ub)
+
+
+CASES = [
+    ("one_tile_one_token", _spec(256, 256, 8), 1),
+    ("rank_not_direct", _spec(256, 512, 20), 97),
+    ("rank_48_clip", _spec(512, 256, 48, bits=2, std=1.0), 450),
+    ("rank_64_group", _spec(256, 768, 64, group=128), 1000),
+    ("int3_packed_a8", _spec(512, 512, 32, bits=3, phi=WL.PHI_INT_PACKED, act=8), 333),
+    ("asym_group", _spec(256, 512, 16, bits=2, group=256, asym=True), 2070),
+    ("bf16_base_ubf16", _spec(256, 512, 32, phi=WL.PHI_BF16, ub=True), 130),
+    ("bits_7", _spec(256, 256, 32, bits=7), 64),
+    ("many_tiles", _spec(2560, 2304, 32), 700),
+]
+
+
+def _grads(spec, T, dl, X, dY, s_x):
+    t = torch()
+    out = [t.empty((T, spec.k), dtype=t.int16, device="cuda"), t.empty((spec.m, spec.r), device="cuda"),
+           t.empty((spec.r, spec.k), device="cuda"), t.empty_like(dl.s)]
+    ws = t.empty(LQ.bwd_workspace_bytes(dl.layer, T), dtype=t.uint8, device="cuda")
+    LQ.linear_bwd(dl.layer, T, dY, X, dl.phi0, dl.s, dl.A, dl.B, s_x, *out, False, ws)
+    LQ.get_device_status()
+    return out
+
+
+@pytest.mark.parametrize("schedule", ["split", "tail"])
+@pytest.mark.parametrize("cid,spec,T", CASES, ids=[c[0] for c in CASES])
+def test_gradients_from_codes_equal_those_from_the_low_rank_tile(cid, spec, T, schedule, lowrank_path, dw_schedule):
+    t = torch()
+    dw_schedule(schedule)
+    data = WL.make_layer(spec, T, seed=4)
+    dl = DeviceLayer(data, 1.05)
+    X, dY = to_dev(data.X_bits), to_dev(data.dY_bits)
+    s_x = t.full((1,), 0.02, device="cuda") if spec.act_bits else None
+    got = {}
+    for path in ("tile", "codes"):
+        lowrank_path(path)
+        got[path] = _grads(spec, T, dl, X, dY, s_x)
+    for name, a, b in zip(("dA", "dB", "ds"), got["tile"][1:], got["codes"][1:]):
+        assert t.equal(a, b), name
+    a, b = (got[p][0].view(t.bfloat16).float() for p in ("tile", "codes"))
+    assert float((a - b).norm() / b.norm()) <= 4e-3
+
+
+def test_codes_of_unaligned_factors_and_outputs():
+    """The merge writes the same codes from padded factors, and to a 16-byte aligned output that is
+    not 32-byte aligned."""
+    t = torch()
+    spec = _spec(384, 640, 32, bits=3)
+    dl = DeviceLayer(WL.make_layer(spec, 1, seed=2, with_activations=False))
+    out = [t.empty(spec.m * spec.k + 16, dtype=t.int8, device="cuda")[o:o + spec.m * spec.k] for o in (0, 16)]
+    for o in out:
+        LQ.merge(dl.layer, dl.phi0, dl.A, dl.B, o)
+    LQ.get_device_status()
+    assert t.equal(out[0], out[1])
+    assert int(out[0].min()) == -4 and int(out[0].max()) == 3
