@@ -28,15 +28,14 @@
  *     64 with bits <= 7), T >= 1 (any T; ragged token tails are handled),
  *     group_size 0 (per output channel) or a multiple of 128 that divides k.
  *   - W_hat is rebuilt on chip inside the GEMMs and never written.  Where the
- *     low-rank term comes from is a tuning choice (lrqat_set_lowrank_path): for
- *     ranks up to 64 and fewer than 3072 tokens each GEMM stage computes the
- *     low-rank tile (alpha/r) A B next to the main product; otherwise one
+ *     low-rank term comes from is a tuning choice (lrqat_set_lowrank_path): one
  *     tensor-core pass per call first writes one byte per weight into the
  *     workspace, the clipped code c = clip(round(u), n, p) biased by 64 (128 for
  *     8-bit weights), which for the weight-gradient kernel carries the clip mask in
- *     its top bit (weights of up to 7 bits); the
- *     GEMMs then turn those bytes into W_hat on chip.  The results are the same
- *     codes, gradients and outputs.
+ *     its top bit (weights of up to 7 bits), and the GEMMs turn those bytes into W_hat
+ *     on chip; or (ranks up to 64; the allocation-free forward) each GEMM stage
+ *     computes the low-rank tile (alpha/r) A B next to the main product.  The results
+ *     are the same codes, gradients and outputs.
  */
 #ifndef LRQAT_H
 #define LRQAT_H
@@ -317,9 +316,8 @@ int lrqat_set_dw_schedule(int schedule);
 
 /* Tuning (no counterpart in the paper): the kernels of the forward, dX and dW GEMMs.
  * CTA pairs run tcgen05 MMAs of 256 rows across the two SMs of a cluster, each SM holding
- * half of the token operand (256 weight rows x 448 tokens per pair); they need a multiple
- * of 256 produced rows (m for the forward, k for dX; dW: ranks up to 64 and m, k multiples
- * of 256, on 256 x 256 tiles).  The one-SM kernels take 128 rows per SM.  0 (the default) =
+ * half of the token operand (256 weight rows x up to 448 tokens per pair); dW on pairs needs m and
+ * k multiples of 256 (256 x 256 tiles).  The one-SM kernels take 128 rows per SM.  0 (the default) =
  * pairs wherever they were measured faster, which is wherever the shapes allow; 1 = the
  * one-SM kernels always; 2 = pairs wherever the shapes allow.  All give the same codes;
  * outputs agree up to fp32 summation order.  Process-wide; the environment variable LRQAT_GEMM_VARIANT ("auto",
@@ -333,9 +331,9 @@ int lrqat_set_gemm_variant(int variant);
  * to 64); 2 = "codes": one tensor-core pass per call writes the code of every weight as one
  * byte (clip(round(u), n, p) + 64, or + 128 for 8-bit weights) into the workspace and the
  * GEMMs read those bytes as their base, with no low-rank work in the stage; 0 (the default)
- * = codes from 3072 tokens
- * on, the tile below (the pass costs two bytes of HBM traffic per weight, the tile a low-rank
- * MMA chain per stage).  Ranks above 64 always take the codes pass.  dW reads the codes where
+ * = codes, except in the allocation-free forward, whose scratch does not hold them (the pass costs
+ * two bytes of HBM traffic per weight, the tile a low-rank MMA chain per stage).  Ranks above 64
+ * always take the codes pass.  dW reads the codes where
  * the pair kernels take it (m and k multiples of 256, up to 7 bits) and computes its own
  * low-rank tile elsewhere.  All settings give the same codes up to
  * fp32 summation order of A B.  Process-wide; the environment variable LRQAT_LOWRANK_PATH

@@ -8,13 +8,14 @@
 // half of every accumulator's tokens, and the tensor cores of the pair exchange the token halves
 // (measured on a 4096 x 4096 layer at T = 8192 on the codes: forward 276 -> 181 us).
 //
-// A pair processes tiles of 256 weight rows (CTA rank c: rows 128 c .. 128 c + 127) x 448
-// tokens (two accumulators of 224 tokens; CTA c holds tokens 112 c .. 112 c + 111 of each), one
+// A pair processes tiles of 256 weight rows (CTA rank c: rows 128 c .. 128 c + 127) x up to 448
+// tokens (an odd last 128-row block leaves the second CTA's half of its tiles empty; two accumulators of 224 tokens; CTA c holds tokens 112 c .. 112 c + 111 of each; the
+// host picks smaller token tiles where 448 leave pairs idle, pair_token_tile in lrqat_api.cu), one
 // 64-wide slice of the contraction per stage:
-//   * token ring (three slots per CTA, four on the codes): one loader warp per slot brings this
-//     CTA's two 112-token halves (SW128) with TMA whose completion lands on the leader's
+//   * token ring (three slots per CTA, four to eight on the codes): loader warps bring this
+//     CTA's token halves (SW128) with TMA whose completion lands on the leader's
 //     barrier; each slot also holds this CTA's W_hat tile of the stage;
-//   * factor ring (4 slots; 2 for 16-bit bases): the stored base of this CTA's rows (completion
+//   * factor ring (four slots, 2 for 16-bit bases, up to eight on the codes): the stored base of this CTA's rows (completion
 //     on its own barrier; only its own producers read it), with it the stage's scales (and zero
 //     offsets) where the producers apply them (dX, group-wise forward), and with the low-rank tile
 //     this CTA's half (32 rows) of the second factor's slice (completion on the leader's
@@ -32,8 +33,8 @@
 // memory whose completion counts on the leader's barrier (a thread-issued remote arrive is
 // several times slower under the pair's operand traffic), after fence.proxy.async has ordered
 // the peer's writes.
-// On the codes (NL: every rank from 3072 tokens on, and ranks above 64) the base holds the
-// one-byte codes of the codes pass; no factors, no L.
+// On the codes (NL: every call but the allocation-free forward of ranks up to 64, unless set
+// otherwise) the base holds the one-byte codes of the codes pass; no factors, no L.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cstdint>
@@ -47,40 +48,40 @@ namespace {
 
 constexpr int BM = 128;                          // weight rows per CTA (256 per pair)
 constexpr int BK = 64;
-constexpr int BNP = 224;                         // tokens per accumulator (N of the pair MMA)
+constexpr int BNP = 224;                         // most tokens per accumulator of two (N of the pair MMA)
 constexpr int BNH = BNP / 2;                     // tokens per accumulator held by one CTA
-constexpr int NACC = 2;
-constexpr int BTP = BNP * NACC;                  // 448 tokens per pair tile
-constexpr int NT_MAX = 4;                        // token ring slots (3 with the low-rank tile)
+constexpr int NACC = 2;                          // accumulators (one for tiles of up to 256 tokens)
+constexpr int NT_MAX = 8;                        // token ring slots
 constexpr int NLB = 1;                           // low-rank TMEM buffers
-constexpr int NF_MAX = 4;                        // factor ring slots (2 for 16-bit bases)
+constexpr int NF_MAX = 8;                        // factor ring slots
 constexpr int NUM_PROD_WARPS = 16;
 constexpr int FIRST_TMA_WARP = 2 + NUM_PROD_WARPS;
-constexpr int NUM_TMA_WARPS = NT_MAX + 1;        // a token loader per slot, the factor loader
+constexpr int NUM_TOK_LOADERS = 4;               // token loaders (every fourth stage each)
+constexpr int NUM_TMA_WARPS = NUM_TOK_LOADERS + 1;   // and the factor loader
 constexpr int NUM_THREADS = 32 * (FIRST_TMA_WARP + NUM_TMA_WARPS);
-constexpr int EPI_COLS = NACC * BNP / 4;         // accumulator columns drained per warp (112)
-constexpr uint32_t SIG_TX = 16u * NUM_PROD_WARPS;   // bytes of the peer's per-warp signals
+// On the codes the producer warps work in four groups, group g on the stages gg % 4 == g: a warp
+// turns 32 rows x 64 columns per stage (16 columns where all sixteen share every stage).
+constexpr int NUM_GROUPS = 4;
+constexpr int GROUP_WARPS = NUM_PROD_WARPS / NUM_GROUPS;
 
 constexpr uint32_t RF_BYTES = 128 * 128;         // 128 rows x 64 rank columns (bf16)
-constexpr uint32_t TOK_BOX = BNH * 128;          // 112 tokens x 64 bf16
-constexpr uint32_t TOK_BYTES = NACC * TOK_BOX;
 constexpr uint32_t W_BYTES = 128 * 128;          // 128 rows x 64 bf16
 constexpr uint32_t SFH_BYTES = 32 * 128;         // 32 slice rows x up to 64 rank columns (bf16)
-constexpr uint32_t TSLOT_BYTES = TOK_BYTES + W_BYTES;
-constexpr uint32_t TS_W = TOK_BYTES;
 
-// Shared-memory rings.  With the low-rank tile: the row factor, three token slots and per stage
-// the stored base and this CTA's half of the second factor's slice.  On the codes (NL): no
-// factors, so a fourth token slot fits (measured on a 4096 x 4096 layer at T = 8192: forward
-// 191 -> 181 us).
+// Shared-memory rings.  A token slot holds this CTA's half of the stage's tokens (a tile of btp
+// tokens: 64 btp bytes) and its W_hat tile, a factor slot the stored base.  With the low-rank tile:
+// the row factor, three token slots of 448 tokens, and this CTA's half of the second factor's slice
+// in each of four (16-bit bases: two) factor slots.  On the codes (NL): as many token slots as the
+// tile leaves room for beside at least four factor slots, and factor slots in the rest (up to eight
+// of each): a slot is refilled by TMA only after its stage's MMAs, so the shorter the stage, the
+// more stages it takes to cover a load's latency.
 // XS: each factor slot also holds the stage's scales (and zero offsets) as bf16, copied by the
 // factor loader, so that the producers read them from shared memory with the base instead of
 // from global memory: for dX the 64 scales of the stage's contraction indices in the CTA's row
 // group, for the group-wise forward the 128 scales of the CTA's rows in the stage's group.
+constexpr uint32_t RING_BYTES = 232448 - 1024 - 1024;   // less the static barriers and the alignment
 template <int FMT, bool NL, bool XS>
 struct PairRing {
-  static constexpr int NT = NL ? 4 : 3;
-  static constexpr int NF = fmt_16bit(FMT) ? 2 : 4;
   static constexpr uint32_t RF = NL ? 0u : RF_BYTES;
   static constexpr uint32_t PHI_BYTES = fmt_16bit(FMT) ? 128 * 128 : 128 * 64;
   static constexpr uint32_t PHI_TX = FMT == FMT_I4 ? PHI_BYTES / 2 : PHI_BYTES;
@@ -90,16 +91,24 @@ struct PairRing {
   static constexpr uint32_t FSLOT_BYTES = FS_X + (XS ? 1024u : 0u);
   static constexpr uint32_t OFF_RF = 0;
   static constexpr uint32_t OFF_TSLOTS = RF;
-  static constexpr uint32_t OFF_FSLOTS = OFF_TSLOTS + NT * TSLOT_BYTES;
-  static constexpr uint32_t SMEM_BYTES = OFF_FSLOTS + NF * FSLOT_BYTES + 1024;
-  static_assert(NT <= NT_MAX, "token slots");
-  static_assert(FSLOT_BYTES % 1024 == 0 && FS_SF % 1024 == 0 && OFF_FSLOTS % 1024 == 0,
-                "swizzled tiles must start on 1024-byte boundaries");
-  static_assert(SMEM_BYTES + 1024 <= 232448, "shared memory budget");
+  static_assert(FSLOT_BYTES % 1024 == 0 && FS_SF % 1024 == 0, "swizzled tiles must start on 1024-byte boundaries");
+  __host__ __device__ static constexpr uint32_t tslot(int btp) { return 64u * btp + W_BYTES; }
+  __host__ __device__ static constexpr int nt(int btp) {
+    if (!NL) return 3;
+    const int n = static_cast<int>((RING_BYTES - 4u * FSLOT_BYTES) / tslot(btp));
+    return n < NT_MAX ? n : NT_MAX;
+  }
+  // on the codes four or eight, multiples of NUM_GROUPS: a group then knows that the previous use of
+  // a slot it waits for has landed (it was its own), so barrier phases cannot alias
+  __host__ __device__ static constexpr int nf(int btp) {
+    if (!NL) return fmt_16bit(FMT) ? 2 : 4;
+    return (RING_BYTES - nt(btp) * tslot(btp)) / FSLOT_BYTES >= 8 ? 8 : 4;
+  }
+  __host__ __device__ static constexpr uint32_t smem(int btp) {
+    return RF + nt(btp) * tslot(btp) + nf(btp) * FSLOT_BYTES + 1024u;
+  }
+  static_assert(nt(448) >= (NL ? NUM_GROUPS : 3) && smem(448) + 1024 <= 232448 && smem(32) + 1024 <= 232448, "shared memory budget");
 };
-static_assert(TSLOT_BYTES % 1024 == 0 && TOK_BOX % 1024 == 0 && TS_W % 1024 == 0,
-              "swizzled tiles must start on 1024-byte boundaries");
-static_assert(EPI_COLS % 16 == 0, "epilogue drains 16-column chunks");
 
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t COL_L = NACC * BNP;           // the 64-column low-rank buffer(s) after the accumulators
@@ -120,7 +129,8 @@ constexpr int BAR_RFEMPTY = BAR_RFFULL + 1;      // both: last low-rank MMA of t
 constexpr int BAR_ACCFULL = BAR_RFEMPTY + 1;     // both: accumulators of the tile complete
 constexpr int BAR_ACCEMPTY = BAR_ACCFULL + 1;    // leader: both CTAs drained them
 constexpr int BAR_DRAIN = BAR_ACCEMPTY + 1;
-constexpr int NUM_BARS = BAR_DRAIN + 1;
+constexpr int BAR_DRAIN_B = BAR_DRAIN + 1;       // the second issuer's
+constexpr int NUM_BARS = BAR_DRAIN_B + 1;
 
 __device__ __forceinline__ void drain_wait(uint32_t bar, uint32_t parity, uint64_t timeout_ns) {
   const uint64_t t0 = global_timer_ns();
@@ -130,18 +140,30 @@ __device__ __forceinline__ void drain_wait(uint32_t bar, uint32_t parity, uint64
 }
 
 // Stages are numbered globally over the pair's tiles (gg), identically in both CTAs: token
-// slot gg % NT, factor slot gg % NF, low-rank buffer gg % 2.
+// slot gg % NT, factor slot gg % NF, low-rank buffer gg % NLB.  A cursor follows a ring's slot and
+// the parity of its use.
+struct Cursor {
+  uint32_t s = 0, ph = 0;
+  __device__ __forceinline__ void next(uint32_t n) {
+    if (++s == n) {
+      s = 0;
+      ph ^= 1u;
+    }
+  }
+  __device__ __forceinline__ void skip(uint32_t k, uint32_t n) {
+    for (s += k; s >= n; s -= n) ph ^= 1u;
+  }
+};
 template <int MODE, int FMT, bool ZP, bool UB, bool NL>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     fused_pair_kernel(const __grid_constant__ CUtensorMap tm_tok, const __grid_constant__ CUtensorMap tm_phi,
                       const __grid_constant__ CUtensorMap tm_rf, const __grid_constant__ CUtensorMap tm_sf,
                       const FusedArgs args) {
   using PR = PairRing<FMT, NL, MODE == FUSED_DX || MODE == FUSED_FWD_GROUP>;
-  constexpr int NT = PR::NT;
-  constexpr int NF = PR::NF;
-  constexpr uint32_t OFF_RF = PR::OFF_RF, OFF_TSLOTS = PR::OFF_TSLOTS, OFF_FSLOTS = PR::OFF_FSLOTS;
+  constexpr uint32_t OFF_RF = PR::OFF_RF, OFF_TSLOTS = PR::OFF_TSLOTS;
   constexpr bool PACKED = FMT == FMT_I4;
   constexpr uint32_t FSLOT_BYTES = PR::FSLOT_BYTES;
+  constexpr int STAGE_WARPS = NL ? GROUP_WARPS : NUM_PROD_WARPS;   // producer warps of one stage (per CTA)
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bars[NUM_BARS];
   __shared__ __align__(16) uint32_t sig_buf[8];   // [0, 4): source of the peer's signals, [4, 8): their target
@@ -157,18 +179,24 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   auto bar = [&](int i) { return smem_u32(&bars[i]); };
   auto lbar = [&](int i) { return map_shared_rank(smem_u32(&bars[i]), 0); };   // the leader's copy
 
+  // the token tile: one accumulator of bnp <= 256 tokens or two of bnp <= 224, half of each per CTA
+  const int bnp = args.bnp, bnh = bnp / 2, nacc = args.nacc, btp = bnp * nacc;
+  const int NT = PR::nt(btp), NF = PR::nf(btp);
+  const uint32_t TSLOT_BYTES = PR::tslot(btp), TOK_BOX = 128u * bnh, TS_W = 64u * btp;
+  const uint32_t OFF_FSLOTS = OFF_TSLOTS + NT * TSLOT_BYTES;
+  const uint32_t issuers = NL ? nacc : 1;   // threads that issue (and commit) the main product
   if (threadIdx.x == 0) {
     abort_s = 0;
     for (int s = 0; s < NT; ++s) {
-      mbar_init(bar(BAR_TFULL + s), 1 + NUM_PROD_WARPS);   // the leader's token loader and producer warps
-      mbar_init(bar(BAR_TEMPTY + s), 1);
+      mbar_init(bar(BAR_TFULL + s), 1 + STAGE_WARPS);   // the leader's token loader and producer warps
+      mbar_init(bar(BAR_TEMPTY + s), issuers);
     }
     for (int s = 0; s < NF; ++s) {
       mbar_init(bar(BAR_PFULL + s), 1);
       mbar_init(bar(BAR_FFULL + s), 1);
       // freed by this CTA's producers after they built W_hat: by then they have waited for the
       // low-rank tile, so the low-rank MMA that read the slot's factor half has completed
-      mbar_init(bar(BAR_FEMPTY + s), NUM_PROD_WARPS);
+      mbar_init(bar(BAR_FEMPTY + s), STAGE_WARPS);
     }
     for (int b = 0; b < NLB; ++b) {
       mbar_init(bar(BAR_LFULL + b), 1);
@@ -176,9 +204,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     }
     mbar_init(bar(BAR_RFFULL), 1);
     mbar_init(bar(BAR_RFEMPTY), 1);
-    mbar_init(bar(BAR_ACCFULL), 1);
+    mbar_init(bar(BAR_ACCFULL), issuers);
     mbar_init(bar(BAR_ACCEMPTY), NUM_PROD_WARPS);
     mbar_init(bar(BAR_DRAIN), 1);
+    mbar_init(bar(BAR_DRAIN_B), 1);
     mbar_fence_init();
   }
   if (warp == 1) tmem_alloc_pair(smem_u32(&tmem_base_s), TMEM_COLS);
@@ -189,26 +218,86 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   const uint32_t tmem = tmem_base_s;
   const WaitCtl ctl{&abort_s, args.status, args.timeout_ns};
   const int nk = args.kdim / BK;   // at least 2 (kdim is a multiple of 128)
-  const int num_rb2 = args.num_rb / 2;   // 256-row blocks
-  const int num_tiles = num_rb2 * ((args.T + BTP - 1) / BTP);
+  const int num_rb2 = (args.num_rb + 1) / 2;   // 256-row blocks
+  // This CTA's first row in row block rb2.  With an odd number of 128-row blocks the last pair's
+  // CTA 1 has none: it takes part with zero-filled loads (and the last block's scales) and stores
+  // nothing.
+  auto row_block = [&](int rb2) {
+    const int r0 = rb2 * 2 * BM + static_cast<int>(rank) * BM;
+    return r0 < args.rows ? r0 : args.rows - BM;
+  };
+  const int num_tiles = num_rb2 * ((args.T + btp - 1) / btp);
   const uint32_t sig_src = smem_u32(&sig_buf[0]);
   const uint32_t sig_dst_leader = map_shared_rank(smem_u32(&sig_buf[4]), 0);
   // A producer warp's event on a leader barrier: the leader's warps arrive (warp 0 also
-  // announces the peer's 16 signal bytes per warp), the peer's warps send their signal.
-  auto report = [&](int b, int pw) {
+  // announces the peer's 16 signal bytes of each of the n warps), the peer's warps send their signal.
+  auto report = [&](int b, int pw, int n) {
     if (leader) {
-      if (pw == 0) mbar_arrive_expect_tx(bar(b), SIG_TX);
+      if (pw == 0) mbar_arrive_expect_tx(bar(b), 16u * n);
       else mbar_arrive(bar(b));
     } else {
       signal_remote16(sig_dst_leader, sig_src, lbar(b));
     }
   };
 
+  // The main product of the pair's tiles into accumulator 0 (and / or 1), by one thread of the leader.
+  // On the codes two threads issue one accumulator each: a thread's barrier test and commit (~110
+  // and ~70 cycles a stage, with the tensor pipe queueing about one MMA ahead) then run beside the
+  // other's MMAs (4096 x 4096, 288-token tiles 906 -> 739 cycles a stage, 320 925 -> 801; at 448 the
+  // operands' shared-memory traffic sets the pace either way, 1101 -> 1106).
+  auto issue_main = [&](bool acc0, bool acc1, int drain) {
+    const uint32_t idesc_main = make_idesc_bf16(256, bnp, 0, 0);
+    const uint32_t TSLOT_D = TSLOT_BYTES >> 4, TOKB_D = TOK_BOX >> 4;
+    const uint64_t d_w0 = make_sdesc(smem + OFF_TSLOTS + TS_W, 16, 1024, SWZ_128B);
+    const uint64_t d_tok0 = make_sdesc(smem + OFF_TSLOTS, 16, 1024, SWZ_128B);
+    uint32_t it = 0;
+    Cursor cur;
+    bool ok = true;
+    for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
+      if (!(ok = wait_spin_bounded(bar(BAR_ACCEMPTY), (it & 1u) ^ 1u, ctl, 7))) break;
+      tc_fence_after();
+      // unrolled: the loop's own overhead between two stages' MMAs was ~120 cycles of idle tensor pipe
+#pragma unroll 4
+      for (int kk = 0; kk < nk; ++kk) {
+        const uint32_t s = cur.s;
+        if (!(ok = wait_spin_bounded(bar(BAR_TFULL + s), cur.ph, ctl, 9))) break;
+        cur.next(NT);
+        tc_fence_after();
+        const uint64_t w = d_w0 + s * TSLOT_D, t = d_tok0 + s * TSLOT_D;
+        const uint32_t acc = kk > 0 ? 1u : 0u;
+        static_assert(NACC == 2 && BK == 64, "issue sequence below: up to 2 accumulators x 4 K steps");
+        if (acc0) {
+          mma_bf16_pair(tmem, w, t, idesc_main, acc);
+          mma_bf16_pair(tmem, w + 2, t + 2, idesc_main, 1u);
+          mma_bf16_pair(tmem, w + 4, t + 4, idesc_main, 1u);
+          mma_bf16_pair(tmem, w + 6, t + 6, idesc_main, 1u);
+        }
+        if (acc1) {
+          mma_bf16_pair(tmem + BNP, w, t + TOKB_D, idesc_main, acc);
+          mma_bf16_pair(tmem + BNP, w + 2, t + TOKB_D + 2, idesc_main, 1u);
+          mma_bf16_pair(tmem + BNP, w + 4, t + TOKB_D + 4, idesc_main, 1u);
+          mma_bf16_pair(tmem + BNP, w + 6, t + TOKB_D + 6, idesc_main, 1u);
+        }
+        mma_commit_pair(bar(BAR_TEMPTY + s));
+      }
+      if (!ok) break;
+      mma_commit_pair(bar(BAR_ACCFULL));
+      ++it;
+    }
+    // the peer's last drain report lands before the CTAs end
+    if (ok) ok = wait_spin_bounded(bar(BAR_ACCEMPTY), (it & 1u) ^ 1u, ctl, 10);
+    mma_commit_pair_self(bar(drain));
+    drain_wait(bar(drain), 0, args.timeout_ns);
+  };
+
   if (warp == 0) {
     // ------------------- row factor (per tile) and, in the leader, the low-rank MMAs
     // A thread of its own issues the low-rank tiles, so that the main product never waits
-    // behind their barriers; each thread's commits track only its own MMAs.
-    if (!NL && lane == 0) {
+    // behind their barriers; each thread's commits track only its own MMAs.  On the codes it is the
+    // second accumulator's issuer.
+    if (NL) {
+      if (leader && lane == 0 && nacc == 2) issue_main(false, true, BAR_DRAIN_B);
+    } else if (lane == 0) {
       prefetch_tensormap(&tm_rf);
       const uint32_t idesc_l = make_idesc_bf16(256, BK, 0, 0);
       const int lsteps = args.r16 / 16;
@@ -218,6 +307,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       const uint64_t d_sf0 = make_sdesc(smem + OFF_FSLOTS + PR::FS_SF, 16, 16u * args.sf_cols, sf_swz);
       constexpr uint32_t FSLOT_D = FSLOT_BYTES >> 4;
       uint32_t it = 0, g = 0;
+      Cursor f;
       bool ok = true;
       for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
         const int rb2 = tile % num_rb2;
@@ -228,8 +318,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           if (!(ok = wait_spin_bounded(bar(BAR_RFFULL), it & 1u, ctl, 6))) break;
           for (int kk = 0; kk < nk && ok; ++kk) {
             // L(gg) into buffer gg % NLB once both factor halves landed and both CTAs read L(gg - NLB)
-            const uint32_t gg = g + kk, s = gg % NF, b = gg % NLB;
-            if (!(ok = wait_spin_bounded(bar(BAR_FFULL + s), (gg / NF) & 1u, ctl, 4))) break;
+            const uint32_t gg = g + kk, s = f.s, b = gg % NLB;
+            if (!(ok = wait_spin_bounded(bar(BAR_FFULL + s), f.ph, ctl, 4))) break;
+            f.next(NF);
             if (!(ok = wait_spin_bounded(bar(BAR_LEMPTY + b), ((gg / NLB) & 1u) ^ 1u, ctl, 5))) break;
             tc_fence_after();
             const uint64_t sf = d_sf0 + s * FSLOT_D;
@@ -249,43 +340,49 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           ok = wait_spin_bounded(bar(BAR_LEMPTY + gg % NLB), (gg / NLB) & 1u, ctl, 11);
       }
     }
-  } else if (warp >= FIRST_TMA_WARP && warp < FIRST_TMA_WARP + NT_MAX) {
-    // ------------------------------------------- token loaders (one per slot)
-    const uint32_t t = warp - FIRST_TMA_WARP;   // slots past NT have no loader work
-    if (lane == 0 && t < static_cast<uint32_t>(NT)) {
+  } else if (warp >= FIRST_TMA_WARP && warp < FIRST_TMA_WARP + NUM_TOK_LOADERS) {
+    // ------------------------------------ token loaders (one warp's copies come one after another)
+    // Loader t takes the stages t, t + NL4, ...  A loader waits for the product of stage gg - NT in
+    // a barrier phase that the next but one use of the slot would alias: it must know that stage
+    // gg - 2 NT has finished, which its previous wait (stage gg - NL4 - NT) tells it for NL4 <= NT.
+    const int NL4 = NT < NUM_TOK_LOADERS ? NT : NUM_TOK_LOADERS;
+    if (lane == 0 && warp - FIRST_TMA_WARP < NL4) {
       prefetch_tensormap(&tm_tok);
-      const uint32_t st = smem + OFF_TSLOTS + t * TSLOT_BYTES;
-      const uint32_t fb = lbar(BAR_TFULL + t), eb = bar(BAR_TEMPTY + t);
-      uint32_t g = 0;
+      int kk = warp - FIRST_TMA_WARP;   // this loader's next stage of the tile
+      Cursor c;
+      c.skip(kk, NT);
       bool ok = true;
       for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
-        const int tb = tile / num_rb2;
-        for (int kk = 0; kk < nk; ++kk) {
-          const uint32_t gg = g + kk;
-          if (gg % NT != t) continue;
-          const uint32_t n = gg / NT;
-          if (!(ok = wait_spin_bounded(eb, (n & 1u) ^ 1u, ctl, 2))) break;
-          if (leader) mbar_arrive_expect_tx(bar(BAR_TFULL + t), 2u * TOK_BYTES);
-          const int tok = tb * BTP + static_cast<int>(rank) * BNH;
+        const int tok = tile / num_rb2 * btp + static_cast<int>(rank) * bnh;
+        for (; kk < nk; kk += NL4) {
+          if (!(ok = wait_spin_bounded(bar(BAR_TEMPTY + c.s), c.ph ^ 1u, ctl, 2))) break;
+          if (leader) mbar_arrive_expect_tx(bar(BAR_TFULL + c.s), 128u * btp);
+          const uint32_t st = smem + OFF_TSLOTS + c.s * TSLOT_BYTES, fb = lbar(BAR_TFULL + c.s);
           tma_load_2d_pair(st, &tm_tok, kk * BK, tok, fb);
-          tma_load_2d_pair(st + TOK_BOX, &tm_tok, kk * BK, tok + BNP, fb);
+          if (nacc == 2) tma_load_2d_pair(st + TOK_BOX, &tm_tok, kk * BK, tok + bnp, fb);
+          c.skip(NL4, NT);
         }
-        g += nk;
+        kk -= nk;
       }
     }
-  } else if (warp == FIRST_TMA_WARP + NT_MAX) {
+  } else if (warp == FIRST_TMA_WARP + NUM_TOK_LOADERS) {
     // ------------------------------------------------- factor-ring loader
     if (lane == 0) {
       prefetch_tensormap(&tm_phi);
       if (!NL) prefetch_tensormap(&tm_sf);
       const uint32_t sf_tx = static_cast<uint32_t>(32 * 2 * args.sf_cols);   // one CTA's half slice
-      uint32_t gg = 0;
-      bool ok = true;
+      Cursor f;
+      uint32_t last = 0, last_ph = 0;   // the last copy's slot and parity
+      bool any = false, ok = true;
       for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
         const int rb2 = tile % num_rb2;
-        for (int kk = 0; kk < nk; ++kk, ++gg) {
-          const uint32_t s = gg % NF;
-          if (!(ok = wait_spin_bounded(bar(BAR_FEMPTY + s), ((gg / NF) & 1u) ^ 1u, ctl, 3))) break;
+        for (int kk = 0; kk < nk; ++kk) {
+          const uint32_t s = f.s;
+          if (!(ok = wait_spin_bounded(bar(BAR_FEMPTY + s), f.ph ^ 1u, ctl, 3))) break;
+          any = true;
+          last = s;
+          last_ph = f.ph;
+          f.next(NF);
           const uint32_t fs = smem + OFF_FSLOTS + s * FSLOT_BYTES;
           constexpr uint32_t XTX = MODE == FUSED_DX        ? (ZP ? 256u : 128u)
                                    : MODE == FUSED_FWD_GROUP ? (ZP ? 512u : 256u)
@@ -296,17 +393,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           if (MODE == FUSED_DX) {
             // the stage's 64 scales (and zero offsets) of this CTA's row group (group sizes are
             // multiples of 128, so a CTA's 128 rows lie in one group)
-            const int64_t xoff = (args.s_ld ? static_cast<int64_t>((rb2 * 2 * BM + static_cast<int>(rank) * BM) /
-                                                                   args.group_size) * args.kdim
-                                            : 0) + kk * BK;
+            const int64_t xoff = (args.s_ld ? static_cast<int64_t>(row_block(rb2) / args.group_size) * args.kdim : 0) +
+                                 kk * BK;
             bulk_load(fs + PR::FS_X, args.s_bf16 + xoff, 128u, bar(BAR_PFULL + s));
             if (ZP) bulk_load(fs + PR::FS_X + 512u, args.z_bf16 + xoff, 128u, bar(BAR_PFULL + s));
           } else if (MODE == FUSED_FWD_GROUP) {
             // the 128 scales (and zero offsets) of this CTA's rows in the stage's group, from the
             // bf16 rows [groups][m] (a group holds a multiple of 128 contraction indices, so two
             // stages never straddle it)
-            const int64_t xoff = static_cast<int64_t>((kk * BK) / args.group_size) * args.rows + rb2 * 2 * BM +
-                                 static_cast<int>(rank) * BM;
+            const int64_t xoff = static_cast<int64_t>((kk * BK) / args.group_size) * args.rows + row_block(rb2);
             bulk_load(fs + PR::FS_X, args.s_bf16 + xoff, 256u, bar(BAR_PFULL + s));
             if (ZP) bulk_load(fs + PR::FS_X + 512u, args.z_bf16 + xoff, 256u, bar(BAR_PFULL + s));
           }
@@ -316,53 +411,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           }
         }
       }
-      if (gg > 0) {
-        const uint32_t last = gg - 1;
-        drain_wait(bar(BAR_PFULL + last % NF), (last / NF) & 1u, args.timeout_ns);
-      }
+      if (any) drain_wait(bar(BAR_PFULL + last), last_ph, args.timeout_ns);
     }
   } else if (warp == 1) {
     // ------------------------------------ main-product MMA issuer (the leader's)
-    if (leader && lane == 0) {
-      const uint32_t idesc_main = make_idesc_bf16(256, BNP, 0, 0);
-      constexpr uint32_t TSLOT_D = TSLOT_BYTES >> 4, TOKB_D = TOK_BOX >> 4;
-      const uint64_t d_w0 = make_sdesc(smem + OFF_TSLOTS + TS_W, 16, 1024, SWZ_128B);
-      const uint64_t d_tok0 = make_sdesc(smem + OFF_TSLOTS, 16, 1024, SWZ_128B);
-      uint32_t g = 0, it = 0;
-      bool ok = true;
-      for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
-        if (!(ok = wait_spin_bounded(bar(BAR_ACCEMPTY), (it & 1u) ^ 1u, ctl, 7))) break;
-        tc_fence_after();
-        // unrolled: the loop's own overhead between two stages' MMAs was ~120 cycles of idle tensor pipe
-#pragma unroll 4
-        for (int kk = 0; kk < nk; ++kk) {
-          const uint32_t gg = g + kk;
-          const uint32_t s = gg % NT, ph = (gg / NT) & 1u;
-          if (!(ok = wait_spin_bounded(bar(BAR_TFULL + s), ph, ctl, 9))) break;
-          tc_fence_after();
-          const uint64_t w = d_w0 + s * TSLOT_D, t = d_tok0 + s * TSLOT_D;
-          const uint32_t acc = kk > 0 ? 1u : 0u;
-          static_assert(NACC == 2 && BK == 64, "issue sequence below is written for 2 accumulators x 4 K steps");
-          mma_bf16_pair(tmem, w, t, idesc_main, acc);
-          mma_bf16_pair(tmem, w + 2, t + 2, idesc_main, 1u);
-          mma_bf16_pair(tmem, w + 4, t + 4, idesc_main, 1u);
-          mma_bf16_pair(tmem, w + 6, t + 6, idesc_main, 1u);
-          mma_bf16_pair(tmem + BNP, w, t + TOKB_D, idesc_main, acc);
-          mma_bf16_pair(tmem + BNP, w + 2, t + TOKB_D + 2, idesc_main, 1u);
-          mma_bf16_pair(tmem + BNP, w + 4, t + TOKB_D + 4, idesc_main, 1u);
-          mma_bf16_pair(tmem + BNP, w + 6, t + TOKB_D + 6, idesc_main, 1u);
-          mma_commit_pair(bar(BAR_TEMPTY + s));
-        }
-        if (!ok) break;
-        mma_commit_pair(bar(BAR_ACCFULL));
-        g += nk;
-        ++it;
-      }
-      // the peer's last drain report lands before the CTAs end
-      if (ok) ok = wait_spin_bounded(bar(BAR_ACCEMPTY), (it & 1u) ^ 1u, ctl, 10);
-      mma_commit_pair_self(bar(BAR_DRAIN));
-      drain_wait(bar(BAR_DRAIN), 0, args.timeout_ns);
-    }
+    if (leader && lane == 0) issue_main(true, !NL && nacc == 2, BAR_DRAIN);
   } else {
     // ------------------------------------------- W_hat producers + epilogue
     const int pw = warp - 2;              // 0..15
@@ -372,144 +425,179 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     const uint32_t lane_off = static_cast<uint32_t>(q * 32) << 16;
     const QuantParams qp = args.q;
     const uint32_t lr2 = pack_rn_bf16x2(qp.lr_scale, qp.lr_scale);
-    // On the codes each warp builds two stages per iteration: both bases are read before either is
-    // decoded and one proxy fence covers both W_hat stores, so that the per-stage chain of
-    // shared-memory round trips (base read, W_hat store, fence, reports) is paid once per two
-    // stages (kdim is a multiple of 128, so nk is even).
-    constexpr int SPI = NL ? 2 : 1;
     uint32_t g = 0;
     uint32_t it = 0;
+    Cursor fc, tc;   // factor and token slots
+    if (NL) {
+      fc.skip(c, NF);
+      tc.skip(c, NT);
+    }
     bool ok = true;
     for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
       const int rb2 = tile % num_rb2;
       const int tb = tile / num_rb2;
-      const int row_g = rb2 * 2 * BM + static_cast<int>(rank) * BM + row;
-      for (int kk = 0; kk < nk; kk += SPI) {
-        uint32_t scw[SPI][8];   // dX: the stage's 16 bf16 scales of its contraction indices, as bf16x2
-        uint32_t zw[SPI][8];    // zero offsets as bf16x2
-        uint32_t sgw[SPI];      // group-wise forward: the stage's scale as bf16x2
-        if (ZP && MODE == FUSED_FWD_PC) {
-          // per-channel forward: this row's zero offset (dX and the group-wise forward read theirs
-          // from the factor slot below)
-          const uint32_t z2 = pack_rn_bf16x2(args.zero[row_g], args.zero[row_g]);
-#pragma unroll
-          for (int j = 0; j < SPI; ++j)
-#pragma unroll
-            for (int e = 0; e < 8; ++e) zw[j][e] = z2;
-        }
-        // the stages' stored bases, each read as soon as it has landed
-        uint32_t raw[SPI][8];
-#pragma unroll
-        for (int j = 0; j < SPI; ++j) {
-          const uint32_t gj = g + kk + j, fslot = gj % NF;
-          ok = wait_bounded(bar(BAR_PFULL + fslot), (gj / NF) & 1u, ctl, 12);
+      const int row_g = row_block(rb2) + row;
+      const bool has_rows = rb2 * 2 * BM + static_cast<int>(rank) * BM < args.rows;
+      if constexpr (NL) {
+        // Group c's stages of the tile (gg % 4 == c).  A ready barrier costs a test of ~110 cycles and
+        // the proxy fence and reports ~100 more, whatever the warp does between them: with all sixteen
+        // warps in every stage these made a stage 770 cycles (4096 x 4096, 32-token tiles), four
+        // groups in flight pay them side by side (596 cycles; 256-token tiles 863 -> 700).
+        for (int kk = static_cast<int>((static_cast<uint32_t>(c) - g) & 3u); kk < nk; kk += NUM_GROUPS) {
+          ok = wait_bounded(bar(BAR_PFULL + fc.s), fc.ph, ctl, 12);
           if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-          const uint32_t fs = smem + OFF_FSLOTS + fslot * FSLOT_BYTES;
+          const uint32_t fs = smem + OFF_FSLOTS + fc.s * FSLOT_BYTES;
+          uint4 raw[4];
+#pragma unroll
+          for (int x = 0; x < 4; ++x) raw[x] = ld_shared_v4(fs + swz_offset(row, x, 64));
+          uint32_t sg = 0, zg = 0;   // forward: the row's scale and zero offset in the stage, as bf16x2
+          if (MODE == FUSED_FWD_GROUP) {
+            sg = ld_shared_u16(fs + PR::FS_X + 2u * row);
+            sg |= sg << 16;
+            if (ZP) {
+              zg = ld_shared_u16(fs + PR::FS_X + 512u + 2u * row);
+              zg |= zg << 16;
+            }
+          } else if (MODE == FUSED_FWD_PC && ZP) {
+            zg = pack_rn_bf16x2(args.zero[row_g], args.zero[row_g]);
+          }
+          uint32_t w[32];
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const uint32_t in[4] = {raw[x].x, raw[x].y, raw[x].z, raw[x].w};
+            if (args.codes_bias == 64) {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) decode_b64_bf16x4(in[i], w[8 * x + 2 * i], w[8 * x + 2 * i + 1]);
+            } else {
+              float v[16];
+              decode_ob16(in, v);
+#pragma unroll
+              for (int e = 0; e < 8; ++e) w[8 * x + e] = pack_int_bf16x2(v[2 * e], v[2 * e + 1]);
+            }
+          }
+#pragma unroll
+          for (int x = 0; x < 8; ++x) {
+            if (MODE == FUSED_DX) {
+              // the bf16 scales (zero offsets) of eight contraction indices, as bf16x2 words
+              const uint4 s4 = ld_shared_v4(fs + PR::FS_X + 16u * x);
+              if (ZP) {
+                const uint4 z4 = ld_shared_v4(fs + PR::FS_X + 512u + 16u * x);
+                w[4 * x] = sub_bf16x2(w[4 * x], z4.x), w[4 * x + 1] = sub_bf16x2(w[4 * x + 1], z4.y);
+                w[4 * x + 2] = sub_bf16x2(w[4 * x + 2], z4.z), w[4 * x + 3] = sub_bf16x2(w[4 * x + 3], z4.w);
+              }
+              w[4 * x] = mul_bf16x2(w[4 * x], s4.x), w[4 * x + 1] = mul_bf16x2(w[4 * x + 1], s4.y);
+              w[4 * x + 2] = mul_bf16x2(w[4 * x + 2], s4.z), w[4 * x + 3] = mul_bf16x2(w[4 * x + 3], s4.w);
+            } else {
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                if (ZP) w[4 * x + e] = sub_bf16x2(w[4 * x + e], zg);
+                if (MODE == FUSED_FWD_GROUP) w[4 * x + e] = mul_bf16x2(w[4 * x + e], sg);
+              }
+            }
+          }
+          // the slot's W_hat buffer was last read by the product of the stage NT before
+          ok = wait_bounded(bar(BAR_TEMPTY + tc.s), tc.ph ^ 1u, ctl, 14);
+          if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+          const uint32_t wt = smem + OFF_TSLOTS + tc.s * TSLOT_BYTES + TS_W;
+#pragma unroll
+          for (int x = 0; x < 8; ++x)
+            st_shared_v4(wt + swz_offset(row, x, 128), w[4 * x], w[4 * x + 1], w[4 * x + 2], w[4 * x + 3]);
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            report(BAR_TFULL + tc.s, q, GROUP_WARPS);
+            mbar_arrive(bar(BAR_FEMPTY + fc.s));
+          }
+          fc.skip(NUM_GROUPS, NF);
+          tc.skip(NUM_GROUPS, NT);
+        }
+      } else {
+        for (int kk = 0; kk < nk; ++kk) {
+          uint32_t scw[8];   // dX: the stage's 16 bf16 scales of its contraction indices, as bf16x2
+          uint32_t zw[8];    // zero offsets as bf16x2
+          uint32_t sgw = 0;  // group-wise forward: the stage's scale as bf16x2
+          if (ZP && MODE == FUSED_FWD_PC) {
+            // per-channel forward: this row's zero offset (dX and the group-wise forward read theirs
+            // from the factor slot below)
+            const uint32_t z2 = pack_rn_bf16x2(args.zero[row_g], args.zero[row_g]);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) zw[e] = z2;
+          }
+          // the stage's stored base, read as soon as it has landed
+          uint32_t raw[8];
+          ok = wait_bounded(bar(BAR_PFULL + fc.s), fc.ph, ctl, 12);
+          if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+          const uint32_t fs = smem + OFF_FSLOTS + fc.s * FSLOT_BYTES;
           if (PACKED) {
             const uint2 r = ld_shared_v2(fs + swz_offset(row, c >> 1, 32) + 8 * (c & 1));
-            raw[j][0] = r.x;
-            raw[j][1] = r.y;
+            raw[0] = r.x;
+            raw[1] = r.y;
           } else if (fmt_16bit(FMT)) {
             const uint4 r0 = ld_shared_v4(fs + swz_offset(row, 2 * c, 128));
             const uint4 r1 = ld_shared_v4(fs + swz_offset(row, 2 * c + 1, 128));
-            raw[j][0] = r0.x, raw[j][1] = r0.y, raw[j][2] = r0.z, raw[j][3] = r0.w;
-            raw[j][4] = r1.x, raw[j][5] = r1.y, raw[j][6] = r1.z, raw[j][7] = r1.w;
+            raw[0] = r0.x, raw[1] = r0.y, raw[2] = r0.z, raw[3] = r0.w;
+            raw[4] = r1.x, raw[5] = r1.y, raw[6] = r1.z, raw[7] = r1.w;
           } else {
             const uint4 r = ld_shared_v4(fs + swz_offset(row, c, 64));
-            raw[j][0] = r.x, raw[j][1] = r.y, raw[j][2] = r.z, raw[j][3] = r.w;
+            raw[0] = r.x, raw[1] = r.y, raw[2] = r.z, raw[3] = r.w;
           }
           if (MODE == FUSED_DX) {
             // the 16 bf16 scales (zero offsets) of this warp's contraction indices, as bf16x2 words
             const uint4 s0 = ld_shared_v4(fs + PR::FS_X + 32u * c), s1 = ld_shared_v4(fs + PR::FS_X + 32u * c + 16u);
-            scw[j][0] = s0.x, scw[j][1] = s0.y, scw[j][2] = s0.z, scw[j][3] = s0.w;
-            scw[j][4] = s1.x, scw[j][5] = s1.y, scw[j][6] = s1.z, scw[j][7] = s1.w;
+            scw[0] = s0.x, scw[1] = s0.y, scw[2] = s0.z, scw[3] = s0.w;
+            scw[4] = s1.x, scw[5] = s1.y, scw[6] = s1.z, scw[7] = s1.w;
             if (ZP) {
               const uint4 z0 = ld_shared_v4(fs + PR::FS_X + 512u + 32u * c);
               const uint4 z1 = ld_shared_v4(fs + PR::FS_X + 512u + 32u * c + 16u);
-              zw[j][0] = z0.x, zw[j][1] = z0.y, zw[j][2] = z0.z, zw[j][3] = z0.w;
-              zw[j][4] = z1.x, zw[j][5] = z1.y, zw[j][6] = z1.z, zw[j][7] = z1.w;
+              zw[0] = z0.x, zw[1] = z0.y, zw[2] = z0.z, zw[3] = z0.w;
+              zw[4] = z1.x, zw[5] = z1.y, zw[6] = z1.z, zw[7] = z1.w;
             }
           } else if (MODE == FUSED_FWD_GROUP) {
             // this thread's row's scale (and zero offset) in the stage's group, as bf16x2
             const uint32_t sv = ld_shared_u16(fs + PR::FS_X + 2u * row);
-            sgw[j] = sv | (sv << 16);
+            sgw = sv | (sv << 16);
             if (ZP) {
               const uint32_t zv = ld_shared_u16(fs + PR::FS_X + 512u + 2u * row);
 #pragma unroll
-              for (int e = 0; e < 8; ++e) zw[j][e] = zv | (zv << 16);
+              for (int e = 0; e < 8; ++e) zw[e] = zv | (zv << 16);
             }
           }
-        }
-        if (!ok) break;
-        uint32_t w[SPI][8];
-#pragma unroll
-        for (int j = 0; j < SPI; ++j) {
-          const uint32_t gj = g + kk + j;
-          float v[16];
-          // the codes base with the clipped codes stored as c + 64: bf16 straight from the bytes
-          const bool b64 = NL && args.codes_bias == 64;
-          uint32_t c8[8];
-          if (b64) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) decode_b64_bf16x4(raw[j][i], c8[2 * i], c8[2 * i + 1]);
-          } else if (NL) {
-            decode_ob16(raw[j], v);
-          } else {
-            decode16<FMT>(raw[j], v);
-          }
-          float Lv[16];
-          if (!NL) {
-            const uint32_t lb = gj % NLB;
-            ok = wait_bounded(bar(BAR_LFULL + lb), (gj / NLB) & 1u, ctl, 13);
-            if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-            tc_fence_after();
-            tmem_ld16(tmem + lane_off + COL_L + BK * lb + 16 * c, Lv);
-            tmem_ld_wait();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) report(BAR_LEMPTY + lb, pw);
-          }
+          float v[16], Lv[16];
+          decode16<FMT>(raw, v);
+          const uint32_t lb = (g + kk) % NLB;
+          ok = wait_bounded(bar(BAR_LFULL + lb), ((g + kk) / NLB) & 1u, ctl, 13);
+          if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+          tc_fence_after();
+          tmem_ld16(tmem + lane_off + COL_L + BK * lb + 16 * c, Lv);
+          tmem_ld_wait();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) report(BAR_LEMPTY + lb, pw, NUM_PROD_WARPS);
+          uint32_t w[8];
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
-            uint32_t cw;
-            if (NL) {
-              cw = b64 ? c8[e] : pack_int_bf16x2(v[2 * e], v[2 * e + 1]);
-            } else {
-              const float2 u = UB ? u_bf16x2(Lv[2 * e], Lv[2 * e + 1], v[2 * e], v[2 * e + 1], lr2)
-                                  : __ffma2_rn(make_float2(Lv[2 * e], Lv[2 * e + 1]),
-                                               make_float2(qp.lr_scale, qp.lr_scale),
-                                               make_float2(v[2 * e], v[2 * e + 1]));
-              cw = codes_bf16x2(__fadd2_rn(u, make_float2(qp.magic, qp.magic)), qp);
-            }
-            if (ZP) cw = sub_bf16x2(cw, zw[j][e]);
-            if (MODE == FUSED_FWD_PC) {
-              w[j][e] = cw;
-            } else {
-              w[j][e] = mul_bf16x2(cw, MODE == FUSED_DX ? scw[j][e] : sgw[j]);
-            }
+            const float2 u = UB ? u_bf16x2(Lv[2 * e], Lv[2 * e + 1], v[2 * e], v[2 * e + 1], lr2)
+                                : __ffma2_rn(make_float2(Lv[2 * e], Lv[2 * e + 1]),
+                                             make_float2(qp.lr_scale, qp.lr_scale),
+                                             make_float2(v[2 * e], v[2 * e + 1]));
+            uint32_t cw = codes_bf16x2(__fadd2_rn(u, make_float2(qp.magic, qp.magic)), qp);
+            if (ZP) cw = sub_bf16x2(cw, zw[e]);
+            w[e] = MODE == FUSED_FWD_PC ? cw : mul_bf16x2(cw, MODE == FUSED_DX ? scw[e] : sgw);
           }
-        }
-        if (!ok) break;
-        // Each stage's W_hat buffer (in its token slot) was last read by the product of stage gj - NT.
-#pragma unroll
-        for (int j = 0; j < SPI; ++j) {
-          const uint32_t gj = g + kk + j, ts = gj % NT;
-          ok = wait_bounded(bar(BAR_TEMPTY + ts), ((gj / NT) & 1u) ^ 1u, ctl, 14);
+          // the W_hat buffer (in the token slot) was last read by the product of the stage NT before
+          ok = wait_bounded(bar(BAR_TEMPTY + tc.s), tc.ph ^ 1u, ctl, 14);
           if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-          const uint32_t wt = smem + OFF_TSLOTS + ts * TSLOT_BYTES + TS_W;
-          st_shared_v4(wt + swz_offset(row, 2 * c, 128), w[j][0], w[j][1], w[j][2], w[j][3]);
-          st_shared_v4(wt + swz_offset(row, 2 * c + 1, 128), w[j][4], w[j][5], w[j][6], w[j][7]);
-        }
-        if (!ok) break;
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) {
-#pragma unroll
-          for (int j = 0; j < SPI; ++j) {
-            const uint32_t gj = g + kk + j;
-            report(BAR_TFULL + gj % NT, pw);
-            mbar_arrive(bar(BAR_FEMPTY + gj % NF));
+          const uint32_t wt = smem + OFF_TSLOTS + tc.s * TSLOT_BYTES + TS_W;
+          st_shared_v4(wt + swz_offset(row, 2 * c, 128), w[0], w[1], w[2], w[3]);
+          st_shared_v4(wt + swz_offset(row, 2 * c + 1, 128), w[4], w[5], w[6], w[7]);
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            report(BAR_TFULL + tc.s, pw, NUM_PROD_WARPS);
+            mbar_arrive(bar(BAR_FEMPTY + fc.s));
           }
+          fc.next(NF);
+          tc.next(NT);
         }
       }
       if (!ok) break;
@@ -522,12 +610,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       tc_fence_after();
       const bool odd = lane & 1;
 #pragma unroll 1
-      for (int ch = 0; ch < EPI_COLS / 16; ++ch) {
+      for (int col = has_rows ? 16 * c : btp; col < btp; col += 64) {   // token offset in the tile
         float acc[16];
-        const int col = c * EPI_COLS + 16 * ch;   // accumulator column = token offset in the tile
-        tmem_ld16(tmem + lane_off + col, acc);
+        tmem_ld16(tmem + lane_off + (col < bnp ? col : BNP + col - bnp), acc);
         tmem_ld_wait();
-        const int tok0 = tb * BTP + col;
+        const int tok0 = tb * btp + col;
         uint32_t mword = 0xffffffffu;
         if (MODE == FUSED_DX && args.xmask != nullptr && tok0 < args.T)
           mword = args.xmask[static_cast<int64_t>(row_g) * args.xmask_ld + tok0 / 32] >> (tok0 & 31);
@@ -537,7 +624,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) report(BAR_ACCEMPTY, pw);
+      if (lane == 0) report(BAR_ACCEMPTY, pw, NUM_PROD_WARPS);
       g += nk;
       ++it;
     }
@@ -556,10 +643,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 template <int MODE, int FMT, bool ZP, bool UB, bool NL>
 cudaError_t launch_pair_one(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c, const CUtensorMap& d,
                             const FusedArgs& args, int npairs, cudaStream_t stream) {
-  constexpr uint32_t smem = PairRing<FMT, NL, MODE == FUSED_DX || MODE == FUSED_FWD_GROUP>::SMEM_BYTES;
+  using PR = PairRing<FMT, NL, MODE == FUSED_DX || MODE == FUSED_FWD_GROUP>;
+  if (!NL && args.bnp * args.nacc > 448) return cudaErrorInvalidValue;
+  const uint32_t smem = PR::smem(args.bnp * args.nacc);
   static bool configured[kMaxDevices] = {};
   const void* fn = reinterpret_cast<const void*>(fused_pair_kernel<MODE, FMT, ZP, UB, NL>);
-  cudaError_t e = ensure_smem_attr(fn, static_cast<int>(smem), configured);
+  cudaError_t e = ensure_smem_attr(fn, 232448 - 1024, configured);   // the most any tile asks for
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(2 * npairs), 1, 1);
@@ -636,8 +725,9 @@ cudaError_t launch_pair_mode(int fmt, const CUtensorMap& a, const CUtensorMap& b
 cudaError_t launch_fused_pair(int mode, int fmt, const CUtensorMap& tm_tok, const CUtensorMap& tm_phi,
                               const CUtensorMap& tm_rf, const CUtensorMap& tm_sf, const FusedArgs& args, int npairs,
                               cudaStream_t stream) {
-  if (npairs < 1 || (args.kdim % 128) != 0 || args.kdim < 128 || (args.rows % 256) != 0 || args.sf_mn ||
-      args.num_rb != args.rows / 128)
+  if (npairs < 1 || (args.kdim % 128) != 0 || args.kdim < 128 || (args.rows % BM) != 0 || args.sf_mn ||
+      args.num_rb != args.rows / 128 || args.bnp < 16 || (args.bnp & 15) ||
+      !(args.nacc == 1 ? args.bnp <= 256 : args.nacc == 2 && args.bnp <= BNP))
     return cudaErrorInvalidValue;
   switch (mode) {
     case FUSED_FWD_PC: return launch_pair_mode<FUSED_FWD_PC>(fmt, tm_tok, tm_phi, tm_rf, tm_sf, args, npairs, stream);

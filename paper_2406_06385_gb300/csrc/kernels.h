@@ -172,15 +172,18 @@ struct FusedArgs {
   // [groups][kdim] (one row per channel scale), written by launch_dx_scales.
   const uint16_t* s_bf16;
   const uint16_t* z_bf16;
+  // Pair kernel: the token tile, nacc accumulators of bnp tokens (a multiple of 16; nacc 1: up to
+  // 256, 2: up to 224)
+  int32_t bnp, nacc;
 };
 // s_out[g][i] = bf16(s[i][g]) (s [m] per channel: g = 0 only) and, with z, z_out likewise: the
 // dX GEMM's producers read 16 consecutive of them per stage with two 16-byte loads.
 cudaError_t launch_dx_scales(const float* s, const float* z, int64_t m, int groups, int s_ld, uint16_t* s_out,
                              uint16_t* z_out, cudaStream_t stream);
 int fused_smem_bytes(int fmt);
-// The same GEMM on CTA pairs (fused_pair.cu): 256-row x 448-token tiles, npairs clusters of 2.
-// Needs rows % 256 == 0 and K-major factor slices (sf_mn == 0); tm_tok boxes of 112 tokens x
-// 64, tm_sf boxes of 32 slice rows x sf_cols; tm_phi and tm_rf as for launch_fused.
+// The same GEMM on CTA pairs (fused_pair.cu): tiles of 256 rows x nacc * bnp tokens, npairs
+// clusters of 2.  Needs rows % 128 == 0 and K-major factor slices (sf_mn == 0); tm_tok boxes of
+// bnp / 2 tokens x 64, tm_sf boxes of 32 slice rows x sf_cols; tm_phi and tm_rf as for launch_fused.
 cudaError_t launch_fused_pair(int mode, int fmt, const CUtensorMap& tm_tok, const CUtensorMap& tm_phi,
                               const CUtensorMap& tm_rf, const CUtensorMap& tm_sf, const FusedArgs& args, int npairs,
                               cudaStream_t stream);

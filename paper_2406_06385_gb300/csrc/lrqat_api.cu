@@ -127,15 +127,15 @@ int frac_bits(const lrqat_layer& L) { return L.phi_format == LRQAT_PHI_QFIXED ? 
 // Where the forward and dX GEMMs take the low-rank term from (lrqat_set_lowrank_path):
 // 1 = the tile that each GEMM stage computes next to the main product (ranks up to 64);
 // 2 = the codes pass: one tensor-core pass per call writes the code of every weight as a byte into
-// the workspace, and the GEMMs read those as their base with the low-rank term switched off.  In the pair GEMM the in-stage tile is a chain of small MMAs
-// whose TMEM buffer holds one stage, so it paces the stage (measured on a 4096 x 4096 layer at
-// T = 8192: forward 218 -> 191 us, dX 254 -> 210 us with the codes, for a pass of 18 us), while
-// the pass moves ~2 bytes per weight through HBM whatever T is.  Measured fwd + bwd per call,
-// tile against codes: 4096 x 4096 at T = 2048 353 / 355 us, at T = 4096 511 / 500 us;
-// 5120 x 13824 at T = 2048 1017 / 1044 us, at T = 4096 1657 / 1625 us.  So 0 (auto) takes the
-// codes from kCodesMinTokens tokens on.  Ranks above 64 always take the codes: their factor slices do not
-// fit next to the GEMMs' token ring, and recomputing A B per 448-token tile would cost r/448 of
-// the GEMM's own tensor work.  The same holds for dW, which otherwise computes its own tile.
+// the workspace, and the GEMMs read those as their base with the low-rank term switched off.
+// 0 (auto) = the codes wherever the workspace holds them (all but the allocation-free forward): the
+// in-stage tile is a chain of small MMAs whose TMEM buffer holds one stage, so it makes a stage ~1700
+// cycles against 550-1100 on the codes, and the pass itself takes 3 us on a 256 x 256 layer and 11
+// on 4096 x 4096.  Measured fwd / bwd per call, tile against codes: 256 x 256 at T = 64 12.3 / 31.4 us,
+// 11.0 / 24.3; 4096 x 4096 at T = 64 57.6 / 114 us, 32.8 / 74.0, at T = 2999 111 / 226 us, 70.0 / 161;
+// 11008 x 4096 at T = 448 58.6 / 302 us, 59.6 / 211.  Ranks above 64 take the codes in every setting:
+// their factor slices do not fit next to the GEMMs' token ring, and recomputing A B per token tile
+// would cost r / 448 of the GEMM's own tensor work.
 int lowrank_path_from_env() {
   const char* v = std::getenv("LRQAT_LOWRANK_PATH");
   if (v && std::strcmp(v, "tile") == 0) return 1;
@@ -143,11 +143,8 @@ int lowrank_path_from_env() {
   return 0;
 }
 std::atomic<int> g_lowrank_path{lowrank_path_from_env()};
-constexpr int64_t kCodesMinTokens = 3072;
-bool codes_gemm(const lrqat_layer& L, int64_t T) {
-  if (L.r > 64) return true;
-  const int v = g_lowrank_path.load(std::memory_order_relaxed);
-  return v == 2 || (v == 0 && T >= kCodesMinTokens);
+bool codes_gemm(const lrqat_layer& L) {
+  return L.r > 64 || g_lowrank_path.load(std::memory_order_relaxed) != 1;
 }
 bool phi_16bit(const lrqat_layer& L) { return L.phi_format == LRQAT_PHI_BF16 || L.phi_format == LRQAT_PHI_FP16; }
 int round16(int r) { return (r + 15) / 16 * 16; }
@@ -304,11 +301,12 @@ int dw_schedule_from_env() {
 std::atomic<int> g_dw_schedule{dw_schedule_from_env()};
 
 // Kernel of the forward and dX GEMMs (lrqat_set_gemm_variant): 0 = CTA pairs (fused_pair.cu)
-// wherever they were measured faster, which is every GEMM whose produced weight operand has a
-// multiple of 256 rows (with the dX scales read as bf16 rows, group-wise dX too: 916 -> 730 us on
-// the 14336 x 4096 g128 projection at T = 8192); 1 = the one-SM kernel (fused_gemm.cu) always;
-// 2 = pairs wherever the rows allow.  LRQAT_GEMM_VARIANT ("auto" / "single" / "pair") sets the
-// start value once, when the library is loaded.
+// wherever they were measured faster, which is every GEMM on the codes (an odd number of 128-row blocks
+// leaves half a pair without rows in the last one; 1664 x 13184 at T = 512, both odd, forward + backward
+// 415 us on one SM, 246 on pairs), and with the in-stage tile those without such a half (1408 x 896 at
+// T = 3: 19.3 us on one SM, which reads the factors themselves, 24.6 on pairs); 1 = the one-SM kernel (fused_gemm.cu)
+// always; 2 = pairs always.  LRQAT_GEMM_VARIANT ("auto" / "single" / "pair") sets the start value
+// once, when the library is loaded.
 int gemm_variant_from_env() {
   const char* v = std::getenv("LRQAT_GEMM_VARIANT");
   if (v && std::strcmp(v, "single") == 0) return 1;
@@ -316,12 +314,42 @@ int gemm_variant_from_env() {
   return 0;
 }
 std::atomic<int> g_gemm_variant{gemm_variant_from_env()};
-bool use_pair(int64_t rows) {
+bool use_pair(int64_t rows, bool codes) {
   const int v = g_gemm_variant.load(std::memory_order_relaxed);
-  return rows % 256 == 0 && v != 1;
+  return v == 2 || (v == 0 && (codes || rows % 256 == 0));
 }
-constexpr int kPairTokens = 448;   // tokens per pair tile (two accumulators of 224)
-
+// The pair GEMM's token tile: nacc accumulators of bnp tokens.
+struct TokenTile {
+  int bnp, nacc;
+  int tokens() const { return bnp * nacc; }
+};
+// The cheapest tile for `rows` weight rows, a contraction of kdim and T tokens on `pairs` pairs, by
+// the rounds of the busiest pair times a tile's cycles: kdim / 64 stages plus the drain.  Stage
+// cycles measured on a 4096 x 4096 layer on the codes (forward, T = 8192, drain taken off): one
+// accumulator 524 (32 tokens) to 605 (256), two 655 (288) to 997 (448), linear in between; dX, whose
+// producers also multiply by the scales, 557 to 692 and 749 to 1042; the drain 2500 + 10 per token.  Up to 256 tokens the stage is bound by the issue of four MMAs whatever their
+// N, beyond by the operands' shared-memory traffic, so 448 tokens are the cheapest per token
+// (2.2 cycles a stage against 2.4 at 256) and smaller tiles pay where 448 leave pairs idle:
+// T = 4096 takes 304 (three rounds; forward 107 -> 82 us, dX 111 -> 92), T = 1024 takes 256.
+// With the low-rank tile in the stage a stage takes ~1700 cycles whatever the tile (one low-rank
+// buffer paces it), so that path keeps 448.
+TokenTile pair_token_tile(int64_t rows, int64_t kdim, int64_t T, int pairs, bool codes, bool dx) {
+  TokenTile best{224, 2};
+  if (!codes) return best;
+  int64_t best_cost = -1;
+  for (int bt = 448; bt >= 32; bt -= 32) {
+    const int64_t tiles = ((rows + 255) / 256) * ((T + bt - 1) / bt);
+    const int64_t rounds = (tiles + pairs - 1) / pairs;
+    const int64_t stage = bt <= 256 ? (dx ? 538 + bt * 60 / 100 : 513 + bt * 36 / 100)
+                                    : (dx ? 749 + (bt - 288) * 183 / 100 : 655 + (bt - 288) * 214 / 100);
+    const int64_t cost = rounds * (kdim / 64 * stage + 2500 + 10 * bt);
+    if (best_cost < 0 || cost < best_cost) {
+      best_cost = cost;
+      best = bt <= 256 ? TokenTile{bt, 1} : TokenTile{bt / 2, 2};
+    }
+  }
+  return best;
+}
 constexpr int kDwPairTokensPerStage = 64;   // the pair dW kernel's stage (dw_pair.cu)
 // dW on CTA pairs (dw_pair.cu): 256 x 256 tiles, ranks up to 64, by the same setting as the
 // forward and dX GEMMs (lrqat_set_gemm_variant: not with 1, the one-SM kernels).
@@ -760,8 +788,8 @@ static int linear_fwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
   FwdWs ws;
   fwd_ws_layout(L, T, allow_codes, workspace, &ws);
   const int r16 = round16(L.r);
-  const bool cb = L.r > 64 || (allow_codes && codes_gemm(L, T));
-  const bool pair = use_pair(L.m);
+  const bool cb = L.r > 64 || (allow_codes && codes_gemm(L));
+  const bool pair = use_pair(L.m, cb);
   // the pair kernel reads K-major factor slices, so it takes B^T from the padded copy
   const bool direct = !cb && !pair && direct_factors(L, A, B);
   if (cb) {
@@ -797,7 +825,8 @@ static int linear_fwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
     tok = ws.x_codes;
   }
   CUtensorMap tm_tok, tm_phi, tm_rf, tm_sf;
-  LRQAT_TRY(encode_2d(&tm_tok, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, tok, L.k, T, L.k * 2, 64, pair ? 112 : 224,
+  const TokenTile tile = pair_token_tile(L.m, L.k, T, dev->sms / 2, cb, false);
+  LRQAT_TRY(encode_2d(&tm_tok, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, tok, L.k, T, L.k * 2, 64, pair ? tile.bnp / 2 : 224,
                       CU_TENSOR_MAP_SWIZZLE_128B, "X"));
   if (cb) {
     // the codes as an 8-bit base; the factor maps are not read
@@ -857,7 +886,9 @@ static int linear_fwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
     a.z_bf16 = ws.z_bf16;
   }
   if (pair) {
-    const int64_t tiles = (L.m / 256) * ((T + kPairTokens - 1) / kPairTokens);
+    a.bnp = tile.bnp;
+    a.nacc = tile.nacc;
+    const int64_t tiles = ((L.m + 255) / 256) * ((T + tile.tokens() - 1) / tile.tokens());
     const int npairs = static_cast<int>(tiles < dev->sms / 2 ? tiles : dev->sms / 2);
     LRQAT_LAUNCH("fused_fwd", 1, stream, launch_fused_pair(fmode, ffmt, tm_tok, tm_phi, tm_rf, tm_sf, a, npairs, stream),
                  "fused forward launch (CTA pairs)");
@@ -941,7 +972,7 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
   const int fmt_t = L.phi_format == LRQAT_PHI_INT_PACKED ? LRQAT_PHI_QFIXED : L.phi_format;
   // cb: the dX GEMM reads the codes (lrqat_set_lowrank_path); cbw: so does dW, with the clip mask in
   // the byte's top bit (needs codes of 7 bits; the pair kernel, and every rank above 64)
-  const bool cb = codes_gemm(L, T);
+  const bool cb = codes_gemm(L);
   const bool cbw = L.r > 64 || (cb && plan.pair && L.bits <= 7);
   const bool direct_ab = direct_factors(L, A, B);
   // with direct factors the dX GEMM reads its A slices from A itself (its row factor stays the
@@ -996,9 +1027,10 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
       LRQAT_LAUNCH("dx_scales", 1, stream,
                    launch_dx_scales(s, L.zero, L.m, groups, L.group_size ? groups : 0, ws.s_bf16, ws.z_bf16, stream),
                    "dX scale rows");
-    const bool pair = use_pair(L.k);
+    const bool pair = use_pair(L.k, cb);
     CUtensorMap tm_tok, tm_phi, tm_rf, tm_sf;
-    LRQAT_TRY(encode_2d(&tm_tok, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, dY, L.m, T, L.m * 2, 64, pair ? 112 : 224,
+    const TokenTile tile = pair_token_tile(L.k, L.m, T, dev->sms / 2, cb, true);
+    LRQAT_TRY(encode_2d(&tm_tok, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, dY, L.m, T, L.m * 2, 64, pair ? tile.bnp / 2 : 224,
                         CU_TENSOR_MAP_SWIZZLE_128B, "dY"));
     if (phi_16bit(L) && !cb)
       LRQAT_TRY(encode_2d(&tm_phi, CU_TENSOR_MAP_DATA_TYPE_UINT16, ws.phit, L.m, L.k, L.m * 2, 64, 128,
@@ -1047,7 +1079,9 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
     a.timeout_ns = kWaitTimeoutNs;
     const int dfmt = cb ? LRQAT_PHI_QFIXED : fmt_t;
     if (pair) {
-      const int64_t tiles = (L.k / 256) * ((T + kPairTokens - 1) / kPairTokens);
+      a.bnp = tile.bnp;
+      a.nacc = tile.nacc;
+      const int64_t tiles = ((L.k + 255) / 256) * ((T + tile.tokens() - 1) / tile.tokens());
       const int npairs = static_cast<int>(tiles < dev->sms / 2 ? tiles : dev->sms / 2);
       LRQAT_LAUNCH("fused_dx", 1, stream,
                    launch_fused_pair(FUSED_DX, dfmt, tm_tok, tm_phi, tm_rf, tm_sf, a, npairs, stream),

@@ -59,6 +59,40 @@ def test_gradients_from_codes_equal_those_from_the_low_rank_tile(cid, spec, T, s
     assert float((a - b).norm() / b.norm()) <= 4e-3
 
 
+TILE_CASES = [
+    # odd numbers of 128-row blocks in both directions, token counts around the tiles' edges
+    ("odd_blocks", _spec(384, 640, 32), 225),
+    ("one_block", _spec(128, 128, 8), 33),
+    ("odd_group_asym", _spec(128, 384, 16, bits=3, group=128, asym=True), 449),
+    ("two_rounds", _spec(640, 384, 32, group=128), 20011),
+    ("bf16_8_bits", _spec(384, 256, 16, bits=8, phi=WL.PHI_BF16), 257),
+]
+
+
+@pytest.mark.parametrize("path", ["tile", "codes"])
+@pytest.mark.parametrize("cid,spec,T", TILE_CASES, ids=[c[0] for c in TILE_CASES])
+def test_pair_gemm_equals_the_one_sm_kernel(cid, spec, T, path, lowrank_path, gemm_variant):
+    """Y and dX of the pair kernel against the one-SM kernel's: the same W_hat and products summed in
+    the same K order, so bf16 outputs agree to a rounding of sums that differ in the last fp32 bits."""
+    t = torch()
+    lowrank_path(path)
+    data = WL.make_layer(spec, T, seed=6)
+    dl = DeviceLayer(data, 1.05)
+    X, dY = to_dev(data.X_bits), to_dev(data.dY_bits)
+    got = {}
+    for variant in ("single", "pair"):
+        gemm_variant(variant)
+        Y = t.full((T + 1, spec.m), 0x7FC0, dtype=t.int16, device="cuda")
+        ws = t.empty(LQ.fwd_workspace_bytes(dl.layer, T), dtype=t.uint8, device="cuda")
+        LQ.linear_fwd(dl.layer, T, X, dl.phi0, dl.s, dl.A, dl.B, None, Y, ws)
+        dX = _grads(spec, T, dl, X, dY, None)[0]
+        assert bool((Y[T] == 0x7FC0).all())   # nothing is written past the last token
+        got[variant] = [x.view(t.bfloat16).float() for x in (Y[:T], dX)]
+    for a, b in zip(*got.values()):
+        assert bool(t.isfinite(b).all())
+        assert float((a - b).norm() / a.norm()) <= 2.0 ** -9
+
+
 def test_codes_of_unaligned_factors_and_outputs():
     """The merge writes the same codes from padded factors, and to a 16-byte aligned output that is
     not 32-byte aligned."""
