@@ -331,8 +331,10 @@ int lrqat_set_gemm_variant(int variant);
  * to 64); 2 = "codes": one tensor-core pass per call writes the code of every weight as one
  * byte (clip(round(u), n, p) + 64, or + 128 for 8-bit weights) into the workspace and the
  * GEMMs read those bytes as their base, with no low-rank work in the stage; 0 (the default)
- * = codes, except in the allocation-free forward, whose scratch does not hold them (the pass costs
- * two bytes of HBM traffic per weight, the tile a low-rank MMA chain per stage).  Ranks above 64
+ * = codes in the backward, and in the forward by a cost model (the pass costs two bytes of HBM
+ * traffic per weight, the tile a low-rank MMA chain per stage); never in the allocation-free forward,
+ * whose scratch does not hold them.  Up to 16 tokens the forward takes a kernel of its own that forms
+ * the codes in registers (unless this or lrqat_set_gemm_variant is set).  Ranks above 64
  * always take the codes pass.  dW reads the codes where
  * the pair kernels take it (m and k multiples of 256, up to 7 bits) and computes its own
  * low-rank tile elsewhere.  All settings give the same codes up to

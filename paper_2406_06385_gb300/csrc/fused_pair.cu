@@ -37,6 +37,7 @@
 // otherwise) the base holds the one-byte codes of the codes pass; no factors, no L.
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <atomic>
 #include <cstdint>
 
 #include "kernels.h"
@@ -49,10 +50,10 @@ namespace {
 constexpr int BM = 128;                          // weight rows per CTA (256 per pair)
 constexpr int BK = 64;
 constexpr int BNP = 224;                         // most tokens per accumulator of two (N of the pair MMA)
-constexpr int BNH = BNP / 2;                     // tokens per accumulator held by one CTA
 constexpr int NACC = 2;                          // accumulators (one for tiles of up to 256 tokens)
 constexpr int NT_MAX = 8;                        // token ring slots
-constexpr int NLB = 1;                           // low-rank TMEM buffers
+constexpr int NLB = 4;                           // low-rank TMEM buffers (one per producer group)
+constexpr int MAX_TILE_L = 256;                  // most tokens of a tile beside them
 constexpr int NF_MAX = 8;                        // factor ring slots
 constexpr int NUM_PROD_WARPS = 16;
 constexpr int FIRST_TMA_WARP = 2 + NUM_PROD_WARPS;
@@ -69,12 +70,10 @@ constexpr uint32_t W_BYTES = 128 * 128;          // 128 rows x 64 bf16
 constexpr uint32_t SFH_BYTES = 32 * 128;         // 32 slice rows x up to 64 rank columns (bf16)
 
 // Shared-memory rings.  A token slot holds this CTA's half of the stage's tokens (a tile of btp
-// tokens: 64 btp bytes) and its W_hat tile, a factor slot the stored base.  With the low-rank tile:
-// the row factor, three token slots of 448 tokens, and this CTA's half of the second factor's slice
-// in each of four (16-bit bases: two) factor slots.  On the codes (NL): as many token slots as the
-// tile leaves room for beside at least four factor slots, and factor slots in the rest (up to eight
-// of each): a slot is refilled by TMA only after its stage's MMAs, so the shorter the stage, the
-// more stages it takes to cover a load's latency.
+// tokens: 64 btp bytes) and its W_hat tile, a factor slot the stored base and, with the low-rank tile
+// (which also has the row factor resident), this CTA's half of the second factor's slice.  As many
+// token slots as the tile leaves room for beside four factor slots, and eight of these where the
+// rest allows (up to eight of each).
 // XS: each factor slot also holds the stage's scales (and zero offsets) as bf16, copied by the
 // factor loader, so that the producers read them from shared memory with the base instead of
 // from global memory: for dX the 64 scales of the stage's contraction indices in the CTA's row
@@ -94,25 +93,26 @@ struct PairRing {
   static_assert(FSLOT_BYTES % 1024 == 0 && FS_SF % 1024 == 0, "swizzled tiles must start on 1024-byte boundaries");
   __host__ __device__ static constexpr uint32_t tslot(int btp) { return 64u * btp + W_BYTES; }
   __host__ __device__ static constexpr int nt(int btp) {
-    if (!NL) return 3;
-    const int n = static_cast<int>((RING_BYTES - 4u * FSLOT_BYTES) / tslot(btp));
+    const int n = static_cast<int>((RING_BYTES - RF - 4u * FSLOT_BYTES) / tslot(btp));
     return n < NT_MAX ? n : NT_MAX;
   }
-  // on the codes four or eight, multiples of NUM_GROUPS: a group then knows that the previous use of
-  // a slot it waits for has landed (it was its own), so barrier phases cannot alias
+  // four or eight, multiples of NUM_GROUPS: a group then knows that the previous use of a slot it
+  // waits for has landed (it was its own), so barrier phases cannot alias
   __host__ __device__ static constexpr int nf(int btp) {
-    if (!NL) return fmt_16bit(FMT) ? 2 : 4;
-    return (RING_BYTES - nt(btp) * tslot(btp)) / FSLOT_BYTES >= 8 ? 8 : 4;
+    return (RING_BYTES - RF - nt(btp) * tslot(btp)) / FSLOT_BYTES >= 8 ? 8 : 4;
   }
+  // the largest token tile: 448 on the codes; beside the low-rank buffers 256 (16-bit bases: 192)
+  static constexpr int MAX_TILE = NL ? 448 : fmt_16bit(FMT) ? 192 : MAX_TILE_L;
   __host__ __device__ static constexpr uint32_t smem(int btp) {
     return RF + nt(btp) * tslot(btp) + nf(btp) * FSLOT_BYTES + 1024u;
   }
-  static_assert(nt(448) >= (NL ? NUM_GROUPS : 3) && smem(448) + 1024 <= 232448 && smem(32) + 1024 <= 232448, "shared memory budget");
+  static_assert(nt(MAX_TILE) >= NUM_GROUPS && smem(MAX_TILE) <= RING_BYTES + 1024 && smem(32) <= RING_BYTES + 1024,
+                "shared memory budget");
 };
 
 constexpr uint32_t TMEM_COLS = 512;
-constexpr uint32_t COL_L = NACC * BNP;           // the 64-column low-rank buffer(s) after the accumulators
-static_assert(COL_L + NLB * BK <= TMEM_COLS, "TMEM budget");
+constexpr uint32_t COL_L = MAX_TILE_L;            // the 64-column low-rank buffers after the one accumulator
+static_assert(COL_L + NLB * BK <= TMEM_COLS && NACC * BNP <= TMEM_COLS, "TMEM budget");
 
 // leader: the stage's operands are in place, i.e. both token halves of the slot landed and both
 // CTAs' producers wrote their W_hat tiles (one barrier, so that the MMA thread tests one per stage)
@@ -163,7 +163,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   constexpr uint32_t OFF_RF = PR::OFF_RF, OFF_TSLOTS = PR::OFF_TSLOTS;
   constexpr bool PACKED = FMT == FMT_I4;
   constexpr uint32_t FSLOT_BYTES = PR::FSLOT_BYTES;
-  constexpr int STAGE_WARPS = NL ? GROUP_WARPS : NUM_PROD_WARPS;   // producer warps of one stage (per CTA)
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bars[NUM_BARS];
   __shared__ __align__(16) uint32_t sig_buf[8];   // [0, 4): source of the peer's signals, [4, 8): their target
@@ -173,22 +172,27 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   const uint32_t smem = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_cta_rank();
+  // A cluster holds `ksplit` pairs that share a tile: pair `slice` takes that part of the contraction
+  // (1: one pair per cluster, persistent over its tiles).  rank: this CTA's place in its pair.
+  const int ksplit = args.ksplit;
+  const uint32_t crank = cluster_cta_rank(), rank = crank & 1u, lead = crank & ~1u;
+  const int slice = static_cast<int>(crank >> 1);
   const bool leader = rank == 0;
-  const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+  const uint32_t pair_mask = 3u << lead;   // the pair's CTAs, for multicast commits
+  const int pair = blockIdx.x / (2 * ksplit), npairs = gridDim.x / (2 * ksplit);
   auto bar = [&](int i) { return smem_u32(&bars[i]); };
-  auto lbar = [&](int i) { return map_shared_rank(smem_u32(&bars[i]), 0); };   // the leader's copy
+  auto lbar = [&](int i) { return map_shared_rank(smem_u32(&bars[i]), lead); };   // the leader's copy
 
   // the token tile: one accumulator of bnp <= 256 tokens or two of bnp <= 224, half of each per CTA
   const int bnp = args.bnp, bnh = bnp / 2, nacc = args.nacc, btp = bnp * nacc;
   const int NT = PR::nt(btp), NF = PR::nf(btp);
   const uint32_t TSLOT_BYTES = PR::tslot(btp), TOK_BOX = 128u * bnh, TS_W = 64u * btp;
   const uint32_t OFF_FSLOTS = OFF_TSLOTS + NT * TSLOT_BYTES;
-  const uint32_t issuers = NL ? nacc : 1;   // threads that issue (and commit) the main product
+  const uint32_t issuers = nacc;   // threads that issue (and commit) the main product
   if (threadIdx.x == 0) {
     abort_s = 0;
     for (int s = 0; s < NT; ++s) {
-      mbar_init(bar(BAR_TFULL + s), 1 + STAGE_WARPS);   // the leader's token loader and producer warps
+      mbar_init(bar(BAR_TFULL + s), 1 + GROUP_WARPS);   // the leader's token loader and producer warps
       mbar_init(bar(BAR_TEMPTY + s), issuers);
     }
     for (int s = 0; s < NF; ++s) {
@@ -196,11 +200,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       mbar_init(bar(BAR_FFULL + s), 1);
       // freed by this CTA's producers after they built W_hat: by then they have waited for the
       // low-rank tile, so the low-rank MMA that read the slot's factor half has completed
-      mbar_init(bar(BAR_FEMPTY + s), STAGE_WARPS);
+      mbar_init(bar(BAR_FEMPTY + s), GROUP_WARPS);
     }
     for (int b = 0; b < NLB; ++b) {
       mbar_init(bar(BAR_LFULL + b), 1);
-      mbar_init(bar(BAR_LEMPTY + b), NUM_PROD_WARPS);
+      mbar_init(bar(BAR_LEMPTY + b), GROUP_WARPS);
     }
     mbar_init(bar(BAR_RFFULL), 1);
     mbar_init(bar(BAR_RFEMPTY), 1);
@@ -217,7 +221,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = tmem_base_s;
   const WaitCtl ctl{&abort_s, args.status, args.timeout_ns};
-  const int nk = args.kdim / BK;   // at least 2 (kdim is a multiple of 128)
+  // this pair's stages k0 .. k0 + nk - 1 (kdim is a multiple of 128, ksplit at most kdim / 64)
+  const int nk_all = args.kdim / BK, k0 = nk_all * slice / ksplit, nk = nk_all * (slice + 1) / ksplit - k0;
   const int num_rb2 = (args.num_rb + 1) / 2;   // 256-row blocks
   // This CTA's first row in row block rb2.  With an odd number of 128-row blocks the last pair's
   // CTA 1 has none: it takes part with zero-filled loads (and the last block's scales) and stores
@@ -228,7 +233,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   };
   const int num_tiles = num_rb2 * ((args.T + btp - 1) / btp);
   const uint32_t sig_src = smem_u32(&sig_buf[0]);
-  const uint32_t sig_dst_leader = map_shared_rank(smem_u32(&sig_buf[4]), 0);
+  const uint32_t sig_dst_leader = map_shared_rank(smem_u32(&sig_buf[4]), lead);
   // A producer warp's event on a leader barrier: the leader's warps arrive (warp 0 also
   // announces the peer's 16 signal bytes of each of the n warps), the peer's warps send their signal.
   auto report = [&](int b, int pw, int n) {
@@ -240,16 +245,16 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     }
   };
 
-  // The main product of the pair's tiles into accumulator 0 (and / or 1), by one thread of the leader.
-  // On the codes two threads issue one accumulator each: a thread's barrier test and commit (~110
+  // The main product of the pair's tiles into accumulator a, by one thread of the leader.  Two
+  // accumulators have a thread each: a thread's barrier test and commit (~110
   // and ~70 cycles a stage, with the tensor pipe queueing about one MMA ahead) then run beside the
   // other's MMAs (4096 x 4096, 288-token tiles 906 -> 739 cycles a stage, 320 925 -> 801; at 448 the
   // operands' shared-memory traffic sets the pace either way, 1101 -> 1106).
-  auto issue_main = [&](bool acc0, bool acc1, int drain) {
+  auto issue_main = [&](int a, int drain) {
     const uint32_t idesc_main = make_idesc_bf16(256, bnp, 0, 0);
-    const uint32_t TSLOT_D = TSLOT_BYTES >> 4, TOKB_D = TOK_BOX >> 4;
+    const uint32_t TSLOT_D = TSLOT_BYTES >> 4, d = tmem + a * BNP;
     const uint64_t d_w0 = make_sdesc(smem + OFF_TSLOTS + TS_W, 16, 1024, SWZ_128B);
-    const uint64_t d_tok0 = make_sdesc(smem + OFF_TSLOTS, 16, 1024, SWZ_128B);
+    const uint64_t d_tok = make_sdesc(smem + OFF_TSLOTS + a * TOK_BOX, 16, 1024, SWZ_128B);
     uint32_t it = 0;
     Cursor cur;
     bool ok = true;
@@ -263,25 +268,17 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         if (!(ok = wait_spin_bounded(bar(BAR_TFULL + s), cur.ph, ctl, 9))) break;
         cur.next(NT);
         tc_fence_after();
-        const uint64_t w = d_w0 + s * TSLOT_D, t = d_tok0 + s * TSLOT_D;
+        const uint64_t w = d_w0 + s * TSLOT_D, t = d_tok + s * TSLOT_D;
         const uint32_t acc = kk > 0 ? 1u : 0u;
-        static_assert(NACC == 2 && BK == 64, "issue sequence below: up to 2 accumulators x 4 K steps");
-        if (acc0) {
-          mma_bf16_pair(tmem, w, t, idesc_main, acc);
-          mma_bf16_pair(tmem, w + 2, t + 2, idesc_main, 1u);
-          mma_bf16_pair(tmem, w + 4, t + 4, idesc_main, 1u);
-          mma_bf16_pair(tmem, w + 6, t + 6, idesc_main, 1u);
-        }
-        if (acc1) {
-          mma_bf16_pair(tmem + BNP, w, t + TOKB_D, idesc_main, acc);
-          mma_bf16_pair(tmem + BNP, w + 2, t + TOKB_D + 2, idesc_main, 1u);
-          mma_bf16_pair(tmem + BNP, w + 4, t + TOKB_D + 4, idesc_main, 1u);
-          mma_bf16_pair(tmem + BNP, w + 6, t + TOKB_D + 6, idesc_main, 1u);
-        }
-        mma_commit_pair(bar(BAR_TEMPTY + s));
+        static_assert(BK == 64, "four K steps below");
+        mma_bf16_pair(d, w, t, idesc_main, acc);
+        mma_bf16_pair(d, w + 2, t + 2, idesc_main, 1u);
+        mma_bf16_pair(d, w + 4, t + 4, idesc_main, 1u);
+        mma_bf16_pair(d, w + 6, t + 6, idesc_main, 1u);
+        mma_commit_pair(bar(BAR_TEMPTY + s), pair_mask);
       }
       if (!ok) break;
-      mma_commit_pair(bar(BAR_ACCFULL));
+      mma_commit_pair(bar(BAR_ACCFULL), pair_mask);
       ++it;
     }
     // the peer's last drain report lands before the CTAs end
@@ -290,13 +287,29 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     drain_wait(bar(drain), 0, args.timeout_ns);
   };
 
+  // Epilogue: the factor of an output row, and 16 tokens of it scaled, masked and stored.
+  auto out_scale = [&](int row_g) {
+    float scale = 1.0f;
+    if (MODE == FUSED_FWD_PC) scale = args.s[row_g];
+    if (MODE != FUSED_DX && args.s_x != nullptr) scale *= *args.s_x;
+    return scale;
+  };
+  auto store_tokens = [&](float (&acc)[16], float scale, int row_g, int tok0) {
+    uint32_t mword = 0xffffffffu;
+    if (MODE == FUSED_DX && args.xmask != nullptr && tok0 < args.T)
+      mword = args.xmask[static_cast<int64_t>(row_g) * args.xmask_ld + tok0 / 32] >> (tok0 & 31);
+#pragma unroll
+    for (int e = 0; e < 16; ++e) acc[e] = ((mword >> e) & 1u) ? acc[e] * scale : 0.0f;
+    store_row_pairs_bf16(acc, lane & 1, args.out, args.out_ld, row_g, tok0, args.T);
+  };
+
   if (warp == 0) {
     // ------------------- row factor (per tile) and, in the leader, the low-rank MMAs
     // A thread of its own issues the low-rank tiles, so that the main product never waits
     // behind their barriers; each thread's commits track only its own MMAs.  On the codes it is the
     // second accumulator's issuer.
     if (NL) {
-      if (leader && lane == 0 && nacc == 2) issue_main(false, true, BAR_DRAIN_B);
+      if (leader && lane == 0 && nacc == 2) issue_main(1, BAR_DRAIN_B);
     } else if (lane == 0) {
       prefetch_tensormap(&tm_rf);
       const uint32_t idesc_l = make_idesc_bf16(256, BK, 0, 0);
@@ -326,10 +339,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             const uint64_t sf = d_sf0 + s * FSLOT_D;
             const uint32_t dl = tmem + COL_L + BK * b;
             for (int ks = 0; ks < lsteps; ++ks) mma_bf16_pair(dl, d_rf + 2 * ks, sf + 2 * ks, idesc_l, ks > 0 ? 1u : 0u);
-            mma_commit_pair(bar(BAR_LFULL + b));
+            mma_commit_pair(bar(BAR_LFULL + b), pair_mask);
           }
           if (!ok) break;
-          mma_commit_pair(bar(BAR_RFEMPTY));   // last read of the row factor issued
+          mma_commit_pair(bar(BAR_RFEMPTY), pair_mask);   // last read of the row factor issued
         }
         g += nk;
         ++it;
@@ -358,8 +371,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           if (!(ok = wait_spin_bounded(bar(BAR_TEMPTY + c.s), c.ph ^ 1u, ctl, 2))) break;
           if (leader) mbar_arrive_expect_tx(bar(BAR_TFULL + c.s), 128u * btp);
           const uint32_t st = smem + OFF_TSLOTS + c.s * TSLOT_BYTES, fb = lbar(BAR_TFULL + c.s);
-          tma_load_2d_pair(st, &tm_tok, kk * BK, tok, fb);
-          if (nacc == 2) tma_load_2d_pair(st + TOK_BOX, &tm_tok, kk * BK, tok + bnp, fb);
+          tma_load_2d_pair(st, &tm_tok, (k0 + kk) * BK, tok, fb);
+          if (nacc == 2) tma_load_2d_pair(st + TOK_BOX, &tm_tok, (k0 + kk) * BK, tok + bnp, fb);
           c.skip(NL4, NT);
         }
         kk -= nk;
@@ -376,7 +389,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       bool any = false, ok = true;
       for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
         const int rb2 = tile % num_rb2;
-        for (int kk = 0; kk < nk; ++kk) {
+        for (int kk = k0; kk < k0 + nk; ++kk) {
           const uint32_t s = f.s;
           if (!(ok = wait_spin_bounded(bar(BAR_FEMPTY + s), f.ph ^ 1u, ctl, 3))) break;
           any = true;
@@ -415,7 +428,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------ main-product MMA issuer (the leader's)
-    if (leader && lane == 0) issue_main(true, !NL && nacc == 2, BAR_DRAIN);
+    if (leader && lane == 0) issue_main(0, BAR_DRAIN);
   } else {
     // ------------------------------------------- W_hat producers + epilogue
     const int pw = warp - 2;              // 0..15
@@ -428,42 +441,44 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     uint32_t g = 0;
     uint32_t it = 0;
     Cursor fc, tc;   // factor and token slots
-    if (NL) {
-      fc.skip(c, NF);
-      tc.skip(c, NT);
-    }
+    fc.skip(c, NF);
+    tc.skip(c, NT);
     bool ok = true;
     for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
       const int rb2 = tile % num_rb2;
       const int tb = tile / num_rb2;
       const int row_g = row_block(rb2) + row;
       const bool has_rows = rb2 * 2 * BM + static_cast<int>(rank) * BM < args.rows;
-      if constexpr (NL) {
-        // Group c's stages of the tile (gg % 4 == c).  A ready barrier costs a test of ~110 cycles and
-        // the proxy fence and reports ~100 more, whatever the warp does between them: with all sixteen
-        // warps in every stage these made a stage 770 cycles (4096 x 4096, 32-token tiles), four
-        // groups in flight pay them side by side (596 cycles; 256-token tiles 863 -> 700).
-        for (int kk = static_cast<int>((static_cast<uint32_t>(c) - g) & 3u); kk < nk; kk += NUM_GROUPS) {
-          ok = wait_bounded(bar(BAR_PFULL + fc.s), fc.ph, ctl, 12);
-          if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-          const uint32_t fs = smem + OFF_FSLOTS + fc.s * FSLOT_BYTES;
-          uint4 raw[4];
+      // Group c's stages of the tile (gg % 4 == c).  A ready barrier costs a test of ~110 cycles and the
+      // proxy fence and reports ~100 more, whatever the warp does between them: with all sixteen warps in
+      // every stage these made a stage on the codes 770 cycles (4096 x 4096, 32-token tiles), four groups
+      // in flight pay them side by side (596 cycles; 256-token tiles 863 -> 700).  With the low-rank tile
+      // a group has a TMEM buffer of its own, so four low-rank tiles are in flight instead of one
+      // (1700 -> 1030 cycles a stage; T = 1024 forward 58 -> 45 us).
+      for (int kk = static_cast<int>((static_cast<uint32_t>(c) - g) & 3u); kk < nk; kk += NUM_GROUPS) {
+        ok = wait_bounded(bar(BAR_PFULL + fc.s), fc.ph, ctl, 12);
+        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+        const uint32_t fs = smem + OFF_FSLOTS + fc.s * FSLOT_BYTES;
+        constexpr int RAW4 = PACKED ? 2 : fmt_16bit(FMT) ? 8 : 4;   // 16-byte words of the row's 64 values
+        constexpr int ROW_BYTES = 16 * RAW4;
+        uint4 raw[RAW4];
 #pragma unroll
-          for (int x = 0; x < 4; ++x) raw[x] = ld_shared_v4(fs + swz_offset(row, x, 64));
-          uint32_t sg = 0, zg = 0;   // forward: the row's scale and zero offset in the stage, as bf16x2
-          if (MODE == FUSED_FWD_GROUP) {
-            sg = ld_shared_u16(fs + PR::FS_X + 2u * row);
-            sg |= sg << 16;
-            if (ZP) {
-              zg = ld_shared_u16(fs + PR::FS_X + 512u + 2u * row);
-              zg |= zg << 16;
-            }
-          } else if (MODE == FUSED_FWD_PC && ZP) {
-            zg = pack_rn_bf16x2(args.zero[row_g], args.zero[row_g]);
+        for (int x = 0; x < RAW4; ++x) raw[x] = ld_shared_v4(fs + swz_offset(row, x, ROW_BYTES));
+        uint32_t sg = 0, zg = 0;   // forward: the row's scale and zero offset in the stage, as bf16x2
+        if (MODE == FUSED_FWD_GROUP) {
+          sg = ld_shared_u16(fs + PR::FS_X + 2u * row);
+          sg |= sg << 16;
+          if (ZP) {
+            zg = ld_shared_u16(fs + PR::FS_X + 512u + 2u * row);
+            zg |= zg << 16;
           }
-          uint32_t w[32];
+        } else if (MODE == FUSED_FWD_PC && ZP) {
+          zg = pack_rn_bf16x2(args.zero[row_g], args.zero[row_g]);
+        }
+        uint32_t w[32];
+        if (NL) {
 #pragma unroll
-          for (int x = 0; x < 4; ++x) {
+          for (int x = 0; x < RAW4; ++x) {
             const uint32_t in[4] = {raw[x].x, raw[x].y, raw[x].z, raw[x].w};
             if (args.codes_bias == 64) {
 #pragma unroll
@@ -475,152 +490,98 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
               for (int e = 0; e < 8; ++e) w[8 * x + e] = pack_int_bf16x2(v[2 * e], v[2 * e + 1]);
             }
           }
-#pragma unroll
-          for (int x = 0; x < 8; ++x) {
-            if (MODE == FUSED_DX) {
-              // the bf16 scales (zero offsets) of eight contraction indices, as bf16x2 words
-              const uint4 s4 = ld_shared_v4(fs + PR::FS_X + 16u * x);
-              if (ZP) {
-                const uint4 z4 = ld_shared_v4(fs + PR::FS_X + 512u + 16u * x);
-                w[4 * x] = sub_bf16x2(w[4 * x], z4.x), w[4 * x + 1] = sub_bf16x2(w[4 * x + 1], z4.y);
-                w[4 * x + 2] = sub_bf16x2(w[4 * x + 2], z4.z), w[4 * x + 3] = sub_bf16x2(w[4 * x + 3], z4.w);
-              }
-              w[4 * x] = mul_bf16x2(w[4 * x], s4.x), w[4 * x + 1] = mul_bf16x2(w[4 * x + 1], s4.y);
-              w[4 * x + 2] = mul_bf16x2(w[4 * x + 2], s4.z), w[4 * x + 3] = mul_bf16x2(w[4 * x + 3], s4.w);
-            } else {
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                if (ZP) w[4 * x + e] = sub_bf16x2(w[4 * x + e], zg);
-                if (MODE == FUSED_FWD_GROUP) w[4 * x + e] = mul_bf16x2(w[4 * x + e], sg);
-              }
-            }
-          }
-          // the slot's W_hat buffer was last read by the product of the stage NT before
-          ok = wait_bounded(bar(BAR_TEMPTY + tc.s), tc.ph ^ 1u, ctl, 14);
-          if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-          const uint32_t wt = smem + OFF_TSLOTS + tc.s * TSLOT_BYTES + TS_W;
-#pragma unroll
-          for (int x = 0; x < 8; ++x)
-            st_shared_v4(wt + swz_offset(row, x, 128), w[4 * x], w[4 * x + 1], w[4 * x + 2], w[4 * x + 3]);
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) {
-            report(BAR_TFULL + tc.s, q, GROUP_WARPS);
-            mbar_arrive(bar(BAR_FEMPTY + fc.s));
-          }
-          fc.skip(NUM_GROUPS, NF);
-          tc.skip(NUM_GROUPS, NT);
-        }
-      } else {
-        for (int kk = 0; kk < nk; ++kk) {
-          uint32_t scw[8];   // dX: the stage's 16 bf16 scales of its contraction indices, as bf16x2
-          uint32_t zw[8];    // zero offsets as bf16x2
-          uint32_t sgw = 0;  // group-wise forward: the stage's scale as bf16x2
-          if (ZP && MODE == FUSED_FWD_PC) {
-            // per-channel forward: this row's zero offset (dX and the group-wise forward read theirs
-            // from the factor slot below)
-            const uint32_t z2 = pack_rn_bf16x2(args.zero[row_g], args.zero[row_g]);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) zw[e] = z2;
-          }
-          // the stage's stored base, read as soon as it has landed
-          uint32_t raw[8];
-          ok = wait_bounded(bar(BAR_PFULL + fc.s), fc.ph, ctl, 12);
-          if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-          const uint32_t fs = smem + OFF_FSLOTS + fc.s * FSLOT_BYTES;
-          if (PACKED) {
-            const uint2 r = ld_shared_v2(fs + swz_offset(row, c >> 1, 32) + 8 * (c & 1));
-            raw[0] = r.x;
-            raw[1] = r.y;
-          } else if (fmt_16bit(FMT)) {
-            const uint4 r0 = ld_shared_v4(fs + swz_offset(row, 2 * c, 128));
-            const uint4 r1 = ld_shared_v4(fs + swz_offset(row, 2 * c + 1, 128));
-            raw[0] = r0.x, raw[1] = r0.y, raw[2] = r0.z, raw[3] = r0.w;
-            raw[4] = r1.x, raw[5] = r1.y, raw[6] = r1.z, raw[7] = r1.w;
-          } else {
-            const uint4 r = ld_shared_v4(fs + swz_offset(row, c, 64));
-            raw[0] = r.x, raw[1] = r.y, raw[2] = r.z, raw[3] = r.w;
-          }
-          if (MODE == FUSED_DX) {
-            // the 16 bf16 scales (zero offsets) of this warp's contraction indices, as bf16x2 words
-            const uint4 s0 = ld_shared_v4(fs + PR::FS_X + 32u * c), s1 = ld_shared_v4(fs + PR::FS_X + 32u * c + 16u);
-            scw[0] = s0.x, scw[1] = s0.y, scw[2] = s0.z, scw[3] = s0.w;
-            scw[4] = s1.x, scw[5] = s1.y, scw[6] = s1.z, scw[7] = s1.w;
-            if (ZP) {
-              const uint4 z0 = ld_shared_v4(fs + PR::FS_X + 512u + 32u * c);
-              const uint4 z1 = ld_shared_v4(fs + PR::FS_X + 512u + 32u * c + 16u);
-              zw[0] = z0.x, zw[1] = z0.y, zw[2] = z0.z, zw[3] = z0.w;
-              zw[4] = z1.x, zw[5] = z1.y, zw[6] = z1.z, zw[7] = z1.w;
-            }
-          } else if (MODE == FUSED_FWD_GROUP) {
-            // this thread's row's scale (and zero offset) in the stage's group, as bf16x2
-            const uint32_t sv = ld_shared_u16(fs + PR::FS_X + 2u * row);
-            sgw = sv | (sv << 16);
-            if (ZP) {
-              const uint32_t zv = ld_shared_u16(fs + PR::FS_X + 512u + 2u * row);
-#pragma unroll
-              for (int e = 0; e < 8; ++e) zw[e] = zv | (zv << 16);
-            }
-          }
-          float v[16], Lv[16];
-          decode16<FMT>(raw, v);
-          const uint32_t lb = (g + kk) % NLB;
-          ok = wait_bounded(bar(BAR_LFULL + lb), ((g + kk) / NLB) & 1u, ctl, 13);
+        } else {
+          // the group's low-rank buffer (gg % NLB == c, used every fourth stage)
+          ok = wait_bounded(bar(BAR_LFULL + c), ((g + kk) / NLB) & 1u, ctl, 13);
           if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
           tc_fence_after();
-          tmem_ld16(tmem + lane_off + COL_L + BK * lb + 16 * c, Lv);
-          tmem_ld_wait();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) report(BAR_LEMPTY + lb, pw, NUM_PROD_WARPS);
-          uint32_t w[8];
+          const uint32_t* rw = reinterpret_cast<const uint32_t*>(raw);
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const float2 u = UB ? u_bf16x2(Lv[2 * e], Lv[2 * e + 1], v[2 * e], v[2 * e + 1], lr2)
-                                : __ffma2_rn(make_float2(Lv[2 * e], Lv[2 * e + 1]),
-                                             make_float2(qp.lr_scale, qp.lr_scale),
-                                             make_float2(v[2 * e], v[2 * e + 1]));
-            uint32_t cw = codes_bf16x2(__fadd2_rn(u, make_float2(qp.magic, qp.magic)), qp);
-            if (ZP) cw = sub_bf16x2(cw, zw[e]);
-            w[e] = MODE == FUSED_FWD_PC ? cw : mul_bf16x2(cw, MODE == FUSED_DX ? scw[e] : sgw);
+          for (int x = 0; x < 4; ++x) {
+            float v[16], Lv[16];
+            tmem_ld16(tmem + lane_off + COL_L + BK * c + 16 * x, Lv);
+            uint32_t in[RAW4];
+#pragma unroll
+            for (int e = 0; e < RAW4; ++e) in[e] = rw[RAW4 * x + e];
+            decode16<FMT>(in, v);
+            tmem_ld_wait();
+            if (x == 3) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) report(BAR_LEMPTY + c, q, GROUP_WARPS);
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              const float2 u = UB ? u_bf16x2(Lv[2 * e], Lv[2 * e + 1], v[2 * e], v[2 * e + 1], lr2)
+                                  : __ffma2_rn(make_float2(Lv[2 * e], Lv[2 * e + 1]),
+                                               make_float2(qp.lr_scale, qp.lr_scale),
+                                               make_float2(v[2 * e], v[2 * e + 1]));
+              w[8 * x + e] = codes_bf16x2(__fadd2_rn(u, make_float2(qp.magic, qp.magic)), qp);
+            }
           }
-          // the W_hat buffer (in the token slot) was last read by the product of the stage NT before
-          ok = wait_bounded(bar(BAR_TEMPTY + tc.s), tc.ph ^ 1u, ctl, 14);
-          if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-          const uint32_t wt = smem + OFF_TSLOTS + tc.s * TSLOT_BYTES + TS_W;
-          st_shared_v4(wt + swz_offset(row, 2 * c, 128), w[0], w[1], w[2], w[3]);
-          st_shared_v4(wt + swz_offset(row, 2 * c + 1, 128), w[4], w[5], w[6], w[7]);
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) {
-            report(BAR_TFULL + tc.s, pw, NUM_PROD_WARPS);
-            mbar_arrive(bar(BAR_FEMPTY + fc.s));
-          }
-          fc.next(NF);
-          tc.next(NT);
         }
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+          if (MODE == FUSED_DX) {
+            // the bf16 scales (zero offsets) of eight contraction indices, as bf16x2 words
+            const uint4 s4 = ld_shared_v4(fs + PR::FS_X + 16u * x);
+            if (ZP) {
+              const uint4 z4 = ld_shared_v4(fs + PR::FS_X + 512u + 16u * x);
+              w[4 * x] = sub_bf16x2(w[4 * x], z4.x), w[4 * x + 1] = sub_bf16x2(w[4 * x + 1], z4.y);
+              w[4 * x + 2] = sub_bf16x2(w[4 * x + 2], z4.z), w[4 * x + 3] = sub_bf16x2(w[4 * x + 3], z4.w);
+            }
+            w[4 * x] = mul_bf16x2(w[4 * x], s4.x), w[4 * x + 1] = mul_bf16x2(w[4 * x + 1], s4.y);
+            w[4 * x + 2] = mul_bf16x2(w[4 * x + 2], s4.z), w[4 * x + 3] = mul_bf16x2(w[4 * x + 3], s4.w);
+          } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              if (ZP) w[4 * x + e] = sub_bf16x2(w[4 * x + e], zg);
+              if (MODE == FUSED_FWD_GROUP) w[4 * x + e] = mul_bf16x2(w[4 * x + e], sg);
+            }
+          }
+        }
+        // the slot's W_hat buffer was last read by the product of the stage NT before
+        ok = wait_bounded(bar(BAR_TEMPTY + tc.s), tc.ph ^ 1u, ctl, 14);
+        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+        const uint32_t wt = smem + OFF_TSLOTS + tc.s * TSLOT_BYTES + TS_W;
+#pragma unroll
+        for (int x = 0; x < 8; ++x)
+          st_shared_v4(wt + swz_offset(row, x, 128), w[4 * x], w[4 * x + 1], w[4 * x + 2], w[4 * x + 3]);
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          report(BAR_TFULL + tc.s, q, GROUP_WARPS);
+          mbar_arrive(bar(BAR_FEMPTY + fc.s));
+        }
+        fc.skip(NUM_GROUPS, NF);
+        tc.skip(NUM_GROUPS, NT);
       }
       if (!ok) break;
       // ------------------------------------------------------------ epilogue
-      float scale = 1.0f;
-      if (MODE == FUSED_FWD_PC) scale = args.s[row_g];
-      if (MODE != FUSED_DX && args.s_x != nullptr) scale *= *args.s_x;
       ok = wait_spin_bounded(bar(BAR_ACCFULL), it & 1u, ctl, 15);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       tc_fence_after();
-      const bool odd = lane & 1;
+      if (ksplit == 1) {
+        const float scale = out_scale(row_g);
 #pragma unroll 1
-      for (int col = has_rows ? 16 * c : btp; col < btp; col += 64) {   // token offset in the tile
-        float acc[16];
-        tmem_ld16(tmem + lane_off + (col < bnp ? col : BNP + col - bnp), acc);
-        tmem_ld_wait();
-        const int tok0 = tb * btp + col;
-        uint32_t mword = 0xffffffffu;
-        if (MODE == FUSED_DX && args.xmask != nullptr && tok0 < args.T)
-          mword = args.xmask[static_cast<int64_t>(row_g) * args.xmask_ld + tok0 / 32] >> (tok0 & 31);
+        for (int col = has_rows ? 16 * c : btp; col < btp; col += 64) {   // token offset in the tile
+          float acc[16];
+          tmem_ld16(tmem + lane_off + (col < bnp ? col : BNP + col - bnp), acc);
+          tmem_ld_wait();
+          store_tokens(acc, scale, row_g, tb * btp + col);
+        }
+      } else {
+        // the other slices' token columns of this CTA's partial sums go to its ring (idle: the tile's
+        // copies, W_hat tiles and products are all done), [token][row]
+#pragma unroll 1
+        for (int col = 16 * c; col < btp; col += 64) {
+          if (col / (btp / ksplit) == slice) continue;
+          float acc[16];
+          tmem_ld16(tmem + lane_off + col, acc);
+          tmem_ld_wait();
 #pragma unroll
-        for (int e = 0; e < 16; ++e) acc[e] = ((mword >> e) & 1u) ? acc[e] * scale : 0.0f;
-        store_row_pairs_bf16(acc, odd, args.out, args.out_ld, row_g, tok0, args.T);
+          for (int e = 0; e < 16; ++e) st_shared_f32(smem + ((col + e) * BM + row) * 4u, acc[e]);
+        }
       }
       tc_fence_before();
       __syncwarp();
@@ -630,6 +591,34 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     }
   }
 
+  if (ksplit > 1) {
+    // One tile per cluster: its pairs' partial sums meet.  Pair p owns the p-th part of the tile's
+    // tokens and adds the slices' sums in order through distributed shared memory.
+    __syncwarp();
+    cluster_sync_all();
+    if (warp >= 2 && warp < FIRST_TMA_WARP && pair < num_tiles && !abort_s) {
+      tc_fence_after();
+      const int q = warp & 3, c = (warp - 2) >> 2, row = q * 32 + lane;
+      const int rb2 = pair % num_rb2, tb = pair / num_rb2, own = btp / ksplit;
+      const int row_g = row_block(rb2) + row;
+      const bool has_rows = rb2 * 2 * BM + static_cast<int>(rank) * BM < args.rows;
+      const float scale = out_scale(row_g);
+#pragma unroll 1
+      for (int col = slice * own + 16 * c; col < (slice + 1) * own; col += 64) {
+        float mine[16], acc[16];
+        tmem_ld16(tmem + (static_cast<uint32_t>(q * 32) << 16) + col, mine);
+        tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < 16; ++e) acc[e] = 0.0f;
+        for (int p = 0; p < ksplit; ++p) {
+          const uint32_t src = map_shared_rank(smem + (col * BM + row) * 4u, 2u * p + rank);
+#pragma unroll
+          for (int e = 0; e < 16; ++e) acc[e] += p == slice ? mine[e] : ld_cluster_f32(src + e * BM * 4u);
+        }
+        if (has_rows) store_tokens(acc, scale, row_g, tb * btp + col);
+      }
+    }
+  }
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();   // neither CTA leaves while the other may still read its shared memory
@@ -644,24 +633,29 @@ template <int MODE, int FMT, bool ZP, bool UB, bool NL>
 cudaError_t launch_pair_one(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c, const CUtensorMap& d,
                             const FusedArgs& args, int npairs, cudaStream_t stream) {
   using PR = PairRing<FMT, NL, MODE == FUSED_DX || MODE == FUSED_FWD_GROUP>;
-  if (!NL && args.bnp * args.nacc > 448) return cudaErrorInvalidValue;
+  if (args.bnp * args.nacc > PR::MAX_TILE || (!NL && args.nacc != 1)) return cudaErrorInvalidValue;
+  if (args.ksplit > 1 && (args.nacc != 1 || args.bnp % (16 * args.ksplit))) return cudaErrorInvalidValue;
   const uint32_t smem = PR::smem(args.bnp * args.nacc);
   static bool configured[kMaxDevices] = {};
   const void* fn = reinterpret_cast<const void*>(fused_pair_kernel<MODE, FMT, ZP, UB, NL>);
   cudaError_t e = ensure_smem_attr(fn, 232448 - 1024, configured);   // the most any tile asks for
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(static_cast<unsigned>(2 * npairs), 1, 1);
+  cfg.gridDim = dim3(static_cast<unsigned>(2 * args.ksplit * npairs), 1, 1);
   cfg.blockDim = dim3(NUM_THREADS, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(2 * args.ksplit);
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  if (args.ksplit > 1) {   // one tile per cluster, however many are resident at once
+    e = cudaLaunchKernelEx(&cfg, fused_pair_kernel<MODE, FMT, ZP, UB, NL>, a, b, c, d, args);
+    return e != cudaSuccess ? e : cudaGetLastError();
+  }
   // The persistent grid holds no more pairs than can be resident at once (an SM that has no
   // partner in its GPC cannot host half of a pair), looked up once per device.
   static int max_pairs[kMaxDevices] = {};
@@ -722,12 +716,42 @@ cudaError_t launch_pair_mode(int fmt, const CUtensorMap& a, const CUtensorMap& b
 
 }  // namespace
 
+int fused_pair_max_clusters(int ksplit) {
+  static std::atomic<int> cache[kMaxDevices][5];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices || ksplit < 1 || ksplit > 4) return 0;
+  int n = cache[dev][ksplit].load(std::memory_order_acquire);
+  if (n > 0) return n;
+  using PR = PairRing<FMT_Q8, true, false>;
+  static bool configured[kMaxDevices] = {};
+  const void* fn = reinterpret_cast<const void*>(fused_pair_kernel<FUSED_FWD_PC, FMT_Q8, false, false, true>);
+  if (ensure_smem_attr(fn, 232448 - 1024, configured) != cudaSuccess) return 0;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(2 * ksplit), 1, 1);
+  cfg.blockDim = dim3(NUM_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = PR::smem(256);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(2 * ksplit);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaOccupancyMaxActiveClusters(&n, fused_pair_kernel<FUSED_FWD_PC, FMT_Q8, false, false, true>, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  cache[dev][ksplit].store(n, std::memory_order_release);
+  return n;
+}
+
 cudaError_t launch_fused_pair(int mode, int fmt, const CUtensorMap& tm_tok, const CUtensorMap& tm_phi,
                               const CUtensorMap& tm_rf, const CUtensorMap& tm_sf, const FusedArgs& args, int npairs,
                               cudaStream_t stream) {
   if (npairs < 1 || (args.kdim % 128) != 0 || args.kdim < 128 || (args.rows % BM) != 0 || args.sf_mn ||
       args.num_rb != args.rows / 128 || args.bnp < 16 || (args.bnp & 15) ||
-      !(args.nacc == 1 ? args.bnp <= 256 : args.nacc == 2 && args.bnp <= BNP))
+      !(args.nacc == 1 ? args.bnp <= 256 : args.nacc == 2 && args.bnp <= BNP) || args.ksplit < 1 || args.ksplit > 4 ||
+      args.ksplit > args.kdim / BK)
     return cudaErrorInvalidValue;
   switch (mode) {
     case FUSED_FWD_PC: return launch_pair_mode<FUSED_FWD_PC>(fmt, tm_tok, tm_phi, tm_rf, tm_sf, args, npairs, stream);

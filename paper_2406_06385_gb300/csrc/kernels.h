@@ -175,6 +175,9 @@ struct FusedArgs {
   // Pair kernel: the token tile, nacc accumulators of bnp tokens (a multiple of 16; nacc 1: up to
   // 256, 2: up to 224)
   int32_t bnp, nacc;
+  // Pair kernel: pairs that share a tile, each with a part of the contraction (1, 2 or 4; above 1 with
+  // one accumulator, bnp a multiple of 16 ksplit, and a cluster per tile)
+  int32_t ksplit;
 };
 // s_out[g][i] = bf16(s[i][g]) (s [m] per channel: g = 0 only) and, with z, z_out likewise: the
 // dX GEMM's producers read 16 consecutive of them per stage with two 16-byte loads.
@@ -182,15 +185,37 @@ cudaError_t launch_dx_scales(const float* s, const float* z, int64_t m, int grou
                              uint16_t* z_out, cudaStream_t stream);
 int fused_smem_bytes(int fmt);
 // The same GEMM on CTA pairs (fused_pair.cu): tiles of 256 rows x nacc * bnp tokens, npairs
-// clusters of 2.  Needs rows % 128 == 0 and K-major factor slices (sf_mn == 0); tm_tok boxes of
+// clusters of 2 ksplit CTAs (ksplit > 1: npairs is the number of tiles).  Needs rows % 128 == 0 and K-major factor slices (sf_mn == 0); tm_tok boxes of
 // bnp / 2 tokens x 64, tm_sf boxes of 32 slice rows x sf_cols; tm_phi and tm_rf as for launch_fused.
 cudaError_t launch_fused_pair(int mode, int fmt, const CUtensorMap& tm_tok, const CUtensorMap& tm_phi,
                               const CUtensorMap& tm_rf, const CUtensorMap& tm_sf, const FusedArgs& args, int npairs,
                               cudaStream_t stream);
+// Clusters of 2 ksplit CTAs of the pair GEMM that can be resident at once on the current device (0
+// when the query fails).
+int fused_pair_max_clusters(int ksplit);
 // fmt: a PhiFmt value (quant.cuh); FMT_I4 only for the forward modes
 cudaError_t launch_fused(int mode, int fmt, const CUtensorMap& tm_tok, const CUtensorMap& tm_phi,
                          const CUtensorMap& tm_rf, const CUtensorMap& tm_sf, const FusedArgs& args, int grid,
                          cudaStream_t stream);
+
+// ---- fused_few.cu ------------------------------------------------------------
+constexpr int kFewTokens = 16;   // most tokens of the few-token forward
+struct FewArgs {
+  int64_t m, k;
+  int32_t T, r16;         // r16 <= 64
+  QuantParams q;
+  const uint16_t* X;      // token operand [T, k] (bf16 activations or quantized codes)
+  const void* phi;        // the stored base
+  const uint16_t* a_pad;  // A [m][64] and B^T [k][64], zero-padded (launch_adapter_layouts)
+  const uint16_t* bt_pad;
+  const float* s;         // [m] or [m, s_ld]
+  const float* zero;      // zero offsets shaped like s, or nullptr
+  int32_t s_ld, group_size;
+  const float* s_x;       // activation scale (device scalar) or nullptr
+  int32_t u_bf16;
+  uint16_t* Y;            // [T, m]
+};
+cudaError_t launch_fused_few(int fmt, const FewArgs& a, cudaStream_t stream);
 
 // ---- dw.cu -------------------------------------------------------------------
 struct DwArgs {

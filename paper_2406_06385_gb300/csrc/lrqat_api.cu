@@ -128,14 +128,13 @@ int frac_bits(const lrqat_layer& L) { return L.phi_format == LRQAT_PHI_QFIXED ? 
 // 1 = the tile that each GEMM stage computes next to the main product (ranks up to 64);
 // 2 = the codes pass: one tensor-core pass per call writes the code of every weight as a byte into
 // the workspace, and the GEMMs read those as their base with the low-rank term switched off.
-// 0 (auto) = the codes wherever the workspace holds them (all but the allocation-free forward): the
-// in-stage tile is a chain of small MMAs whose TMEM buffer holds one stage, so it makes a stage ~1700
-// cycles against 550-1100 on the codes, and the pass itself takes 3 us on a 256 x 256 layer and 11
-// on 4096 x 4096.  Measured fwd / bwd per call, tile against codes: 256 x 256 at T = 64 12.3 / 31.4 us,
-// 11.0 / 24.3; 4096 x 4096 at T = 64 57.6 / 114 us, 32.8 / 74.0, at T = 2999 111 / 226 us, 70.0 / 161;
-// 11008 x 4096 at T = 448 58.6 / 302 us, 59.6 / 211.  Ranks above 64 take the codes in every setting:
-// their factor slices do not fit next to the GEMMs' token ring, and recomputing A B per token tile
-// would cost r / 448 of the GEMM's own tensor work.
+// 0 (auto) = the codes in every backward (the transposed base and the weight gradient's codes come from
+// the same pass) and in the forward where its cost model says so (prefer_codes_fwd).  Measured fwd / bwd
+// per call, in-stage tile against codes, with one low-rank buffer per pair: 256 x 256 at T = 64 12.3 /
+// 31.4 us, 11.0 / 24.3; 4096 x 4096 at T = 64 57.6 / 114 us, 32.8 / 74.0, at T = 2999 111 / 226 us,
+// 70.0 / 161.  Ranks above 64 take the codes in every setting: their factor slices do not fit next to
+// the GEMMs' token ring, and recomputing A B per token tile would cost r / 448 of the GEMM's own
+// tensor work.
 int lowrank_path_from_env() {
   const char* v = std::getenv("LRQAT_LOWRANK_PATH");
   if (v && std::strcmp(v, "tile") == 0) return 1;
@@ -143,9 +142,7 @@ int lowrank_path_from_env() {
   return 0;
 }
 std::atomic<int> g_lowrank_path{lowrank_path_from_env()};
-bool codes_gemm(const lrqat_layer& L) {
-  return L.r > 64 || g_lowrank_path.load(std::memory_order_relaxed) != 1;
-}
+bool codes_bwd(const lrqat_layer& L) { return L.r > 64 || g_lowrank_path.load(std::memory_order_relaxed) != 1; }
 bool phi_16bit(const lrqat_layer& L) { return L.phi_format == LRQAT_PHI_BF16 || L.phi_format == LRQAT_PHI_FP16; }
 int round16(int r) { return (r + 15) / 16 * 16; }
 
@@ -301,10 +298,9 @@ int dw_schedule_from_env() {
 std::atomic<int> g_dw_schedule{dw_schedule_from_env()};
 
 // Kernel of the forward and dX GEMMs (lrqat_set_gemm_variant): 0 = CTA pairs (fused_pair.cu)
-// wherever they were measured faster, which is every GEMM on the codes (an odd number of 128-row blocks
-// leaves half a pair without rows in the last one; 1664 x 13184 at T = 512, both odd, forward + backward
-// 415 us on one SM, 246 on pairs), and with the in-stage tile those without such a half (1408 x 896 at
-// T = 3: 19.3 us on one SM, which reads the factors themselves, 24.6 on pairs); 1 = the one-SM kernel (fused_gemm.cu)
+// wherever they were measured faster, which is every GEMM (an odd number of 128-row blocks leaves half
+// a pair without rows in the last one; 1664 x 13184 at T = 512, both odd, forward + backward 415 us on
+// one SM, 246 on pairs), but for a few tokens (fused_few.cu); 1 = the one-SM kernel (fused_gemm.cu)
 // always; 2 = pairs always.  LRQAT_GEMM_VARIANT ("auto" / "single" / "pair") sets the start value
 // once, when the library is loaded.
 int gemm_variant_from_env() {
@@ -314,42 +310,61 @@ int gemm_variant_from_env() {
   return 0;
 }
 std::atomic<int> g_gemm_variant{gemm_variant_from_env()};
-bool use_pair(int64_t rows, bool codes) {
-  const int v = g_gemm_variant.load(std::memory_order_relaxed);
-  return v == 2 || (v == 0 && (codes || rows % 256 == 0));
-}
-// The pair GEMM's token tile: nacc accumulators of bnp tokens.
-struct TokenTile {
-  int bnp, nacc;
+bool use_pair() { return g_gemm_variant.load(std::memory_order_relaxed) != 1; }
+// The pair GEMM's tile: nacc accumulators of bnp tokens, its contraction shared by ksplit pairs.
+struct PairTile {
+  int bnp, nacc, ksplit;
+  int64_t cost;   // cycles by the model below
   int tokens() const { return bnp * nacc; }
 };
 // The cheapest tile for `rows` weight rows, a contraction of kdim and T tokens on `pairs` pairs, by
-// the rounds of the busiest pair times a tile's cycles: kdim / 64 stages plus the drain.  Stage
+// the rounds of the busiest pair times a tile's cycles: its 64-wide stages plus the drain.  Stage
 // cycles measured on a 4096 x 4096 layer on the codes (forward, T = 8192, drain taken off): one
 // accumulator 524 (32 tokens) to 605 (256), two 655 (288) to 997 (448), linear in between; dX, whose
-// producers also multiply by the scales, 557 to 692 and 749 to 1042; the drain 2500 + 10 per token.  Up to 256 tokens the stage is bound by the issue of four MMAs whatever their
-// N, beyond by the operands' shared-memory traffic, so 448 tokens are the cheapest per token
-// (2.2 cycles a stage against 2.4 at 256) and smaller tiles pay where 448 leave pairs idle:
-// T = 4096 takes 304 (three rounds; forward 107 -> 82 us, dX 111 -> 92), T = 1024 takes 256.
-// With the low-rank tile in the stage a stage takes ~1700 cycles whatever the tile (one low-rank
-// buffer paces it), so that path keeps 448.
-TokenTile pair_token_tile(int64_t rows, int64_t kdim, int64_t T, int pairs, bool codes, bool dx) {
-  TokenTile best{224, 2};
-  if (!codes) return best;
+// producers also multiply by the scales, 557 to 692 and 749 to 1042; the drain 2500 + 10 per token.
+// Up to 256 tokens the stage is bound by the issue of four MMAs whatever their N, beyond by the
+// operands' shared-memory traffic, so 448 tokens are the cheapest per token (2.2 cycles a stage
+// against 2.4 at 256) and smaller tiles pay where 448 leave pairs idle: T = 4096 takes 304 (three
+// rounds; forward 107 -> 82 us, dX 111 -> 92), T = 1024 takes 256.  Where even one round leaves pairs
+// idle, two or four pairs share a tile's contraction and add their sums through distributed shared
+// memory (T = 256, forward 26.6 us with one pair, 22.8 with two; dX 29.1, 22.6).  With the low-rank tile in the stage (one accumulator: its buffers
+// take the other's TMEM) a stage takes 971 to 1050 cycles.
+PairTile pair_tile(int64_t rows, int64_t kdim, int64_t T, int pairs, bool codes, bool dx, bool phi16) {
+  PairTile best{0, 0, 1, 0};
   int64_t best_cost = -1;
-  for (int bt = 448; bt >= 32; bt -= 32) {
-    const int64_t tiles = ((rows + 255) / 256) * ((T + bt - 1) / bt);
-    const int64_t rounds = (tiles + pairs - 1) / pairs;
-    const int64_t stage = bt <= 256 ? (dx ? 538 + bt * 60 / 100 : 513 + bt * 36 / 100)
-                                    : (dx ? 749 + (bt - 288) * 183 / 100 : 655 + (bt - 288) * 214 / 100);
-    const int64_t cost = rounds * (kdim / 64 * stage + 2500 + 10 * bt);
-    if (best_cost < 0 || cost < best_cost) {
-      best_cost = cost;
-      best = bt <= 256 ? TokenTile{bt, 1} : TokenTile{bt / 2, 2};
+  for (int ks = 1; ks <= 4; ks *= 2) {
+    const int64_t slots = ks == 1 ? pairs : fused_pair_max_clusters(ks);
+    const int64_t nk = (kdim / 64 + ks - 1) / ks;
+    if (slots < 1 || nk < 2) continue;
+    for (int bt = !codes ? (phi16 ? 192 : 256) : ks > 1 ? 256 : 448; bt >= 32; bt -= 32) {
+      if (bt % (16 * ks)) continue;
+      const int64_t tiles = ((rows + 255) / 256) * ((T + bt - 1) / bt);
+      const int64_t rounds = (tiles + slots - 1) / slots;
+      const int64_t stage = !codes ? 960 + bt * 35 / 100
+                            : bt <= 256 ? (dx ? 538 + bt * 60 / 100 : 513 + bt * 36 / 100)
+                                        : (dx ? 749 + (bt - 288) * 183 / 100 : 655 + (bt - 288) * 214 / 100);
+      const int64_t cost = rounds * (nk * stage + 2500 + 10 * bt + (ks > 1 ? 2500 + 8 * bt : 0));
+      if (best_cost < 0 || cost < best_cost) {
+        best_cost = cost;
+        best = bt <= 256 ? PairTile{bt, 1, ks, cost} : PairTile{bt / 2, 2, ks, cost};
+      }
     }
   }
   return best;
 }
+// Whether a forward (rank up to 64) takes the codes pass rather than the in-stage tile: the pass (2.5 us
+// and 0.5 us per million weights; 10.8 us on 4096 x 4096, 34.7 on 13824 x 5120) and its GEMM against the
+// adapter layouts (2 us) and the slower stages.  Measured, codes / tile: 4096 x 4096 at T = 200 28.0 /
+// 26.9 us, at T = 1024 37 / 47; 14336 x 4096 at T = 64 49 / 40 us, at T = 2999 (11008 x 4096) 164 / 216.
+bool prefer_codes_fwd(const lrqat_layer& L, int64_t T, int pairs) {
+  constexpr double kCyclesPerUs = 1920.0;
+  const double pass = (2.5 + 0.5e-6 * static_cast<double>(L.m) * static_cast<double>(L.k)) * kCyclesPerUs;
+  const double codes = pass + static_cast<double>(pair_tile(L.m, L.k, T, pairs, true, false, false).cost);
+  const double tile = 2.0 * kCyclesPerUs +
+                      static_cast<double>(pair_tile(L.m, L.k, T, pairs, false, false, phi_16bit(L)).cost);
+  return codes <= tile;
+}
+
 constexpr int kDwPairTokensPerStage = 64;   // the pair dW kernel's stage (dw_pair.cu)
 // dW on CTA pairs (dw_pair.cu): 256 x 256 tiles, ranks up to 64, by the same setting as the
 // forward and dX GEMMs (lrqat_set_gemm_variant: not with 1, the one-SM kernels).
@@ -788,10 +803,17 @@ static int linear_fwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
   FwdWs ws;
   fwd_ws_layout(L, T, allow_codes, workspace, &ws);
   const int r16 = round16(L.r);
-  const bool cb = L.r > 64 || (allow_codes && codes_gemm(L));
-  const bool pair = use_pair(L.m, cb);
+  // A few tokens: their own kernel (ranks up to 64, unless a setting asks for a path).  Per call against
+  // the faster of the codes and the in-stage tile, r = 32: 4096 x 4096 at T = 16 15.1 / 25.1 us,
+  // 14336 x 4096 38 / 40, 256 x 256 7.0 / 9.6; its tile for 32 tokens spilled and lost (27 us).
+  const bool few = L.r <= 64 && T <= kFewTokens && g_gemm_variant.load(std::memory_order_relaxed) == 0 &&
+                   g_lowrank_path.load(std::memory_order_relaxed) == 0;
+  const bool pair = use_pair();
+  const int path = g_lowrank_path.load(std::memory_order_relaxed);
+  const bool cb = L.r > 64 || (!few && allow_codes && path != 1 &&
+                               (path == 2 || !pair || prefer_codes_fwd(L, T, dev->sms / 2)));
   // the pair kernel reads K-major factor slices, so it takes B^T from the padded copy
-  const bool direct = !cb && !pair && direct_factors(L, A, B);
+  const bool direct = !cb && !few && !pair && direct_factors(L, A, B);
   if (cb) {
     // the codes of every weight, once per call (from A and B themselves when the factors are direct)
     if (!direct_factors(L, A, B))
@@ -824,8 +846,29 @@ static int linear_fwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
                  "activation quantizer");
     tok = ws.x_codes;
   }
+  if (few) {
+    FewArgs f{};
+    f.m = L.m;
+    f.k = L.k;
+    f.T = static_cast<int32_t>(T);
+    f.r16 = r16;
+    f.q = make_quant_params(L.bits, frac_bits(L), L.alpha, L.r);
+    f.X = tok;
+    f.phi = Phi0;
+    f.a_pad = ws.a_pad;
+    f.bt_pad = ws.bt_pad;
+    f.s = s;
+    f.zero = L.zero;
+    f.s_ld = L.group_size ? static_cast<int32_t>(L.k / L.group_size) : 0;
+    f.group_size = L.group_size;
+    f.s_x = L.act_bits == 8 && !L.act_per_token ? s_x : nullptr;
+    f.u_bf16 = L.u_bf16;
+    f.Y = Y;
+    LRQAT_LAUNCH("fused_fwd", 1, stream, launch_fused_few(L.phi_format, f, stream), "few-token forward launch");
+    return LRQAT_OK;
+  }
   CUtensorMap tm_tok, tm_phi, tm_rf, tm_sf;
-  const TokenTile tile = pair_token_tile(L.m, L.k, T, dev->sms / 2, cb, false);
+  const PairTile tile = pair_tile(L.m, L.k, T, dev->sms / 2, cb, false, phi_16bit(L));
   LRQAT_TRY(encode_2d(&tm_tok, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, tok, L.k, T, L.k * 2, 64, pair ? tile.bnp / 2 : 224,
                       CU_TENSOR_MAP_SWIZZLE_128B, "X"));
   if (cb) {
@@ -888,8 +931,9 @@ static int linear_fwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
   if (pair) {
     a.bnp = tile.bnp;
     a.nacc = tile.nacc;
+    a.ksplit = tile.ksplit;
     const int64_t tiles = ((L.m + 255) / 256) * ((T + tile.tokens() - 1) / tile.tokens());
-    const int npairs = static_cast<int>(tiles < dev->sms / 2 ? tiles : dev->sms / 2);
+    const int npairs = static_cast<int>(tile.ksplit > 1 || tiles < dev->sms / 2 ? tiles : dev->sms / 2);
     LRQAT_LAUNCH("fused_fwd", 1, stream, launch_fused_pair(fmode, ffmt, tm_tok, tm_phi, tm_rf, tm_sf, a, npairs, stream),
                  "fused forward launch (CTA pairs)");
   } else {
@@ -972,7 +1016,7 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
   const int fmt_t = L.phi_format == LRQAT_PHI_INT_PACKED ? LRQAT_PHI_QFIXED : L.phi_format;
   // cb: the dX GEMM reads the codes (lrqat_set_lowrank_path); cbw: so does dW, with the clip mask in
   // the byte's top bit (needs codes of 7 bits; the pair kernel, and every rank above 64)
-  const bool cb = codes_gemm(L);
+  const bool cb = codes_bwd(L);
   const bool cbw = L.r > 64 || (cb && plan.pair && L.bits <= 7);
   const bool direct_ab = direct_factors(L, A, B);
   // with direct factors the dX GEMM reads its A slices from A itself (its row factor stays the
@@ -1027,9 +1071,9 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
       LRQAT_LAUNCH("dx_scales", 1, stream,
                    launch_dx_scales(s, L.zero, L.m, groups, L.group_size ? groups : 0, ws.s_bf16, ws.z_bf16, stream),
                    "dX scale rows");
-    const bool pair = use_pair(L.k, cb);
+    const bool pair = use_pair();
     CUtensorMap tm_tok, tm_phi, tm_rf, tm_sf;
-    const TokenTile tile = pair_token_tile(L.k, L.m, T, dev->sms / 2, cb, true);
+    const PairTile tile = pair_tile(L.k, L.m, T, dev->sms / 2, cb, true, phi_16bit(L));
     LRQAT_TRY(encode_2d(&tm_tok, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, dY, L.m, T, L.m * 2, 64, pair ? tile.bnp / 2 : 224,
                         CU_TENSOR_MAP_SWIZZLE_128B, "dY"));
     if (phi_16bit(L) && !cb)
@@ -1081,8 +1125,9 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
     if (pair) {
       a.bnp = tile.bnp;
       a.nacc = tile.nacc;
+      a.ksplit = tile.ksplit;
       const int64_t tiles = ((L.k + 255) / 256) * ((T + tile.tokens() - 1) / tile.tokens());
-      const int npairs = static_cast<int>(tiles < dev->sms / 2 ? tiles : dev->sms / 2);
+      const int npairs = static_cast<int>(tile.ksplit > 1 || tiles < dev->sms / 2 ? tiles : dev->sms / 2);
       LRQAT_LAUNCH("fused_dx", 1, stream,
                    launch_fused_pair(FUSED_DX, dfmt, tm_tok, tm_phi, tm_rf, tm_sf, a, npairs, stream),
                    "fused dX launch (CTA pairs)");

@@ -342,12 +342,21 @@ __device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, 
 __device__ __forceinline__ void mma_commit_pair_self(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-// Arrives on `bar` (same offset) in both CTAs of the pair once the pair MMAs issued so far
-// have completed.
-__device__ __forceinline__ void mma_commit_pair(uint32_t bar) {
+// Arrives on `bar` (same offset) in the CTAs of `mask` (both CTAs of the pair) once the pair MMAs
+// issued so far have completed.
+__device__ __forceinline__ void mma_commit_pair(uint32_t bar, uint32_t mask = 3u) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               ::"r"(bar), "h"(static_cast<uint16_t>(3))
+               ::"r"(bar), "h"(static_cast<uint16_t>(mask))
                : "memory");
+}
+// Distributed shared memory of the cluster (addresses of map_shared_rank).
+__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_shared_f32(uint32_t addr, float v) {
+  asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
 
 }  // namespace lrqat
