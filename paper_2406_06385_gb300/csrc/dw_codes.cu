@@ -100,6 +100,7 @@ struct Unit {
   int ib, jt, sp, t0, nsteps;   // ib: 256-row block of the pair
   int rev;                      // stages in descending token order
   int half_last;                // the last stage holds 32 tokens of the unit (an odd multiple of 32)
+  uint32_t keep;                // the 128 x 128 tiles that the unit writes (bit 2 r + c; wide plan)
 };
 
 __device__ __forceinline__ Unit decode_unit(int u, const DwArgs& a) {
@@ -114,6 +115,7 @@ __device__ __forceinline__ Unit decode_unit(int u, const DwArgs& a) {
   // the splits of ranks above 64 are multiples of 32 tokens: what follows in the stage's box
   // belongs to the next split
   x.half_last = (t1 - x.t0 + 31) / 32 & 1;
+  x.keep = 15u;
   x.rev = 0;
   return x;
 }
@@ -138,19 +140,22 @@ __device__ __forceinline__ void dw_whole_tile(int64_t u, int ni, int64_t full_ti
 struct WorkIter {
   int64_t u;
   bool tail;
+  int64_t st, st_u;   // wide plan: the tile that holds unit u or one before it, and its first unit
 };
 
 __device__ __forceinline__ WorkIter work_begin(const DwArgs& a, int pair) {
-  return {static_cast<int64_t>(pair), a.sched.tail != 0 && pair < a.sched.tail_grid};
+  return {static_cast<int64_t>(pair), a.sched.tail != 0 && pair < a.sched.tail_grid, a.sched.full_tiles,
+          a.sched.full_tiles};
 }
 
+template <bool WIDE>
 __device__ __forceinline__ bool work_next(WorkIter& it, const DwArgs& a, int pair, int npairs, Unit& x) {
   // Odd waves run their stages in descending token order: a wave shares its column (or row) blocks
   // with the wave before it, whose last stages are then still in L2 when it starts.
   if (!a.sched.tail) {
     if (it.u >= a.num_units) return false;
     x = decode_unit(static_cast<int>(it.u), a);
-    x.rev = a.r16 <= 64 ? static_cast<int>((it.u / npairs) & 1) : 0;
+    x.rev = WIDE || a.r16 > 64 ? 0 : static_cast<int>((it.u / npairs) & 1);
     it.u += npairs;
     return true;
   }
@@ -160,9 +165,38 @@ __device__ __forceinline__ bool work_next(WorkIter& it, const DwArgs& a, int pai
     x.t0 = 0;
     x.nsteps = static_cast<int>(a.sched.tsteps);
     x.half_last = 0;
-    x.rev = static_cast<int>((it.u / npairs) & 1);
+    x.keep = 15u;
+    x.rev = WIDE || a.r16 > 64 ? 0 : static_cast<int>((it.u / npairs) & 1);
     it.u += npairs;
     return true;
+  }
+  if (WIDE) {
+    // the tiles past the leading whole column tiles, in order, each with its passes
+    const int64_t tiles = static_cast<int64_t>(a.ni) * a.nj;
+    for (; it.st < tiles; ++it.st) {
+      int q[3];
+      uint32_t keep[3];
+      x.ib = static_cast<int>(it.st % a.ni);
+      x.jt = static_cast<int>(it.st / a.ni);
+      const int n = wide_passes(x.ib, x.jt, 2 * a.ni, a.base, q, keep);
+      int64_t p = it.u - it.st_u;   // which pass of this tile, if it is one
+      x.sp = static_cast<int>(p);
+      for (int y = 0; y < n; ++y) {
+        if (p < q[y]) {
+          const int64_t s0 = p * a.base.tsteps / q[y], s1 = (p + 1) * a.base.tsteps / q[y];   // 32-token stages
+          x.t0 = static_cast<int>(s0 * 32);
+          x.nsteps = static_cast<int>((s1 - s0 + 1) / 2);
+          x.half_last = static_cast<int>((s1 - s0) & 1);
+          x.rev = 0;
+          x.keep = keep[y];
+          it.u += npairs;
+          return true;
+        }
+        p -= q[y];
+      }
+      it.st_u = it.u - p;
+    }
+    return false;
   }
   if (!it.tail) return false;
   it.tail = false;
@@ -177,11 +211,14 @@ __device__ __forceinline__ bool work_next(WorkIter& it, const DwArgs& a, int pai
   x.t0 = static_cast<int>(s0 * BKT);
   x.nsteps = static_cast<int>(s1 - s0);
   x.half_last = 0;
+  x.keep = 15u;
   x.rev = 0;
   return true;
 }
 
-template <bool ZP>
+// WIDE: the wide plan of ranks above 64 (its pass bookkeeping costs registers: 169 -> 178 us where it
+// was compiled into every launch).
+template <bool ZP, bool WIDE>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     dw_codes_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_constant__ CUtensorMap tm_x,
                     const __grid_constant__ CUtensorMap tm_at, const __grid_constant__ CUtensorMap tm_b,
@@ -246,11 +283,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       bool ok = true;
       WorkIter wi = work_begin(args, pair);
       Unit w;
-      while (ok && work_next(wi, args, pair, npairs, w)) {
+      while (ok && work_next<WIDE>(wi, args, pair, npairs, w)) {
         if (args.sched.tail && w.sp == 0) {   // the reduction reads which slots hold data
           const int64_t tile2 = w.ib + static_cast<int64_t>(args.ni) * w.jt;
-          args.tile_segs[(2 * w.ib + static_cast<int>(rank)) + static_cast<int64_t>(ni128) * w.jt] =
-              dw_tile_segments(tile2, args.sched);
+          int segs;
+          if (WIDE) {
+            int q[3];
+            uint32_t keep[3];
+            const int n = wide_passes(w.ib, w.jt, ni128, args.base, q, keep);
+            segs = q[0] + (n > 1 ? q[1] : 0) + (n > 2 ? q[2] : 0);
+          } else {
+            segs = dw_tile_segments(tile2, args.sched);
+          }
+          args.tile_segs[(2 * w.ib + static_cast<int>(rank)) + static_cast<int64_t>(ni128) * w.jt] = segs;
         }
         const int i_own = w.ib * 256 + static_cast<int>(rank) * 128, j0 = w.jt * BN;
         for (int rc = 0; rc < rounds; ++rc, ++n) {
@@ -278,7 +323,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       bool ok = true;
       WorkIter wi = work_begin(args, pair);
       Unit w;
-      while (ok && work_next(wi, args, pair, npairs, w)) {
+      while (ok && work_next<WIDE>(wi, args, pair, npairs, w)) {
         const int i_own = w.ib * 256 + static_cast<int>(rank) * 128;
         const int j_own = w.jt * BN + static_cast<int>(rank) * 128;
         for (int step = 0; step < w.nsteps; ++step, ++g) {
@@ -305,7 +350,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       bool ok = true;
       WorkIter wi = work_begin(args, pair);
       Unit w;
-      while (ok && work_next(wi, args, pair, npairs, w)) {
+      while (ok && work_next<WIDE>(wi, args, pair, npairs, w)) {
         if (!(ok = wait_spin_bounded(bar(BAR_ACCEMPTY), (it & 1u) ^ 1u, ctl, 4))) break;
         tc_fence_after();
         for (int step = 0; step < w.nsteps; ++step) {
@@ -344,7 +389,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       bool ok = true;
       WorkIter wi = work_begin(args, pair);
       Unit w;
-      while (ok && work_next(wi, args, pair, npairs, w)) {
+      while (ok && work_next<WIDE>(wi, args, pair, npairs, w)) {
         if (!(ok = wait_spin_bounded(bar(BAR_DUFULL), it & 1u, ctl, 8))) break;
         for (int rc = 0; rc < rounds && ok; ++rc, ++n) {
           if (!(ok = wait_spin_bounded(bar(BAR_EFFULL), n & 1u, ctl, 6))) break;
@@ -408,7 +453,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     bool ok = true;
     WorkIter wi = work_begin(args, pair);
     Unit w;
-    while (ok && work_next(wi, args, pair, npairs, w)) {
+    while (ok && work_next<WIDE>(wi, args, pair, npairs, w)) {
       const int ib128 = 2 * w.ib + static_cast<int>(rank);
       const int i_g = ib128 * 128 + row;
       // this thread's code bytes (columns 64 h .. 64 h + 63 of both chunks of row i_g) and scales,
@@ -431,6 +476,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const float gs_i = gscale * s_i[c];
+        // a 128 x 128 tile that this unit does not write: no mask bits (dU = 0) and no ds
+        const bool keep = !WIDE || (w.keep >> (2 * rank + c)) & 1u;
+        const uint32_t kept = keep ? 0xffffffffu : 0x7f7f7f7fu;
         float2 ds2 = make_float2(0.0f, 0.0f);
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
@@ -448,7 +496,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
             const uint4& r4 = raw[4 * c + 2 * p + (e >> 2)];
-            const uint32_t wd = (e & 3) == 0 ? r4.x : (e & 3) == 1 ? r4.y : (e & 3) == 2 ? r4.z : r4.w;
+            const uint32_t wd = ((e & 3) == 0 ? r4.x : (e & 3) == 1 ? r4.y : (e & 3) == 2 ? r4.z : r4.w) & kept;
             float2 cv[2];
             decode_codes4(wd, cv[0], cv[1]);
 #pragma unroll
@@ -465,7 +513,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             st_shared_v4(dub + swz_offset(row, 4 * p + wq, 128), du[4 * wq], du[4 * wq + 1], du[4 * wq + 2],
                          du[4 * wq + 3]);
         }
-        args.ds_part[(static_cast<int64_t>(w.sp * 2 + h) * args.m + i_g) * nb + w.jt * 2 + c] = (ds2.x + ds2.y) * gscale;
+        args.ds_part[(static_cast<int64_t>(w.sp * 2 + h) * args.m + i_g) * nb + w.jt * 2 + c] = keep ? (ds2.x + ds2.y) * gscale : 0.0f;
       }
       tc_fence_before();
       fence_proxy_async_smem();
@@ -522,11 +570,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   }
 }
 
-template <bool ZP>
+template <bool ZP, bool WIDE>
 cudaError_t launch_codes_one(const CUtensorMap& dy, const CUtensorMap& x, const CUtensorMap& at, const CUtensorMap& b,
                              const DwArgs& args, int npairs, cudaStream_t stream) {
   static bool configured[kMaxDevices] = {};
-  const void* fn = reinterpret_cast<const void*>(dw_codes_kernel<ZP>);
+  const void* fn = reinterpret_cast<const void*>(dw_codes_kernel<ZP, WIDE>);
   cudaError_t e = ensure_smem_attr(fn, static_cast<int>(SMEM_BYTES), configured);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
@@ -541,7 +589,7 @@ cudaError_t launch_codes_one(const CUtensorMap& dy, const CUtensorMap& x, const 
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, dw_codes_kernel<ZP>, dy, x, at, b, args);
+  e = cudaLaunchKernelEx(&cfg, dw_codes_kernel<ZP, WIDE>, dy, x, at, b, args);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -552,10 +600,13 @@ cudaError_t launch_dw_codes(const CUtensorMap& tm_dy, const CUtensorMap& tm_x, c
                             const CUtensorMap& tm_b, const DwArgs& args, int npairs, cudaStream_t stream) {
   if (npairs < 1 || args.nchunks != 2 || args.r16 < 16 || args.r16 > 256 || (args.r16 & 15) || args.m % 256 ||
       args.k % 256 || args.ni != args.m / 256 || args.nj != args.k / 256 || args.u_bf16 || args.phi == nullptr ||
-      (args.sched.tail && args.r16 > 64))
+      (args.sched.tail && args.r16 > 64 && !args.wide))
     return cudaErrorInvalidValue;
-  return args.zero != nullptr ? launch_codes_one<true>(tm_dy, tm_x, tm_at, tm_b, args, npairs, stream)
-                              : launch_codes_one<false>(tm_dy, tm_x, tm_at, tm_b, args, npairs, stream);
+  if (args.wide)
+    return args.zero != nullptr ? launch_codes_one<true, true>(tm_dy, tm_x, tm_at, tm_b, args, npairs, stream)
+                                : launch_codes_one<false, true>(tm_dy, tm_x, tm_at, tm_b, args, npairs, stream);
+  return args.zero != nullptr ? launch_codes_one<true, false>(tm_dy, tm_x, tm_at, tm_b, args, npairs, stream)
+                              : launch_codes_one<false, false>(tm_dy, tm_x, tm_at, tm_b, args, npairs, stream);
 }
 
 }  // namespace lrqat

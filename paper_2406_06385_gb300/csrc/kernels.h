@@ -237,7 +237,35 @@ struct DwArgs {
   // Ranks above 64: the base (tm_phi) holds the code bytes (c + 64, bit 7 the clip mask); no
   // low-rank tile, nchunks == 1, tm_at / tm_b boxes of 64 rank rows.
   int32_t codes_base;
+  // Pair kernel on the codes, ranks above 64 whose plan (base, over 128 x 128 tiles of 32-token stages)
+  // has a tail: every 256 x 256 tile is passed once per token range that its 128 x 128 tiles have
+  // there, each pass keeping the tiles of that range (wide_passes); sched.full_tiles counts the
+  // 256 x 256 tiles of the leading column tiles that are whole.
+  int32_t wide;
+  DwSched base;
 };
+// The passes over 256 x 256 tile (I, J) of the wide plan: its 128 x 128 tiles (bit 2 r + c: row half
+// r, column half c) grouped by their part count q, ascending; q passes each.  Returns the groups.
+__host__ __device__ inline int wide_passes(int64_t I, int64_t J, int64_t ni128, const DwSched& base, int (&q)[3],
+                                           uint32_t (&tiles)[3]) {
+  int n = 0;
+  for (int x = 0; x < 4; ++x) {
+    const int v = dw_tile_segments(2 * I + (x >> 1) + ni128 * (2 * J + (x & 1)), base);
+    int at = 0;
+    while (at < n && q[at] < v) ++at;
+    if (at == n || q[at] != v) {   // part counts are 1 and two neighbouring numbers: at most three
+      for (int y = n; y > at; --y) {
+        q[y] = q[y - 1];
+        tiles[y] = tiles[y - 1];
+      }
+      q[at] = v;
+      tiles[at] = 0;
+      ++n;
+    }
+    tiles[at] |= 1u << x;
+  }
+  return n;
+}
 int dw_smem_bytes(int r16, int fmt);
 // The same kernel on CTA pairs (dw_pair.cu) for ranks up to 64, m and k multiples of 256:
 // units of 256 x 256 tiles (args.ni = m / 256, args.nj = k / 256, nchunks 2), npairs clusters of
@@ -248,7 +276,7 @@ cudaError_t launch_dw_pair(int fmt, const CUtensorMap& tm_dy, const CUtensorMap&
                            const CUtensorMap& tm_bh, const DwArgs& args, int npairs, cudaStream_t stream);
 // The pair kernel on the codes (dw_codes.cu), any rank up to 256: args.phi holds the code bytes
 // [m, k] (c + 64, bit 7 the clip mask); tm_at boxes of min(r16, 64) rank rows, tm_b of half as many;
-// ranks above 64 take equal token splits only.
+// ranks above 64 take equal token splits or the wide plan.
 cudaError_t launch_dw_codes(const CUtensorMap& tm_dy, const CUtensorMap& tm_x, const CUtensorMap& tm_at,
                             const CUtensorMap& tm_b, const DwArgs& args, int npairs, cudaStream_t stream);
 // Clusters of two of the pair dW kernel that can be resident at once on the current device

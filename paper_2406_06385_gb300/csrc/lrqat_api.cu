@@ -379,6 +379,8 @@ struct DwPlan {
   bool pair;   // the pair kernel: ni counts 256-row tiles and sched.grid pairs
   int ni128;   // 128-row blocks (the partial outputs)
   int bkt;     // tokens per pipeline stage
+  bool wide = false;   // passes of 256 x 256 tiles over the token ranges of `base` (ranks above 64)
+  DwSched base{};
 };
 
 // sms: the work slots of the persistent grid (SMs for the one-SM kernel, resident pairs for
@@ -443,24 +445,57 @@ DwPlan plan_dw(const lrqat_layer& L, int64_t T, int sms, bool pair) {
 }
 
 // The plan of a layer's dW on the current device (pairs: the pair kernels' resident clusters).
-// Ranks above 64 are planned as 128 x 128 tiles of 32-token stages over the SMs; where that plan
-// has equal token splits and the shape allows, the pair kernel on the codes takes the same splits
-// in 256 x 256 tiles, so every G has the same tokens in the same order.  A pair tile's stage costs
-// about as much as a 128 x 128 tile's, so pairs are taken when their rounds are no more.
+// Ranks above 64 are planned as 128 x 128 tiles of 32-token stages over the SMs, and where the shape
+// allows the pair kernel on the codes takes the same token ranges in 256 x 256 tiles, so every G has the
+// same tokens in the same order: equal splits as they are; with a tail, one pass per distinct range
+// of a 256 x 256 tile's four (DwArgs::wide), which repeats a few of them.  A pair stage of 64 tokens costs
+// about what a 128 x 128 tile's takes for 32 (690 cycles against ~585 with its epilogues), and its
+// epilogue runs beside the next main loop, so pairs are taken when their busiest one has no more
+// tokens to pass than the busiest SM (4096 x 4096 at T = 8192, r = 256: 4 tiles against 7 of a quarter the
+// size; dW 552 -> 290 us).
 DwPlan plan_layer_dw(const lrqat_layer& L, int64_t T, int sms, int pairs) {
   if (use_pair_dw(L)) return plan_dw(L, T, pairs, true);
-  DwPlan p = plan_dw(L, T, sms, false);
-  if (L.r <= 64 || p.sched.tail || !pair_dw_shape(L) || pairs < 1) return p;
-  const int64_t tiles = (L.m / 256) * (L.k / 256), units = tiles * p.nsplit;
-  if ((units + pairs - 1) / pairs > (p.units + sms - 1) / sms) return p;
+  const DwPlan one = plan_dw(L, T, sms, false);
+  if (L.r <= 64 || !pair_dw_shape(L) || pairs < 1) return one;
+  DwPlan p = one;
   p.pair = true;
   p.nchunks = 2;
   p.ni = static_cast<int>(L.m / 256);
   p.nj = static_cast<int>(L.k / 256);
   p.bkt = kDwPairTokensPerStage;
-  p.units = static_cast<int>(units);
-  p.sched = DwSched{0, static_cast<int32_t>(units < pairs ? units : pairs), (T + p.bkt - 1) / p.bkt, 0, 0, 0};
-  return p;
+  const int64_t tiles = static_cast<int64_t>(p.ni) * p.nj, tsteps = (T + p.bkt - 1) / p.bkt;
+  // the busiest pair's and SM's tokens, in 32-token stages
+  int64_t mine, theirs;
+  if (!one.sched.tail) {
+    const int64_t units = tiles * p.nsplit;
+    mine = (units + pairs - 1) / pairs * (one.tchunk / 32);
+    theirs = (one.units + one.sched.grid - 1) / one.sched.grid * (one.tchunk / 32);
+    p.units = static_cast<int>(units);
+    p.sched = DwSched{0, static_cast<int32_t>(units < pairs ? units : pairs), tsteps, 0, 0, 0};
+  } else {
+    const int64_t whole_cols = one.sched.full_tiles / one.ni128 / 2;   // column tiles of 256 that are whole
+    int64_t units = whole_cols * p.ni, total = units * one.sched.tsteps;
+    int most = 1;
+    for (int64_t st = units; st < tiles; ++st) {
+      int q[3];
+      uint32_t keep[3];
+      const int n = wide_passes(st % p.ni, st / p.ni, one.ni128, one.sched, q, keep);
+      int passes = 0;
+      for (int y = 0; y < n; ++y) passes += q[y];
+      units += passes;
+      total += n * one.sched.tsteps;
+      most = passes > most ? passes : most;
+    }
+    const int64_t rounds = (whole_cols * p.ni + pairs - 1) / pairs * one.sched.tsteps;
+    mine = (total + pairs - 1) / pairs > rounds ? (total + pairs - 1) / pairs : rounds;
+    theirs = one.sched.full_tiles / sms * one.sched.tsteps + one.sched.tsteps / (one.sched.tail_grid / one.sched.tail_tiles);
+    p.wide = true;
+    p.base = one.sched;
+    p.nsplit = most;
+    p.units = static_cast<int>(units);
+    p.sched = DwSched{1, static_cast<int32_t>(units < pairs ? units : pairs), tsteps, whole_cols * p.ni, 0, 0};
+  }
+  return mine <= theirs ? p : one;
 }
 
 struct FwdWs {
@@ -1185,6 +1220,8 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
     a.sched = plan.sched;
     a.tile_segs = ws.tile_segs;
     a.codes_base = cbw ? 1 : 0;
+    a.wide = plan.wide ? 1 : 0;
+    a.base = plan.base;
     const int grid = plan.sched.grid;
     if (plan.pair && cbw) {
       // each CTA of a pair loads half of a round's ranks of B

@@ -59,6 +59,32 @@ def test_gradients_from_codes_equal_those_from_the_low_rank_tile(cid, spec, T, s
     assert float((a - b).norm() / b.norm()) <= 4e-3
 
 
+WIDE_CASES = [
+    ("r96_few_tiles", _spec(512, 768, 96), 700),
+    ("r72_not_direct_odd_tokens", _spec(2560, 2304, 68), 333),
+    ("r256_mixed_parts", _spec(1280, 1536, 256), 1000),
+    ("r128_group_asym", _spec(768, 2816, 128, bits=3, group=128, asym=True), 2081),
+]
+
+
+@pytest.mark.parametrize("schedule", ["auto", "split", "tail"])
+@pytest.mark.parametrize("cid,spec,T", WIDE_CASES, ids=[c[0] for c in WIDE_CASES])
+def test_pair_gradients_of_large_ranks(cid, spec, T, schedule, gemm_variant, dw_schedule):
+    """Ranks above 64 on pairs against one SM: the same token ranges per 128 x 128 tile, so dU is the
+    same bit for bit and only the order of fp32 sums of partials differs (2^-18 relative)."""
+    t = torch()
+    dw_schedule(schedule)
+    data = WL.make_layer(spec, T, seed=4)
+    dl = DeviceLayer(data, 1.05)
+    X, dY = to_dev(data.X_bits), to_dev(data.dY_bits)
+    got = {}
+    for variant in ("single", "pair"):
+        gemm_variant(variant)
+        got[variant] = _grads(spec, T, dl, X, dY, None)[1:]
+    for name, a, b in zip(("dA", "dB", "ds"), *got.values()):
+        assert float((a - b).norm() / a.norm()) <= 2.0 ** -18, name
+
+
 TILE_CASES = [
     # odd numbers of 128-row blocks in both directions, token counts around the tiles' edges
     ("odd_blocks", _spec(384, 640, 32), 225),
