@@ -538,10 +538,13 @@ __global__ void __launch_bounds__(256) bwd_prep_kernel(LayoutJob lj, int64_t n_l
 }
 
 // ------------------------------------------------------------------- reduce --
-// One launch sums every gradient partial. Block ranges: [0, nblk_a) dA, then dB, then ds.
-// dA / dB: a block owns 32 float4 columns; warp w adds parts w, w + 8, w + 16, ... in that
-// order, and the eight warp sums are added in a fixed tree, so results are deterministic.
-constexpr int kRedSlices = kThreads / 32;
+// One launch sums every gradient partial. Block ranges: ds, then dA, then dB.
+// dA / dB: a thread adds the parts w, w + 4, w + 8, ... of one float4 column in that order, eight loads in
+// flight, and the four slices' sums are added in order, so results are deterministic.  Bound by latency:
+// fewer slices are longer chains of loads per thread, more are more blocks with little to do each
+// (4096 x 4096 at r = 32 with 1 / 2 / 4 / 8 slices 20.1 / 13.7 / 11.8 / 14.0 us, r = 256 61 / 53 / 54 / 77,
+// 13824 x 5120 48 / 37 / 32 / 40; before, eight slices with four loads in flight, 13.0, 71 and 41 us).
+constexpr int kRedSlices = 4;
 
 struct RedJob {
   const float4* part;
@@ -552,15 +555,6 @@ struct RedJob {
   int64_t width;   // r (dA) or k (dB): elements per row of a partial
 };
 
-// Whether partial slot sp of tile (ib, jt) was written by the dW kernel: every slot, unless
-// its schedule had a tail (then a tail tile has as many slots as parts, which the dW kernel
-// recorded).
-__device__ __forceinline__ bool slot_written(const ReduceArgs& a, int64_t ib, int64_t jt, int sp) {
-  if (!a.sched.tail || sp == 0) return true;
-  const int64_t tile = ib + a.ni * jt;
-  return tile >= a.sched.full_tiles && sp < __ldg(a.tile_segs + tile);
-}
-
 __device__ __forceinline__ void add4(float4& a, const float4& b) {
   a.x += b.x;
   a.y += b.y;
@@ -568,77 +562,69 @@ __device__ __forceinline__ void add4(float4& a, const float4& b) {
   a.w += b.w;
 }
 
-__device__ __forceinline__ void reduce_parts_block(const RedJob& j, int64_t blk, const ReduceArgs& a,
-                                                   float4 (*sm)[32]) {
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t e = blk * 32 + lane;
+__device__ __forceinline__ void reduce_parts_block(const RedJob& j, int64_t blk, const ReduceArgs& a, float4* sm) {
+  constexpr int slices = kRedSlices, cols = kThreads / slices;   // float4 columns of the block
+  const int w = threadIdx.x / cols, lane = threadIdx.x % cols;
+  const int64_t e = blk * cols + lane;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  auto part = [&](int64_t p) { return __ldg(j.part + p * j.n4 + e); };
-  if (e < j.n4 && !a.sched.tail) {
-    int p = w;
-    for (; p + 3 * kRedSlices < j.nparts; p += 4 * kRedSlices) {
-      const float4 v0 = part(p);
-      const float4 v1 = part(p + kRedSlices);
-      const float4 v2 = part(p + 2 * kRedSlices);
-      const float4 v3 = part(p + 3 * kRedSlices);
-      add4(acc, v0);
-      add4(acc, v1);
-      add4(acc, v2);
-      add4(acc, v3);
-    }
-    for (; p < j.nparts; p += kRedSlices) add4(acc, part(p));
-  } else if (e < j.n4) {
-    // With a tail: slot 0 of every tile (always written), spread over the warps, then the further
-    // slots of the tail's tiles.  Slot p = o * nsplit + sp, o the other tile coordinate (jt for
-    // dA, ib for dB); the tile coordinate this element fixes is the same for the whole block.
-    const int ns = a.nsplit;
+  if (e < j.n4) {
+    // Slot 0 of every tile (always written), then the further slots.  Slot p = o * nsplit + sp, o the other
+    // tile coordinate (jt for dA, ib for dB).  Without a tail every slot is written.
+    const int ns = a.sched.tail ? a.nsplit : 1;
     const int64_t n_other = j.nparts / ns;
-    const int64_t fixed = j.kind == 0 ? (4 * e / j.width) / 128 : ((4 * e) % j.width) / a.bn;
-    // first o whose tile (fixed + ni o for dA, o + ni fixed for dB) is past the whole tiles;
-    // this warp's first tail tile's part count is requested before the slot-0 loads
-    const int64_t ft = a.sched.full_tiles;
-    const int64_t o_tail = j.kind == 0 ? (ft > fixed ? (ft - fixed + a.ni - 1) / a.ni : 0)
-                                       : (ft > a.ni * fixed ? ft - a.ni * fixed : 0);
-    auto tile_of = [&](int64_t oo) { return j.kind == 0 ? fixed + a.ni * oo : oo + a.ni * fixed; };
-    int segs0 = o_tail + w < n_other ? __ldg(a.tile_segs + tile_of(o_tail + w)) : 0;
+    const float4* src = j.part + e;
+    const int64_t step = static_cast<int64_t>(slices) * ns * j.n4;
+    const float4* p = src + static_cast<int64_t>(w) * ns * j.n4;
     int64_t o = w;
-    for (; o + 3 * kRedSlices < n_other; o += 4 * kRedSlices) {
-      const float4 v0 = part(o * ns);
-      const float4 v1 = part((o + kRedSlices) * ns);
-      const float4 v2 = part((o + 2 * kRedSlices) * ns);
-      const float4 v3 = part((o + 3 * kRedSlices) * ns);
-      add4(acc, v0);
-      add4(acc, v1);
-      add4(acc, v2);
-      add4(acc, v3);
+    for (; o + 7 * slices < n_other; o += 8 * slices, p += 8 * step) {
+      float4 v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = __ldg(p + u * step);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) add4(acc, v[u]);
     }
-#pragma unroll 4
-    for (; o < n_other; o += kRedSlices) add4(acc, part(o * ns));
-    for (int64_t o2 = o_tail + w; o2 < n_other; o2 += kRedSlices) {
-      const int segs = segs0;
-      if (o2 + kRedSlices < n_other) segs0 = __ldg(a.tile_segs + tile_of(o2 + kRedSlices));
-      // slots 1 .. segs - 1, four loads in flight at a time
-      for (int sp = 1; sp < segs; sp += 4) {
-        float4 v[4];
+    for (; o + 3 * slices < n_other; o += 4 * slices, p += 4 * step) {
+      float4 v[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          v[q] = sp + q < segs ? part(o2 * ns + sp + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int u = 0; u < 4; ++u) v[u] = __ldg(p + u * step);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) add4(acc, v[q]);
+      for (int u = 0; u < 4; ++u) add4(acc, v[u]);
+    }
+    for (; o < n_other; o += slices, p += step) add4(acc, __ldg(p));
+    if (a.sched.tail) {
+      // the tile coordinate that this element fixes, and the first o whose tile (fixed + ni o for dA,
+      // o + ni fixed for dB) is past the whole tiles
+      const int64_t fixed = j.kind == 0 ? (4 * e / j.width) / 128 : ((4 * e) % j.width) / a.bn;
+      const int64_t ft = a.sched.full_tiles;
+      const int64_t o_tail = j.kind == 0 ? (ft > fixed ? (ft - fixed + a.ni - 1) / a.ni : 0)
+                                         : (ft > a.ni * fixed ? ft - a.ni * fixed : 0);
+      auto segs_of = [&](int64_t oo) {
+        return oo < n_other ? __ldg(a.tile_segs + (j.kind == 0 ? fixed + a.ni * oo : oo + a.ni * fixed)) : 0;
+      };
+      int segs0 = segs_of(o_tail + w);
+      for (int64_t o2 = o_tail + w; o2 < n_other; o2 += slices) {
+        const int segs = segs0;
+        segs0 = segs_of(o2 + slices);
+        // slots 1 .. segs - 1, four loads in flight at a time
+        for (int sp = 1; sp < segs; sp += 4) {
+          float4 v[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            v[q] = sp + q < segs ? __ldg(src + (o2 * ns + sp + q) * j.n4) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) add4(acc, v[q]);
+        }
       }
     }
   }
-  sm[w][lane] = acc;
+  sm[threadIdx.x] = acc;
   __syncthreads();
+  if (w == 0) {
+#pragma unroll
+    for (int s = 1; s < slices; ++s) add4(acc, sm[s * cols + lane]);
+  }
   if (w == 0 && e < j.n4) {
-    float4 s[kRedSlices];
-#pragma unroll
-    for (int i = 0; i < kRedSlices; ++i) s[i] = sm[i][lane];
-#pragma unroll
-    for (int h = kRedSlices / 2; h > 0; h >>= 1)
-#pragma unroll
-      for (int i = 0; i < h; ++i) add4(s[i], s[i + h]);
-    float4 r = make_float4(s[0].x * a.lr, s[0].y * a.lr, s[0].z * a.lr, s[0].w * a.lr);
+    float4 r = make_float4(acc.x * a.lr, acc.y * a.lr, acc.z * a.lr, acc.w * a.lr);
     if (a.accumulate) add4(r, j.dst[e]);
     j.dst[e] = r;
   }
@@ -714,17 +700,18 @@ __device__ __forceinline__ void reduce_ds_group(const float* __restrict__ part, 
 
 __global__ void __launch_bounds__(kThreads) reduce_grads_kernel(RedJob ja, RedJob jb, int64_t nblk_a, int64_t nblk_b,
                                                                 ReduceArgs a, int64_t nb, int ngroups) {
-  __shared__ float4 sm[kRedSlices][32];
-  const int64_t blk = blockIdx.x;
-  if (blk < nblk_a) {
+  __shared__ float4 sm[kThreads];
+  // the ds blocks first: a row's sums are a chain of dependent loads
+  const int64_t nblk_s = gridDim.x - nblk_a - nblk_b, blk = static_cast<int64_t>(blockIdx.x) - nblk_s;
+  if (blk < 0) {
+    if (a.group_size == 0)
+      reduce_ds_row(a.ds_part, a.nS, a.m, nb, a.accumulate, a.ds, blockIdx.x, a);
+    else
+      reduce_ds_group(a.ds_part, a.nS, a.m, nb, ngroups, a.group_size / 128, a.accumulate, a.ds, blockIdx.x, a);
+  } else if (blk < nblk_a) {
     reduce_parts_block(ja, blk, a, sm);
-  } else if (blk < nblk_a + nblk_b) {
-    reduce_parts_block(jb, blk - nblk_a, a, sm);
-  } else if (a.group_size == 0) {
-    reduce_ds_row(a.ds_part, a.nS, a.m, nb, a.accumulate, a.ds, blk - nblk_a - nblk_b, a);
   } else {
-    reduce_ds_group(a.ds_part, a.nS, a.m, nb, ngroups, a.group_size / 128, a.accumulate, a.ds,
-                    blk - nblk_a - nblk_b, a);
+    reduce_parts_block(jb, blk - nblk_a, a, sm);
   }
 }
 
@@ -826,7 +813,8 @@ cudaError_t launch_reduce(const ReduceArgs& a, cudaStream_t stream) {
   const int64_t nA4 = a.m * a.r / 4, nB4 = static_cast<int64_t>(a.r) * a.k / 4;   // m, k are multiples of 128
   const RedJob ja{reinterpret_cast<const float4*>(a.dA_part), a.nA, nA4, reinterpret_cast<float4*>(a.dA), 0, a.r};
   const RedJob jb{reinterpret_cast<const float4*>(a.dB_part), a.nB, nB4, reinterpret_cast<float4*>(a.dB), 1, a.k};
-  const int64_t nblk_a = (nA4 + 31) / 32, nblk_b = (nB4 + 31) / 32;
+  constexpr int64_t cols = kThreads / kRedSlices;
+  const int64_t nblk_a = (nA4 + cols - 1) / cols, nblk_b = (nB4 + cols - 1) / cols;
   const int64_t nb = a.k / 128;
   const int ngroups = a.group_size ? static_cast<int>(a.k / a.group_size) : 1;
   const int64_t nblk_s = a.group_size == 0 ? blocks_for(a.m * 32, kThreads) : blocks_for(a.m * ngroups, kThreads);
