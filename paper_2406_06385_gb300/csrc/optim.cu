@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <atomic>
 #include <cstdint>
+#include <utility>
 
 #include "kernels.h"
 #include "quant.cuh"
@@ -106,6 +107,9 @@ __device__ __noinline__ double norm_share_wide(const NormSeg& s, int64_t t0, int
 __global__ void __launch_bounds__(kNormThreads) grad_sqnorm_kernel(NormSeg a, NormSeg b, NormSeg c,
                                                                    float* __restrict__ sqnorm) {
   cg::cluster_group cluster = cg::this_cluster();
+  // Every CTA has to have started before another writes its shared memory: arrive here, wait before
+  // that write (the loads lie between, so the wait costs nothing).
+  auto started = cluster.barrier_arrive();
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kNormThreads;
   const int64_t t0 = static_cast<int64_t>(blockIdx.x) * kNormThreads + threadIdx.x;
   __shared__ double part[kNormThreads / 32];
@@ -145,8 +149,9 @@ __global__ void __launch_bounds__(kNormThreads) grad_sqnorm_kernel(NormSeg a, No
     acc = part[threadIdx.x];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (threadIdx.x == 0) cluster.map_shared_rank(cta_sum, 0)[blockIdx.x] = acc;
   }
+  cluster.barrier_wait(std::move(started));
+  if (threadIdx.x == 0) cluster.map_shared_rank(cta_sum, 0)[blockIdx.x] = acc;
   cluster.sync();
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     double total = 0.0;
