@@ -111,12 +111,14 @@ __global__ void __launch_bounds__(kThreads) range_minmax_kernel(const float* __r
 // idle at N = 100).  The segments pass through shared memory in chunks of kLpChunk values,
 // which all threads of a segment read at the same address (broadcast); rows kLpChunk + 4
 // values apart keep the segments that one warp spans on different banks.  Two neighbouring
-// values are one packed fp32x2 step: y = w r with r = fl32(1 / s) clamped to [n, p] (clip and
-// round commute, n and p being integers), rounded by the magic add; y lies within 2^-15 of the
-// exact quotient, so only when a y of eight lies within 2^-12 of a half-integer are they redone
-// with the IEEE division.  Measured on a 5120 x 5120 layer, N = 100, p = 2: 4232 us -> 962 us
-// (the FP32 and ALU pipes: 8 and 3
-// operations per weight and candidate).
+// values are one packed fp32x2 step but for the clip, which is the saturation of an FMA: with
+// r = fl32(1 / s) and W = p - n, t = sat(w r / W - n / W) and t W + n is the clipped quotient (clip and
+// round commute, n and p being integers) within 3 W 2^-24 of the IEEE one; the magic add rounds
+// it.  Only when one of eight values lies within W 2^-20 of a half-integer are they redone with the
+// IEEE division: a margin of 2^-12 for every width sent one warp step in eight there, this one in
+// 140 at 4 bits.  Measured on a 5120 x 5120 layer, N = 100, p = 2: 4232 us with a block per segment,
+// 962 us with clips by fminf / fmaxf and the fixed margin, 798 us now (the FP32 pipe: 7 operations per
+// weight and candidate).
 constexpr int kLpPairs = 4;             // packed pairs per step: one near-tie test for all of them
 constexpr int kLpChunk = 512;
 constexpr int kLpRow = kLpChunk + 4;
@@ -161,10 +163,11 @@ __global__ void __launch_bounds__(kLpMaxThreads) range_lp_kernel(const float* __
   const int g = threadIdx.x / n_cand, j = threadIdx.x % n_cand;
   const bool live = g < nloc;
   const float s = live ? static_cast<float>(static_cast<double>(seg_max[g]) * (j + 1) / n_cand) : 1.0f;
-  const float r = __frcp_rn(s);
-  const float2 r2 = make_float2(r, r), s2 = make_float2(-s, -s);
-  // a scale whose reciprocal overflows takes the division for every value
-  const float tie = r < INFINITY ? 0.499755859375f : -1.0f;   // 0.5 - 2^-12
+  const float r = __frcp_rn(s), width = pmax - nmin, c = -nmin / width, rw = r / width;
+  const float2 s2 = make_float2(-s, -s), width2 = make_float2(width, width);
+  const float2 up = make_float2(kMagic + nmin, kMagic + nmin);
+  // a scale whose reciprocal overflows or comes near the subnormals takes the division for every value
+  const float tie = r < INFINITY && r > 0x1p-100f ? 0.5f - width * 0x1p-20f : -1.0f;
   float2 acc = make_float2(0.0f, 0.0f);
   for (int c0 = 0; c0 < seg; c0 += kLpChunk) {
     const int len = seg - c0 < kLpChunk ? seg - c0 : kLpChunk;   // a multiple of 128
@@ -188,10 +191,10 @@ __global__ void __launch_bounds__(kLpMaxThreads) range_lp_kernel(const float* __
         }
 #pragma unroll
         for (int h = 0; h < kLpPairs; ++h) {
-          float2 y = __fmul2_rn(w[h], r2);
-          y = make_float2(fminf(fmaxf(y.x, nmin), pmax), fminf(fmaxf(y.y, nmin), pmax));
-          q[h] = __fadd2_rn(__fadd2_rn(y, make_float2(kMagic, kMagic)), make_float2(-kMagic, -kMagic));
-          const float2 d = __fadd2_rn(y, make_float2(-q[h].x, -q[h].y));
+          const float2 t = make_float2(__saturatef(__fmaf_rn(w[h].x, rw, c)), __saturatef(__fmaf_rn(w[h].y, rw, c)));
+          const float2 m = __fadd2_rn(__ffma2_rn(t, width2, up), make_float2(-kMagic, -kMagic));   // the code
+          q[h] = m;
+          const float2 d = __ffma2_rn(t, width2, make_float2(nmin - m.x, nmin - m.y));
           dmax = fmaxf(dmax, fmaxf(fabsf(d.x), fabsf(d.y)));
         }
         if (dmax > tie) {

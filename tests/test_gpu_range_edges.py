@@ -42,6 +42,33 @@ def test_lp_range_candidate_counts(n, m, k, group, p):
     assert bool((got <= best * (1 + 1e-4)).all())
 
 
+@pytest.mark.parametrize("bits,phi", [(2, WL.PHI_QFIXED), (4, WL.PHI_INT_PACKED), (7, WL.PHI_QFIXED), (8, WL.PHI_BF16)])
+@pytest.mark.parametrize("scale", [1.0, 0.0137, 2.0 ** -128, 2.0 ** 112])
+def test_lp_range_on_rounding_boundaries(bits, phi, scale):
+    """Weights at and next to the half steps of the full scale (one candidate in two of which the other is
+    the full scale itself), at ordinary and extreme scales: the summed |error| of the chosen scale is
+    the smallest up to the rounding of the fp32 sums (640 values: 640 * 2^-24 < 1e-4)."""
+    t = torch()
+    m, k, n = 128, 640, 2
+    top = 2 ** (bits - 1) - 1
+    rng = np.random.default_rng(bits)
+    W = (rng.integers(-2 * top, 2 * top + 1, size=(m, k)) / 2 * scale).astype(np.float32)
+    W = np.where(rng.random((m, k)) < 0.5, np.nextafter(W, np.float32(0)), W).astype(np.float32)
+    W[:, 0] = np.float32(top * scale)
+    s = t.empty(m, device="cuda")
+    LQ.range_lp(LQ.Layer.from_spec(_spec(m, k, bits=bits, phi=phi)), t.from_numpy(W).cuda(), s, 1.0, n)
+    s_max = (np.abs(W).max(1) / np.float32(top)).astype(np.float64)
+
+    def loss(sc):
+        sc = sc[:, None]
+        q = np.clip(np.rint((W / sc.astype(np.float32)).astype(np.float32)), -top - 1, top)
+        return np.abs(W - sc * q).sum(1)
+
+    got = s.cpu().numpy().astype(np.float64)
+    best = np.minimum(loss((s_max / 2).astype(np.float32).astype(np.float64)), loss(s_max))
+    assert (loss(got) <= best * (1 + 1e-4)).all()
+
+
 @pytest.mark.parametrize("phi,bits", [(WL.PHI_QFIXED, 4), (WL.PHI_QFIXED, 7), (WL.PHI_INT_PACKED, 3),
                                       (WL.PHI_FP8_E4M3, 4), (WL.PHI_BF16, 4)])
 @pytest.mark.parametrize("scale", [1.0, 2.0 ** -130, 2.0 ** 100, 0.0137])
