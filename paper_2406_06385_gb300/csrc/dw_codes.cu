@@ -269,6 +269,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   __syncthreads();
   cluster_sync_all();   // both CTAs' barriers exist before either signals the other
   tc_fence_after();
+  griddep_launch();
+  griddep_wait();   // no global memory is touched above
   const uint32_t tmem = tmem_base_s;
   const WaitCtl ctl{&abort_s, args.status, args.timeout_ns};
   const uint32_t sig_src = smem_u32(&sig_buf[0]);
@@ -464,7 +466,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) raw[4 * c + e] = __ldg(reinterpret_cast<const uint4*>(cp + 128 * c) + e);
+        for (int e = 0; e < 4; ++e) raw[4 * c + e] = reinterpret_cast<const uint4*>(cp + 128 * c)[e];
         const int64_t si = args.s_ld ? static_cast<int64_t>(i_g) * args.s_ld + (w.jt * BN + 128 * c) / args.group_size : i_g;
         s_i[c] = args.s[si];
         z_i[c] = ZP ? args.zero[si] : 0.0f;
@@ -582,13 +584,14 @@ cudaError_t launch_codes_one(const CUtensorMap& dy, const CUtensorMap& x, const 
   cfg.blockDim = dim3(NUM_THREADS, 1, 1);
   cfg.dynamicSmemBytes = SMEM_BYTES;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
+  attr[1] = follows_in_call();
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   e = cudaLaunchKernelEx(&cfg, dw_codes_kernel<ZP, WIDE>, dy, x, at, b, args);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();

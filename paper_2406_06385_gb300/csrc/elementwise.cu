@@ -5,6 +5,7 @@
 #include <cstdint>
 
 #include "kernels.h"
+#include "ptx.cuh"
 #include "quant.cuh"
 
 namespace lrqat {
@@ -410,6 +411,7 @@ __global__ void adapter_layouts_kernel(const uint16_t* __restrict__ A, const uin
                                        int64_t k, int r, int r16, uint4* __restrict__ A_pad,
                                        uint4* __restrict__ Bt_pad, uint4* __restrict__ At,
                                        uint4* __restrict__ B_pad, int b_aligned) {
+  griddep_launch();
   adapter_layouts_body(blockIdx.x, gridDim.x, A, B, m, k, r, r16, A_pad, Bt_pad, At, B_pad, b_aligned);
 }
 
@@ -579,18 +581,18 @@ __device__ __forceinline__ void reduce_parts_block(const RedJob& j, int64_t blk,
     for (; o + 7 * slices < n_other; o += 8 * slices, p += 8 * step) {
       float4 v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = __ldg(p + u * step);
+      for (int u = 0; u < 8; ++u) v[u] = p[u * step];
 #pragma unroll
       for (int u = 0; u < 8; ++u) add4(acc, v[u]);
     }
     for (; o + 3 * slices < n_other; o += 4 * slices, p += 4 * step) {
       float4 v[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) v[u] = __ldg(p + u * step);
+      for (int u = 0; u < 4; ++u) v[u] = p[u * step];
 #pragma unroll
       for (int u = 0; u < 4; ++u) add4(acc, v[u]);
     }
-    for (; o < n_other; o += slices, p += step) add4(acc, __ldg(p));
+    for (; o < n_other; o += slices, p += step) add4(acc, *p);
     if (a.sched.tail) {
       // the tile coordinate that this element fixes, and the first o whose tile (fixed + ni o for dA,
       // o + ni fixed for dB) is past the whole tiles
@@ -599,7 +601,7 @@ __device__ __forceinline__ void reduce_parts_block(const RedJob& j, int64_t blk,
       const int64_t o_tail = j.kind == 0 ? (ft > fixed ? (ft - fixed + a.ni - 1) / a.ni : 0)
                                          : (ft > a.ni * fixed ? ft - a.ni * fixed : 0);
       auto segs_of = [&](int64_t oo) {
-        return oo < n_other ? __ldg(a.tile_segs + (j.kind == 0 ? fixed + a.ni * oo : oo + a.ni * fixed)) : 0;
+        return oo < n_other ? a.tile_segs[j.kind == 0 ? fixed + a.ni * oo : oo + a.ni * fixed] : 0;
       };
       int segs0 = segs_of(o_tail + w);
       for (int64_t o2 = o_tail + w; o2 < n_other; o2 += slices) {
@@ -610,7 +612,7 @@ __device__ __forceinline__ void reduce_parts_block(const RedJob& j, int64_t blk,
           float4 v[4];
 #pragma unroll
           for (int q = 0; q < 4; ++q)
-            v[q] = sp + q < segs ? __ldg(src + (o2 * ns + sp + q) * j.n4) : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[q] = sp + q < segs ? src[(o2 * ns + sp + q) * j.n4] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
           for (int q = 0; q < 4; ++q) add4(acc, v[q]);
         }
@@ -633,20 +635,20 @@ __device__ __forceinline__ void reduce_parts_block(const RedJob& j, int64_t blk,
 // Sum over the 128-column blocks b = b0, b0 + step, ... < b_end of row i of the parts that the
 // tail wrote past slot 0 (tiles past the whole ones; their part count read once per block, the
 // slots' loads issued together).
-__device__ __forceinline__ float ds_tail_slots(const float* __restrict__ part, int64_t m, int64_t nb, int64_t i,
+__device__ __forceinline__ float ds_tail_slots(const float* part, int64_t m, int64_t nb, int64_t i,
                                                int64_t b0, int64_t step, const ReduceArgs& a, int64_t b_end = -1) {
   if (b_end < 0) b_end = nb;
   float acc = 0.0f;
   for (int64_t b = b0; b < b_end; b += step) {
     const int64_t tile = i / 128 + a.ni * (b * 128 / a.bn);
     if (tile < a.sched.full_tiles) continue;
-    const int segs = __ldg(a.tile_segs + tile);
+    const int segs = a.tile_segs[tile];
     for (int sp = 1; sp < segs; sp += 2) {
       float v[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int p = 2 * (sp + q / 2) + (q & 1);
-        v[q] = sp + q / 2 < segs ? __ldg(part + (static_cast<int64_t>(p) * m + i) * nb + b) : 0.0f;
+        v[q] = sp + q / 2 < segs ? part[(static_cast<int64_t>(p) * m + i) * nb + b] : 0.0f;
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc += v[q];
@@ -657,8 +659,8 @@ __device__ __forceinline__ float ds_tail_slots(const float* __restrict__ part, i
 
 // ds[i] (per channel): one warp per row; lane l sums blocks l, l + 32, ... of every
 // part, then a fixed shuffle tree adds the lanes.
-__device__ __forceinline__ void reduce_ds_row(const float* __restrict__ part, int nparts, int64_t m, int64_t nb,
-                                              int accumulate, float* __restrict__ ds, int64_t blk,
+__device__ __forceinline__ void reduce_ds_row(const float* part, int nparts, int64_t m, int64_t nb,
+                                              int accumulate, float* ds, int64_t blk,
                                               const ReduceArgs& a) {
   const int64_t i = (blk * kThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -678,9 +680,9 @@ __device__ __forceinline__ void reduce_ds_row(const float* __restrict__ part, in
 }
 
 // ds[i][g] (per group): one thread per (row, group), sequential over its blocks.
-__device__ __forceinline__ void reduce_ds_group(const float* __restrict__ part, int nparts, int64_t m, int64_t nb,
+__device__ __forceinline__ void reduce_ds_group(const float* part, int nparts, int64_t m, int64_t nb,
                                                 int ngroups, int blocks_per_group, int accumulate,
-                                                float* __restrict__ ds, int64_t blk, const ReduceArgs& a) {
+                                                float* ds, int64_t blk, const ReduceArgs& a) {
   const int64_t e = blk * kThreads + threadIdx.x;
   if (e >= m * ngroups) return;
   const int64_t i = e / ngroups;
@@ -701,6 +703,7 @@ __device__ __forceinline__ void reduce_ds_group(const float* __restrict__ part, 
 __global__ void __launch_bounds__(kThreads) reduce_grads_kernel(RedJob ja, RedJob jb, int64_t nblk_a, int64_t nblk_b,
                                                                 ReduceArgs a, int64_t nb, int ngroups) {
   __shared__ float4 sm[kThreads];
+  griddep_wait();   // the loads below are plain ones: a read-only load may move up past this
   // the ds blocks first: a row's sums are a chain of dependent loads
   const int64_t nblk_s = gridDim.x - nblk_a - nblk_b, blk = static_cast<int64_t>(blockIdx.x) - nblk_s;
   if (blk < 0) {
@@ -818,9 +821,15 @@ cudaError_t launch_reduce(const ReduceArgs& a, cudaStream_t stream) {
   const int64_t nb = a.k / 128;
   const int ngroups = a.group_size ? static_cast<int>(a.k / a.group_size) : 1;
   const int64_t nblk_s = a.group_size == 0 ? blocks_for(a.m * 32, kThreads) : blocks_for(a.m * ngroups, kThreads);
-  reduce_grads_kernel<<<static_cast<unsigned>(nblk_a + nblk_b + nblk_s), kThreads, 0, stream>>>(ja, jb, nblk_a, nblk_b,
-                                                                                               a, nb, ngroups);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(nblk_a + nblk_b + nblk_s), 1, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1] = {follows_in_call()};
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, reduce_grads_kernel, ja, jb, nblk_a, nblk_b, a, nb, ngroups);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace lrqat

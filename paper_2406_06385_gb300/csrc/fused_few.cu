@@ -21,6 +21,7 @@
 #include <cstdint>
 
 #include "kernels.h"
+#include "ptx.cuh"
 #include "quant.cuh"
 
 namespace lrqat {
@@ -71,6 +72,20 @@ __global__ void __launch_bounds__(kThreads, 1) fused_few_kernel(const FewArgs ar
   const uint32_t lr2 = pack_rn_bf16x2(qp.lr_scale, qp.lr_scale);   // exact: a power of two with u_bf16
   const bool ub = args.u_bf16, zp = args.zero != nullptr, grouped = args.group_size != 0;
 
+  const int nblocks = static_cast<int>(k / 64);
+  Raw<FMT> raw[2][2], nxt[2][2];
+  auto load_block = [&](int b, Raw<FMT> (&r)[2][2]) {
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        load_raw<FMT>(args.phi, row0 + 16 * mt + 8 * h + g, k, static_cast<int64_t>(b) * 64 + 16 * c, r[mt][h]);
+  };
+  if (warp < nblocks) load_block(warp, nxt);
+  // The base is the caller's, complete before the call's first kernel began; X and the factors may come
+  // from the call's kernels before this one and are read with plain loads after the wait.
+  griddep_wait();
+
   // A [32 rows, r16] as fragments: rows g, g + 8 of each m16 tile, this thread's r16 / 4 ranks
   uint32_t af[2][KS][4];
 #pragma unroll
@@ -80,7 +95,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_few_kernel(const FewArgs ar
       const uint2* src = reinterpret_cast<const uint2*>(args.a_pad + (row0 + 16 * mt + 8 * h + g) * 64 + c * (4 * KS));
 #pragma unroll
       for (int ks = 0; ks < KS; ++ks) {
-        const uint2 v = __ldg(src + ks);   // ranks at positions 2 c, 2 c + 1 | 2 c + 8, 2 c + 9
+        const uint2 v = src[ks];   // ranks at positions 2 c, 2 c + 1 | 2 c + 8, 2 c + 9
         af[mt][ks][h] = v.x;
         af[mt][ks][2 + h] = v.y;
       }
@@ -96,16 +111,6 @@ __global__ void __launch_bounds__(kThreads, 1) fused_few_kernel(const FewArgs ar
       }
   }
   float acc[2][NT8][4] = {};
-  const int nblocks = static_cast<int>(k / 64);
-  Raw<FMT> raw[2][2], nxt[2][2];
-  auto load_block = [&](int b, Raw<FMT> (&r)[2][2]) {
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-      for (int h = 0; h < 2; ++h)
-        load_raw<FMT>(args.phi, row0 + 16 * mt + 8 * h + g, k, static_cast<int64_t>(b) * 64 + 16 * c, r[mt][h]);
-  };
-  if (warp < nblocks) load_block(warp, nxt);
   for (int b = warp; b < nblocks; b += kWarps) {
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
@@ -131,7 +136,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_few_kernel(const FewArgs ar
       const int t = 8 * n + g;
       const uint4* src = reinterpret_cast<const uint4*>(args.X + static_cast<int64_t>(t) * k + col0 + 16 * c);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) x[n][h] = t < args.T ? __ldg(src + h) : make_uint4(0u, 0u, 0u, 0u);
+      for (int h = 0; h < 2; ++h) x[n][h] = t < args.T ? src[h] : make_uint4(0u, 0u, 0u, 0u);
     }
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
@@ -143,7 +148,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_few_kernel(const FewArgs ar
         const uint2* src = reinterpret_cast<const uint2*>(args.bt_pad + col * 64 + c * (4 * KS));
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks) {
-          const uint2 v = __ldg(src + ks);
+          const uint2 v = src[ks];
 #pragma unroll
           for (int mt = 0; mt < 2; ++mt) mma16816(L[mt][hf], af[mt][ks], v.x, v.y);
         }
@@ -210,15 +215,22 @@ __global__ void __launch_bounds__(kThreads, 1) fused_few_kernel(const FewArgs ar
 
 template <int FMT, int NT8>
 cudaError_t launch_ks(const FewArgs& a, cudaStream_t stream) {
-  const unsigned grid = static_cast<unsigned>(a.m / kRows);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(a.m / kRows), 1, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1] = {follows_in_call()};
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaError_t e;
   switch (a.r16) {
-    case 16: fused_few_kernel<FMT, NT8, 1><<<grid, kThreads, 0, stream>>>(a); break;
-    case 32: fused_few_kernel<FMT, NT8, 2><<<grid, kThreads, 0, stream>>>(a); break;
-    case 48: fused_few_kernel<FMT, NT8, 3><<<grid, kThreads, 0, stream>>>(a); break;
-    case 64: fused_few_kernel<FMT, NT8, 4><<<grid, kThreads, 0, stream>>>(a); break;
+    case 16: e = cudaLaunchKernelEx(&cfg, fused_few_kernel<FMT, NT8, 1>, a); break;
+    case 32: e = cudaLaunchKernelEx(&cfg, fused_few_kernel<FMT, NT8, 2>, a); break;
+    case 48: e = cudaLaunchKernelEx(&cfg, fused_few_kernel<FMT, NT8, 3>, a); break;
+    case 64: e = cudaLaunchKernelEx(&cfg, fused_few_kernel<FMT, NT8, 4>, a); break;
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <int FMT>

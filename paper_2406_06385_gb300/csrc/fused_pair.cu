@@ -219,6 +219,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   __syncthreads();
   cluster_sync_all();   // both CTAs' barriers exist before either signals the other
   tc_fence_after();
+  griddep_launch();
+  griddep_wait();   // no global memory is touched above
   const uint32_t tmem = tmem_base_s;
   const WaitCtl ctl{&abort_s, args.status, args.timeout_ns};
   // this pair's stages k0 .. k0 + nk - 1 (kdim is a multiple of 128, ksplit at most kdim / 64)
@@ -645,7 +647,8 @@ cudaError_t launch_pair_one(const CUtensorMap& a, const CUtensorMap& b, const CU
   cfg.blockDim = dim3(NUM_THREADS, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
+  attr[1] = follows_in_call();
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = static_cast<unsigned>(2 * args.ksplit);
   attr[0].val.clusterDim.y = 1;
@@ -653,6 +656,7 @@ cudaError_t launch_pair_one(const CUtensorMap& a, const CUtensorMap& b, const CU
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (args.ksplit > 1) {   // one tile per cluster, however many are resident at once
+    cfg.numAttrs = 2;
     e = cudaLaunchKernelEx(&cfg, fused_pair_kernel<MODE, FMT, ZP, UB, NL>, a, b, c, d, args);
     return e != cudaSuccess ? e : cudaGetLastError();
   }
@@ -673,6 +677,7 @@ cudaError_t launch_pair_one(const CUtensorMap& a, const CUtensorMap& b, const CU
     npairs = max_pairs[dev];
     cfg.gridDim = dim3(static_cast<unsigned>(2 * npairs), 1, 1);
   }
+  cfg.numAttrs = 2;
   e = cudaLaunchKernelEx(&cfg, fused_pair_kernel<MODE, FMT, ZP, UB, NL>, a, b, c, d, args);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();

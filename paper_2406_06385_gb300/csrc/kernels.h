@@ -29,6 +29,20 @@ inline cudaError_t ensure_smem_attr(const void* kernel, int bytes, bool* done) {
   return cudaSuccess;
 }
 
+// Launch attribute of a kernel that follows another one of the same call: its blocks may be set up (barriers,
+// TMEM, cluster) while the kernel before it ends; it waits (griddep_wait, ptx.cuh) before it touches
+// memory.  Only such kernels carry it: a call's first launch depends on the whole stream as usual, so
+// what a program launches before and between calls never overlaps with ours.
+// Measured (eager calls; the gaps between a call's launches): 256 x 256 layer, T = 64, r = 4, forward and
+// backward 51.2 -> 41.4 us; 4096 x 4096 few-token forward 18.4 -> 16.4; two micro-batches of 1024 tokens
+// 292 -> 281; at T = 8192 within the runs' difference.
+inline cudaLaunchAttribute follows_in_call() {
+  cudaLaunchAttribute a{};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  return a;
+}
+
 // ---- range.cu --------------------------------------------------------------
 // z0 == nullptr: symmetric range setting (s0 only); else asymmetric (s0 and zero offsets z0).
 cudaError_t launch_range_minmax(const float* W0, int64_t m, int64_t k, int group_size, int bits, float* s0,

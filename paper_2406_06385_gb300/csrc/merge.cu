@@ -237,6 +237,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 2) merge_tc_kernel(const __grid_c
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  griddep_launch();
   const uint32_t tmem = tmem_base_s;
   const WaitCtl ctl{&abort_s, args.status, args.timeout_ns};
 
