@@ -41,6 +41,21 @@ def test_gradient_norm_range_and_alignment(scale, shift):
     assert t.isnan(sq).item()
 
 
+@pytest.mark.parametrize("m,k,r", [(128, 128, 1), (4096, 2048, 130), (2048, 4096, 256)])
+@pytest.mark.parametrize("shift", [0, 3])
+def test_gradient_norm_sizes(m, k, r, shift):
+    """From less than one 16-byte item per thread to several batches of loads, the arrays' borders inside
+    a batch; 2^-23 relative as above, over values of very different size in the three arrays."""
+    t = torch()
+    g = t.Generator(device="cuda").manual_seed(m + r)
+    mk = lambda n, f: (t.randn(n + shift, generator=g, device="cuda") * f)[shift:]
+    dA, dB, ds = mk(m * r, 1.0), mk(r * k, 1e-3), mk(m, 30.0)
+    sq = t.zeros(1, device="cuda")
+    LQ.grad_sqnorm(LQ.Layer.from_spec(_spec(m, k, r)), dA, dB, ds, sq)
+    want = sum(x.double().square().sum() for x in (dA, dB, ds)).item()
+    assert abs(sq.item() - want) <= 2.0 ** -23 * want
+
+
 @pytest.mark.parametrize("r", [1, 20])
 def test_adamw_of_unaligned_arrays(r):
     """Arrays that start off a 16-byte boundary take the one-element kernel: same values."""
