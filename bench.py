@@ -38,7 +38,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustain
 GEMM_KERNELS = ("fused_fwd", "fused_dx", "fused_dw")
 # the sources whose kernels a traced name can refer to (the forward and dX run on CTA pairs or on one SM)
 KERNEL_SOURCES = {"fused_fwd": ("fused_gemm.cu", "fused_pair.cu"), "fused_dx": ("fused_gemm.cu", "fused_pair.cu"),
-                  "fused_dw": ("dw.cu", "dw_pair.cu")}
+                  "fused_dw": ("dw.cu", "dw_pair.cu", "dw_codes.cu")}
 
 
 # --------------------------------------------------------------------------- helpers

@@ -8,24 +8,25 @@
 // half of every accumulator's tokens, and the tensor cores of the pair exchange the token halves
 // (measured on a 4096 x 4096 layer at T = 8192 on the codes: forward 276 -> 181 us).
 //
-// A pair processes tiles of 256 weight rows (CTA rank c: rows 128 c .. 128 c + 127) x up to 448
-// tokens (an odd last 128-row block leaves the second CTA's half of its tiles empty; two accumulators of 224 tokens; CTA c holds tokens 112 c .. 112 c + 111 of each; the
-// host picks smaller token tiles where 448 leave pairs idle, pair_token_tile in lrqat_api.cu), one
-// 64-wide slice of the contraction per stage:
-//   * token ring (three slots per CTA, four to eight on the codes): loader warps bring this
-//     CTA's token halves (SW128) with TMA whose completion lands on the leader's
-//     barrier; each slot also holds this CTA's W_hat tile of the stage;
-//   * factor ring (four slots, 2 for 16-bit bases, up to eight on the codes): the stored base of this CTA's rows (completion
+// A pair processes tiles of 256 weight rows (CTA rank c: rows 128 c .. 128 c + 127; an odd last
+// 128-row block leaves CTA 1's half of its tiles empty) x up to 448 tokens (one accumulator of up to 256
+// tokens or two of up to 224; CTA c holds half of each one's; the host picks smaller token tiles where
+// 448 leave pairs idle, and two or four pairs per tile where those do too: pair_tile in
+// lrqat_api.cu), one 64-wide slice of the contraction per stage:
+//   * token ring (four to eight slots per CTA): loader warps bring this CTA's token halves
+//     (SW128) with TMA whose completion lands on the leader's barrier; each slot also holds this
+//     CTA's W_hat tile of the stage;
+//   * factor ring (four or eight slots): the stored base of this CTA's rows (completion
 //     on its own barrier; only its own producers read it), with it the stage's scales (and zero
 //     offsets) where the producers apply them (dX, group-wise forward), and with the low-rank tile
 //     this CTA's half (32 rows) of the second factor's slice (completion on the leader's
 //     barrier: the low-rank MMA reads both halves);
-//   * in the leader, one thread issues the main product (M = 256, N = 224, 8 MMAs per stage) and,
-//     with the low-rank tile in the stage, another the tile L = RF SF^T (M = 256, N = 64) into a
-//     TMEM buffer after the accumulators, so that neither waits behind the other's barriers;
-//     every commit is multicast to both CTAs;
-//   * sixteen producer warps per CTA build this CTA's W_hat tile exactly as the one-SM kernel
-//     does (on the codes, two stages per iteration), and drain this CTA's 128 rows of the
+//   * in the leader, one thread per accumulator issues its main product (M = 256, 4 MMAs per stage)
+//     and, with the low-rank tile in the stage (one accumulator), another the tile L = RF SF^T
+//     (M = 256, N = 64) into one of four TMEM buffers after it, so that neither waits behind the
+//     other's barriers; every commit is multicast to both CTAs;
+//   * sixteen producer warps per CTA, in four groups that take every fourth stage each, build this
+//     CTA's W_hat tile exactly as the one-SM kernel does, and drain this CTA's 128 rows of the
 //     accumulators in the epilogue.
 // One barrier per slot in the leader counts the stage's token bytes and both CTAs' "W_hat
 // written" events, so the MMA thread tests one barrier per stage; the peer's events ("W_hat
@@ -33,8 +34,8 @@
 // memory whose completion counts on the leader's barrier (a thread-issued remote arrive is
 // several times slower under the pair's operand traffic), after fence.proxy.async has ordered
 // the peer's writes.
-// On the codes (NL: every call but the allocation-free forward of ranks up to 64, unless set
-// otherwise) the base holds the one-byte codes of the codes pass; no factors, no L.
+// On the codes (NL: every backward, and the forwards for which prefer_codes_fwd in lrqat_api.cu says
+// so, unless set otherwise) the base holds the one-byte codes of the codes pass; no factors, no L.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <atomic>

@@ -5,12 +5,12 @@
 // transposed for dX, and for dW row-major with the clip mask in the byte's top bit.
 //
 // Tiles of 128 x 128: the tile's rows of A and columns of B land by TMA, r16 / 16 tcgen05
-// MMAs write the low-rank tile L = A B into TMEM, and warp q turns rows 32q .. 32q + 31 into
-// codes (TMEM lane = row): it reads L 32 columns at a time, takes the stored base of the same
-// 32 columns (staged by TMA into the operand slot), rounds, clamps to [lo, hi] of the quantizer
-// constants, adds the bias and stores 32 one-byte codes as two 16-byte words.  The CTAs are persistent and overlap one tile's
-// codes with the next tile's copies and MMAs (two TMEM buffers).  The pass moves the base and the codes once (the product costs 2 m k r flops
-// on the tensor cores instead of the CUDA cores).
+// MMAs write the low-rank tile L = A B into TMEM, and warps q and q + 4 turn rows 32q .. 32q + 31
+// into codes (TMEM lane = row): they read L 32 columns at a time, take the stored base of the same
+// 32 columns (staged by TMA into the operand slot), round, clip, add the bias and store 32
+// one-byte codes as one 32-byte word.  The CTAs are persistent and overlap one tile's codes with
+// the next tile's copies and MMAs (two TMEM buffers).  The pass moves the base and the codes once (the
+// product costs 2 m k r flops on the tensor cores instead of the CUDA cores).
 //   A operand: K-major boxes of 64 rank columns read from A [m, r] (r % 8 == 0; columns
 //   past r read as zeros), or (AMN) two MN-major boxes of r16 rank rows x 64 rows read
 //   from the zero-padded A^T [r16, m].
