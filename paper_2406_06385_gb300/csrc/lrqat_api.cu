@@ -329,9 +329,14 @@ struct PairTile {
 // idle, two or four pairs share a tile's contraction and add their sums through distributed shared
 // memory (T = 256, forward 26.6 us with one pair, 22.8 with two; dX 29.1, 22.6).  With the low-rank tile in the stage (one accumulator: its buffers
 // take the other's TMEM) a stage takes 971 to 1050 cycles.
+// Those figures are of operands that stay in L2.  Beyond it smaller tiles, which read the operands more
+// often, are slower than the model says: 288-token tiles, 1% cheaper by it, took 1408 us for a 5120 x
+// 13824 forward at T = 16384 and 418 for 4096 x 11008 at T = 8192, 448-token tiles 1153 and 380.  There a
+// smaller tile has to be cheaper by an eighth.
 PairTile pair_tile(int64_t rows, int64_t kdim, int64_t T, int pairs, bool codes, bool dx, bool phi16) {
   PairTile best{0, 0, 1, 0};
   int64_t best_cost = -1;
+  const bool beyond_l2 = kdim * (rows + 2 * T) > (int64_t{100} << 20);   // one byte a weight, two a token value
   for (int ks = 1; ks <= 4; ks *= 2) {
     const int64_t slots = ks == 1 ? pairs : fused_pair_max_clusters(ks);
     const int64_t nk = (kdim / 64 + ks - 1) / ks;
@@ -344,7 +349,7 @@ PairTile pair_tile(int64_t rows, int64_t kdim, int64_t T, int pairs, bool codes,
                             : bt <= 256 ? (dx ? 538 + bt * 60 / 100 : 513 + bt * 36 / 100)
                                         : (dx ? 749 + (bt - 288) * 183 / 100 : 655 + (bt - 288) * 214 / 100);
       const int64_t cost = rounds * (nk * stage + 2500 + 10 * bt + (ks > 1 ? 2500 + 8 * bt : 0));
-      if (best_cost < 0 || cost < best_cost) {
+      if (best_cost < 0 || (beyond_l2 ? 8 * cost < 7 * best_cost : cost < best_cost)) {
         best_cost = cost;
         best = bt <= 256 ? PairTile{bt, 1, ks, cost} : PairTile{bt / 2, 2, ks, cost};
       }
