@@ -27,7 +27,11 @@ namespace cg = cooperative_groups;
 // (20 us while every thread still added its four sums in doubles).
 constexpr int kNormThreads = 1024;
 constexpr int kNormCluster = 16;         // CTAs; 8 (the portable size) where 16 cannot be resident
-constexpr float kNormBig = 1.1529215e18f;    // 2^60: squares and their sums stay finite below it
+// 2^48: sums of squares of values up to it stay finite.  A warp adds 128 squares per item of its
+// threads before it goes to doubles, and 128 x items x 2^96 < 2^127 up to 2^24 items per thread, which would be
+// 2^39 gradients on eight CTAs.  (With 2^60 the warps' sums left fp32 from about 2^58 on, and the
+// two-sum then makes inf - inf: a NaN norm, which AdamW does not clip by.)
+constexpr float kNormBig = 2.8147498e14f;
 constexpr float kNormSmall = 9.094947e-13f;  // 2^-40: the squares' rounding errors stay normal above it
 
 // hi + lo += x^2, exactly up to the rounding of lo.
