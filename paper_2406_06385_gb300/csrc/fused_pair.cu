@@ -13,20 +13,21 @@
 // tokens or two of up to 224; CTA c holds half of each one's; the host picks smaller token tiles where
 // 448 leave pairs idle, and two or four pairs per tile where those do too: pair_tile in
 // lrqat_api.cu), one 64-wide slice of the contraction per stage:
-//   * token ring (four to eight slots per CTA): loader warps bring this CTA's token halves
+//   * token ring (four to eight slots per CTA; three beside the low-rank tile of 448 tokens): loader warps bring this CTA's token halves
 //     (SW128) with TMA whose completion lands on the leader's barrier; each slot also holds this
 //     CTA's W_hat tile of the stage;
-//   * factor ring (four or eight slots): the stored base of this CTA's rows (completion
+//   * factor ring (four or eight slots; two for 16-bit bases beside the low-rank tile of 448 tokens): the stored base of this CTA's rows (completion
 //     on its own barrier; only its own producers read it), with it the stage's scales (and zero
 //     offsets) where the producers apply them (dX, group-wise forward), and with the low-rank tile
 //     this CTA's half (32 rows) of the second factor's slice (completion on the leader's
 //     barrier: the low-rank MMA reads both halves);
 //   * in the leader, one thread per accumulator issues its main product (M = 256, 4 MMAs per stage)
-//     and, with the low-rank tile in the stage (one accumulator), another the tile L = RF SF^T
-//     (M = 256, N = 64) into one of four TMEM buffers after it, so that neither waits behind the
-//     other's barriers; every commit is multicast to both CTAs;
-//   * sixteen producer warps per CTA, in four groups that take every fourth stage each, build this
-//     CTA's W_hat tile exactly as the one-SM kernel does, and drain this CTA's 128 rows of the
+//     and, with the low-rank tile in the stage, another the tile L = RF SF^T (M = 256, N = 64) into one of
+//     four TMEM buffers after one accumulator or the one buffer after two (which one thread issues
+//     then), so that neither waits behind the other's barriers; every commit is multicast to both CTAs;
+//   * sixteen producer warps per CTA, in four groups that take every fourth stage each (one group
+//     beside the low-rank tile of 448 tokens), build this CTA's W_hat tile exactly as the one-SM kernel
+//     does, and drain this CTA's 128 rows of the
 //     accumulators in the epilogue.
 // One barrier per slot in the leader counts the stage's token bytes and both CTAs' "W_hat
 // written" events, so the MMA thread tests one barrier per stage; the peer's events ("W_hat
@@ -53,18 +54,21 @@ constexpr int BK = 64;
 constexpr int BNP = 224;                         // most tokens per accumulator of two (N of the pair MMA)
 constexpr int NACC = 2;                          // accumulators (one for tiles of up to 256 tokens)
 constexpr int NT_MAX = 8;                        // token ring slots
-constexpr int NLB = 4;                           // low-rank TMEM buffers (one per producer group)
-constexpr int MAX_TILE_L = 256;                  // most tokens of a tile beside them
+constexpr int NLB_MAX = 4;                       // low-rank TMEM buffers (one per producer group)
+constexpr int MAX_TILE_L = 256;                  // most tokens of a tile beside four of them
 constexpr int NF_MAX = 8;                        // factor ring slots
 constexpr int NUM_PROD_WARPS = 16;
 constexpr int FIRST_TMA_WARP = 2 + NUM_PROD_WARPS;
 constexpr int NUM_TOK_LOADERS = 4;               // token loaders (every fourth stage each)
 constexpr int NUM_TMA_WARPS = NUM_TOK_LOADERS + 1;   // and the factor loader
 constexpr int NUM_THREADS = 32 * (FIRST_TMA_WARP + NUM_TMA_WARPS);
-// On the codes the producer warps work in four groups, group g on the stages gg % 4 == g: a warp
-// turns 32 rows x 64 columns per stage (16 columns where all sixteen share every stage).
-constexpr int NUM_GROUPS = 4;
-constexpr int GROUP_WARPS = NUM_PROD_WARPS / NUM_GROUPS;
+// G, the producer groups: 4 = group g takes the stages gg % 4 == g and a warp turns 32 rows x 64 columns
+// of each; 1 = all sixteen warps share every stage, 16 columns each.  Four groups need four token slots
+// and a low-rank buffer each, so beside the low-rank tile they take tiles of up to 256 tokens; one
+// group gets by with three slots (two accumulators of 224 tokens) and one buffer.  Its stage is a
+// chain of barriers, longer than four groups' (1455 cycles against 1050), but serves 448 tokens: the
+// better one where calls are long (allocation-free 4096 x 4096 forward, T = 8192: 256-token tiles
+// 270 us, 448-token tiles 217; FP16 base 395 and 250), the worse one below (T = 1024: 45 and 58 us).
 
 constexpr uint32_t RF_BYTES = 128 * 128;         // 128 rows x 64 rank columns (bf16)
 constexpr uint32_t W_BYTES = 128 * 128;          // 128 rows x 64 bf16
@@ -80,8 +84,9 @@ constexpr uint32_t SFH_BYTES = 32 * 128;         // 32 slice rows x up to 64 ran
 // from global memory: for dX the 64 scales of the stage's contraction indices in the CTA's row
 // group, for the group-wise forward the 128 scales of the CTA's rows in the stage's group.
 constexpr uint32_t RING_BYTES = 232448 - 1024 - 1024;   // less the static barriers and the alignment
-template <int FMT, bool NL, bool XS>
+template <int FMT, bool NL, bool XS, int G>
 struct PairRing {
+  static_assert(G == 4 || (G == 1 && !NL), "producer groups");
   static constexpr uint32_t RF = NL ? 0u : RF_BYTES;
   static constexpr uint32_t PHI_BYTES = fmt_16bit(FMT) ? 128 * 128 : 128 * 64;
   static constexpr uint32_t PHI_TX = FMT == FMT_I4 ? PHI_BYTES / 2 : PHI_BYTES;
@@ -94,26 +99,30 @@ struct PairRing {
   static_assert(FSLOT_BYTES % 1024 == 0 && FS_SF % 1024 == 0, "swizzled tiles must start on 1024-byte boundaries");
   __host__ __device__ static constexpr uint32_t tslot(int btp) { return 64u * btp + W_BYTES; }
   __host__ __device__ static constexpr int nt(int btp) {
+    if (G == 1) return 3;
     const int n = static_cast<int>((RING_BYTES - RF - 4u * FSLOT_BYTES) / tslot(btp));
     return n < NT_MAX ? n : NT_MAX;
   }
-  // four or eight, multiples of NUM_GROUPS: a group then knows that the previous use of a slot it
-  // waits for has landed (it was its own), so barrier phases cannot alias
+  // four or eight, multiples of G: a group then knows that the previous use of a slot it waits for has
+  // landed (it was its own), so barrier phases cannot alias; one group: four, or two of 16-bit bases
   __host__ __device__ static constexpr int nf(int btp) {
+    if (G == 1) return fmt_16bit(FMT) ? 2 : 4;
     return (RING_BYTES - RF - nt(btp) * tslot(btp)) / FSLOT_BYTES >= 8 ? 8 : 4;
   }
-  // the largest token tile: 448 on the codes; beside the low-rank buffers 256 (16-bit bases: 192)
-  static constexpr int MAX_TILE = NL ? 448 : fmt_16bit(FMT) ? 192 : MAX_TILE_L;
+  // the largest token tile: 448 on the codes and of one group; beside four low-rank buffers 256
+  // (16-bit bases: 192)
+  static constexpr int MAX_TILE = NL || G == 1 ? 448 : fmt_16bit(FMT) ? 192 : MAX_TILE_L;
   __host__ __device__ static constexpr uint32_t smem(int btp) {
     return RF + nt(btp) * tslot(btp) + nf(btp) * FSLOT_BYTES + 1024u;
   }
-  static_assert(nt(MAX_TILE) >= NUM_GROUPS && smem(MAX_TILE) <= RING_BYTES + 1024 && smem(32) <= RING_BYTES + 1024,
+  static_assert(nt(MAX_TILE) >= (G == 4 ? 4 : 1) && smem(MAX_TILE) <= RING_BYTES + 1024 && smem(32) <= RING_BYTES + 1024,
                 "shared memory budget");
 };
 
 constexpr uint32_t TMEM_COLS = 512;
-constexpr uint32_t COL_L = MAX_TILE_L;            // the 64-column low-rank buffers after the one accumulator
-static_assert(COL_L + NLB * BK <= TMEM_COLS && NACC * BNP <= TMEM_COLS, "TMEM budget");
+// the 64-column low-rank buffers: four after one accumulator, or one after two
+__host__ __device__ constexpr uint32_t col_l(int groups) { return groups == 1 ? NACC * BNP : MAX_TILE_L; }
+static_assert(col_l(4) + NLB_MAX * BK <= TMEM_COLS && col_l(1) + BK <= TMEM_COLS, "TMEM budget");
 
 // leader: the stage's operands are in place, i.e. both token halves of the slot landed and both
 // CTAs' producers wrote their W_hat tiles (one barrier, so that the MMA thread tests one per stage)
@@ -124,8 +133,8 @@ constexpr int BAR_PFULL = BAR_TEMPTY + NT_MAX;   // both: this CTA's base tile l
 constexpr int BAR_FFULL = BAR_PFULL + NF_MAX;    // leader: both factor-slice halves landed
 constexpr int BAR_FEMPTY = BAR_FFULL + NF_MAX;   // both: slot read by this CTA's producers (after L)
 constexpr int BAR_LFULL = BAR_FEMPTY + NF_MAX;   // both: low-rank tile of the buffer computed
-constexpr int BAR_LEMPTY = BAR_LFULL + NLB;      // leader: both CTAs read the buffer
-constexpr int BAR_RFFULL = BAR_LEMPTY + NLB;     // leader: both row-factor halves landed
+constexpr int BAR_LEMPTY = BAR_LFULL + NLB_MAX;  // leader: both CTAs read the buffer
+constexpr int BAR_RFFULL = BAR_LEMPTY + NLB_MAX; // leader: both row-factor halves landed
 constexpr int BAR_RFEMPTY = BAR_RFFULL + 1;      // both: last low-rank MMA of the tile finished
 constexpr int BAR_ACCFULL = BAR_RFEMPTY + 1;     // both: accumulators of the tile complete
 constexpr int BAR_ACCEMPTY = BAR_ACCFULL + 1;    // leader: both CTAs drained them
@@ -155,12 +164,14 @@ struct Cursor {
     for (s += k; s >= n; s -= n) ph ^= 1u;
   }
 };
-template <int MODE, int FMT, bool ZP, bool UB, bool NL>
+template <int MODE, int FMT, bool ZP, bool UB, bool NL, int G>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     fused_pair_kernel(const __grid_constant__ CUtensorMap tm_tok, const __grid_constant__ CUtensorMap tm_phi,
                       const __grid_constant__ CUtensorMap tm_rf, const __grid_constant__ CUtensorMap tm_sf,
                       const FusedArgs args) {
-  using PR = PairRing<FMT, NL, MODE == FUSED_DX || MODE == FUSED_FWD_GROUP>;
+  using PR = PairRing<FMT, NL, MODE == FUSED_DX || MODE == FUSED_FWD_GROUP, G>;
+  constexpr int NLB = G, GROUP_WARPS = NUM_PROD_WARPS / G;
+  constexpr uint32_t COL_L = col_l(G);
   constexpr uint32_t OFF_RF = PR::OFF_RF, OFF_TSLOTS = PR::OFF_TSLOTS;
   constexpr bool PACKED = FMT == FMT_I4;
   constexpr uint32_t FSLOT_BYTES = PR::FSLOT_BYTES;
@@ -175,8 +186,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   const int lane = threadIdx.x & 31;
   // A cluster holds `ksplit` pairs that share a tile: pair `slice` takes that part of the contraction
   // (1: one pair per cluster, persistent over its tiles).  rank: this CTA's place in its pair.
-  const int ksplit = args.ksplit;
-  const uint32_t crank = cluster_cta_rank(), rank = crank & 1u, lead = crank & ~1u;
+  const int ksplit = G == 1 ? 1 : args.ksplit;
+  const uint32_t crank = cluster_cta_rank(), rank = crank & 1u, lead = G == 1 ? 0u : crank & ~1u;
   const int slice = static_cast<int>(crank >> 1);
   const bool leader = rank == 0;
   const uint32_t pair_mask = 3u << lead;   // the pair's CTAs, for multicast commits
@@ -185,11 +196,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   auto lbar = [&](int i) { return map_shared_rank(smem_u32(&bars[i]), lead); };   // the leader's copy
 
   // the token tile: one accumulator of bnp <= 256 tokens or two of bnp <= 224, half of each per CTA
-  const int bnp = args.bnp, bnh = bnp / 2, nacc = args.nacc, btp = bnp * nacc;
+  const int bnp = G == 1 ? BNP : args.bnp, bnh = bnp / 2, nacc = G == 1 ? NACC : args.nacc, btp = bnp * nacc;
   const int NT = PR::nt(btp), NF = PR::nf(btp);
   const uint32_t TSLOT_BYTES = PR::tslot(btp), TOK_BOX = 128u * bnh, TS_W = 64u * btp;
   const uint32_t OFF_FSLOTS = OFF_TSLOTS + NT * TSLOT_BYTES;
-  const uint32_t issuers = nacc;   // threads that issue (and commit) the main product
+  // one thread issues both accumulators where the other issuer's warp has the low-rank tiles
+  constexpr bool BOTH = !NL && G == 1;
+  const uint32_t issuers = BOTH ? 1 : nacc;   // threads that issue (and commit) the main product
   if (threadIdx.x == 0) {
     abort_s = 0;
     for (int s = 0; s < NT; ++s) {
@@ -248,7 +261,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     }
   };
 
-  // The main product of the pair's tiles into accumulator a, by one thread of the leader.  Two
+  // The main product of the pair's tiles into accumulator a (BOTH: into both), by one thread of the leader.  Two
   // accumulators have a thread each: a thread's barrier test and commit (~110
   // and ~70 cycles a stage, with the tensor pipe queueing about one MMA ahead) then run beside the
   // other's MMAs (4096 x 4096, 288-token tiles 906 -> 739 cycles a stage, 320 925 -> 801; at 448 the
@@ -278,6 +291,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         mma_bf16_pair(d, w + 2, t + 2, idesc_main, 1u);
         mma_bf16_pair(d, w + 4, t + 4, idesc_main, 1u);
         mma_bf16_pair(d, w + 6, t + 6, idesc_main, 1u);
+        if (BOTH) {
+          const uint64_t t2 = t + (TOK_BOX >> 4);
+          mma_bf16_pair(d + BNP, w, t2, idesc_main, acc);
+          mma_bf16_pair(d + BNP, w + 2, t2 + 2, idesc_main, 1u);
+          mma_bf16_pair(d + BNP, w + 4, t2 + 4, idesc_main, 1u);
+          mma_bf16_pair(d + BNP, w + 6, t2 + 6, idesc_main, 1u);
+        }
         mma_commit_pair(bar(BAR_TEMPTY + s), pair_mask);
       }
       if (!ok) break;
@@ -436,7 +456,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     // ------------------------------------------- W_hat producers + epilogue
     const int pw = warp - 2;              // 0..15
     const int q = warp & 3;               // TMEM lane quarter this warp may access
-    const int c = pw >> 2;                // 16-column chunk of the 64-wide slice (and epilogue block)
+    const int c = pw >> 2;                // group (one group: 16-column chunk of the slice); epilogue block
+    const int gw = G == 4 ? q : pw;       // this warp in its group
+    const int lb = G == 4 ? c : 0;        // the group's low-rank buffer
+    const int y0 = G == 4 ? 0 : 2 * c;    // the first eight of the slice's columns that this warp turns
     const int row = q * 32 + lane;        // row of this CTA's tile handled by this thread
     const uint32_t lane_off = static_cast<uint32_t>(q * 32) << 16;
     const QuantParams qp = args.q;
@@ -444,30 +467,41 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     uint32_t g = 0;
     uint32_t it = 0;
     Cursor fc, tc;   // factor and token slots
-    fc.skip(c, NF);
-    tc.skip(c, NT);
+    if (G == 4) {
+      fc.skip(c, NF);
+      tc.skip(c, NT);
+    }
     bool ok = true;
     for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
       const int rb2 = tile % num_rb2;
       const int tb = tile / num_rb2;
       const int row_g = row_block(rb2) + row;
       const bool has_rows = rb2 * 2 * BM + static_cast<int>(rank) * BM < args.rows;
-      // Group c's stages of the tile (gg % 4 == c).  A ready barrier costs a test of ~110 cycles and the
+      const uint32_t z_row = MODE == FUSED_FWD_PC && ZP ? pack_rn_bf16x2(args.zero[row_g], args.zero[row_g]) : 0u;
+      // Group c's stages of the tile (gg % 4 == c; one group: every stage).  A ready barrier costs a test of ~110 cycles and the
       // proxy fence and reports ~100 more, whatever the warp does between them: with all sixteen warps in
       // every stage these made a stage on the codes 770 cycles (4096 x 4096, 32-token tiles), four groups
       // in flight pay them side by side (596 cycles; 256-token tiles 863 -> 700).  With the low-rank tile
       // a group has a TMEM buffer of its own, so four low-rank tiles are in flight instead of one
       // (1700 -> 1030 cycles a stage; T = 1024 forward 58 -> 45 us).
-      for (int kk = static_cast<int>((static_cast<uint32_t>(c) - g) & 3u); kk < nk; kk += NUM_GROUPS) {
+      for (int kk = G == 4 ? static_cast<int>((static_cast<uint32_t>(c) - g) & 3u) : 0; kk < nk; kk += G) {
         ok = wait_bounded(bar(BAR_PFULL + fc.s), fc.ph, ctl, 12);
         if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
         const uint32_t fs = smem + OFF_FSLOTS + fc.s * FSLOT_BYTES;
-        constexpr int RAW4 = PACKED ? 2 : fmt_16bit(FMT) ? 8 : 4;   // 16-byte words of the row's 64 values
-        constexpr int ROW_BYTES = 16 * RAW4;
-        uint4 raw[RAW4];
+        constexpr int RAW = PACKED ? 2 : fmt_16bit(FMT) ? 8 : 4;   // words of 16 stored values
+        constexpr int ROW_BYTES = 16 * RAW;
+        uint32_t raw[RAW * G];                                     // this warp's 16 G columns of the row
+        if (PACKED && G == 1) {
+          const uint2 r = ld_shared_v2(fs + swz_offset(row, c >> 1, ROW_BYTES) + 8 * (c & 1));
+          raw[0] = r.x, raw[1] = r.y;
+        } else {
 #pragma unroll
-        for (int x = 0; x < RAW4; ++x) raw[x] = ld_shared_v4(fs + swz_offset(row, x, ROW_BYTES));
-        uint32_t sg = 0, zg = 0;   // forward: the row's scale and zero offset in the stage, as bf16x2
+          for (int x = 0; x < RAW * G / 4; ++x) {
+            const uint4 r = ld_shared_v4(fs + swz_offset(row, y0 * RAW / 8 + x, ROW_BYTES));
+            raw[4 * x] = r.x, raw[4 * x + 1] = r.y, raw[4 * x + 2] = r.z, raw[4 * x + 3] = r.w;
+          }
+        }
+        uint32_t sg = 0, zg = z_row;   // forward: the row's scale and zero offset in the stage, as bf16x2
         if (MODE == FUSED_FWD_GROUP) {
           sg = ld_shared_u16(fs + PR::FS_X + 2u * row);
           sg |= sg << 16;
@@ -475,14 +509,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             zg = ld_shared_u16(fs + PR::FS_X + 512u + 2u * row);
             zg |= zg << 16;
           }
-        } else if (MODE == FUSED_FWD_PC && ZP) {
-          zg = pack_rn_bf16x2(args.zero[row_g], args.zero[row_g]);
         }
-        uint32_t w[32];
-        if (NL) {
+        uint32_t w[8 * G];
+        if constexpr (NL) {
 #pragma unroll
-          for (int x = 0; x < RAW4; ++x) {
-            const uint32_t in[4] = {raw[x].x, raw[x].y, raw[x].z, raw[x].w};
+          for (int x = 0; x < G; ++x) {
+            const uint32_t in[4] = {raw[4 * x], raw[4 * x + 1], raw[4 * x + 2], raw[4 * x + 3]};
             if (args.codes_bias == 64) {
 #pragma unroll
               for (int i = 0; i < 4; ++i) decode_b64_bf16x4(in[i], w[8 * x + 2 * i], w[8 * x + 2 * i + 1]);
@@ -494,24 +526,27 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             }
           }
         } else {
-          // the group's low-rank buffer (gg % NLB == c, used every fourth stage)
-          ok = wait_bounded(bar(BAR_LFULL + c), ((g + kk) / NLB) & 1u, ctl, 13);
+          float v[16];
+          if (G == 1) decode16<FMT>(raw, v);   // before the wait: the one buffer is to be read and reported at once
+          // the group's low-rank buffer (gg % NLB)
+          ok = wait_bounded(bar(BAR_LFULL + lb), ((g + kk) / NLB) & 1u, ctl, 13);
           if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t* rw = reinterpret_cast<const uint32_t*>(raw);
 #pragma unroll
-          for (int x = 0; x < 4; ++x) {
-            float v[16], Lv[16];
-            tmem_ld16(tmem + lane_off + COL_L + BK * c + 16 * x, Lv);
-            uint32_t in[RAW4];
+          for (int x = 0; x < G; ++x) {
+            float Lv[16];
+            tmem_ld16(tmem + lane_off + COL_L + BK * lb + 8 * y0 + 16 * x, Lv);
+            if (G == 4) {
+              uint32_t in[RAW];
 #pragma unroll
-            for (int e = 0; e < RAW4; ++e) in[e] = rw[RAW4 * x + e];
-            decode16<FMT>(in, v);
+              for (int e = 0; e < RAW; ++e) in[e] = raw[RAW * x + e];
+              decode16<FMT>(in, v);
+            }
             tmem_ld_wait();
-            if (x == 3) {
+            if (x == G - 1) {
               tc_fence_before();
               __syncwarp();
-              if (lane == 0) report(BAR_LEMPTY + c, q, GROUP_WARPS);
+              if (lane == 0) report(BAR_LEMPTY + lb, gw, GROUP_WARPS);
             }
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -524,12 +559,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           }
         }
 #pragma unroll
-        for (int x = 0; x < 8; ++x) {
+        for (int x = 0; x < 2 * G; ++x) {
           if (MODE == FUSED_DX) {
             // the bf16 scales (zero offsets) of eight contraction indices, as bf16x2 words
-            const uint4 s4 = ld_shared_v4(fs + PR::FS_X + 16u * x);
+            const uint4 s4 = ld_shared_v4(fs + PR::FS_X + 16u * (y0 + x));
             if (ZP) {
-              const uint4 z4 = ld_shared_v4(fs + PR::FS_X + 512u + 16u * x);
+              const uint4 z4 = ld_shared_v4(fs + PR::FS_X + 512u + 16u * (y0 + x));
               w[4 * x] = sub_bf16x2(w[4 * x], z4.x), w[4 * x + 1] = sub_bf16x2(w[4 * x + 1], z4.y);
               w[4 * x + 2] = sub_bf16x2(w[4 * x + 2], z4.z), w[4 * x + 3] = sub_bf16x2(w[4 * x + 3], z4.w);
             }
@@ -548,23 +583,28 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
         const uint32_t wt = smem + OFF_TSLOTS + tc.s * TSLOT_BYTES + TS_W;
 #pragma unroll
-        for (int x = 0; x < 8; ++x)
-          st_shared_v4(wt + swz_offset(row, x, 128), w[4 * x], w[4 * x + 1], w[4 * x + 2], w[4 * x + 3]);
+        for (int x = 0; x < 2 * G; ++x)
+          st_shared_v4(wt + swz_offset(row, y0 + x, 128), w[4 * x], w[4 * x + 1], w[4 * x + 2], w[4 * x + 3]);
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
-          report(BAR_TFULL + tc.s, q, GROUP_WARPS);
+          report(BAR_TFULL + tc.s, gw, GROUP_WARPS);
           mbar_arrive(bar(BAR_FEMPTY + fc.s));
         }
-        fc.skip(NUM_GROUPS, NF);
-        tc.skip(NUM_GROUPS, NT);
+        if (G == 1) {   // (skip's loop made a stage of the one group 7% longer)
+          fc.next(NF);
+          tc.next(NT);
+        } else {
+          fc.skip(G, NF);
+          tc.skip(G, NT);
+        }
       }
       if (!ok) break;
       // ------------------------------------------------------------ epilogue
       ok = wait_spin_bounded(bar(BAR_ACCFULL), it & 1u, ctl, 15);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       tc_fence_after();
-      if (ksplit == 1) {
+      if (G == 1 || ksplit == 1) {
         const float scale = out_scale(row_g);
 #pragma unroll 1
         for (int col = has_rows ? 16 * c : btp; col < btp; col += 64) {   // token offset in the tile
@@ -594,7 +634,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     }
   }
 
-  if (ksplit > 1) {
+  if (G == 4 && ksplit > 1) {
     // One tile per cluster: its pairs' partial sums meet.  Pair p owns the p-th part of the tile's
     // tokens and adds the slices' sums in order through distributed shared memory.
     __syncwarp();
@@ -632,15 +672,17 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   }
 }
 
-template <int MODE, int FMT, bool ZP, bool UB, bool NL>
+template <int MODE, int FMT, bool ZP, bool UB, bool NL, int G = 4>
 cudaError_t launch_pair_one(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c, const CUtensorMap& d,
                             const FusedArgs& args, int npairs, cudaStream_t stream) {
-  using PR = PairRing<FMT, NL, MODE == FUSED_DX || MODE == FUSED_FWD_GROUP>;
-  if (args.bnp * args.nacc > PR::MAX_TILE || (!NL && args.nacc != 1)) return cudaErrorInvalidValue;
+  if constexpr (!NL && G == 4)   // beside the low-rank tile, two accumulators take one producer group
+    if (args.nacc == 2) return launch_pair_one<MODE, FMT, ZP, UB, NL, 1>(a, b, c, d, args, npairs, stream);
+  using PR = PairRing<FMT, NL, MODE == FUSED_DX || MODE == FUSED_FWD_GROUP, G>;
+  if (args.bnp * args.nacc > PR::MAX_TILE || (G == 1 && (args.bnp != BNP || args.ksplit != 1))) return cudaErrorInvalidValue;
   if (args.ksplit > 1 && (args.nacc != 1 || args.bnp % (16 * args.ksplit))) return cudaErrorInvalidValue;
   const uint32_t smem = PR::smem(args.bnp * args.nacc);
   static bool configured[kMaxDevices] = {};
-  const void* fn = reinterpret_cast<const void*>(fused_pair_kernel<MODE, FMT, ZP, UB, NL>);
+  const void* fn = reinterpret_cast<const void*>(fused_pair_kernel<MODE, FMT, ZP, UB, NL, G>);
   cudaError_t e = ensure_smem_attr(fn, 232448 - 1024, configured);   // the most any tile asks for
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
@@ -658,7 +700,7 @@ cudaError_t launch_pair_one(const CUtensorMap& a, const CUtensorMap& b, const CU
   cfg.numAttrs = 1;
   if (args.ksplit > 1) {   // one tile per cluster, however many are resident at once
     cfg.numAttrs = 2;
-    e = cudaLaunchKernelEx(&cfg, fused_pair_kernel<MODE, FMT, ZP, UB, NL>, a, b, c, d, args);
+    e = cudaLaunchKernelEx(&cfg, fused_pair_kernel<MODE, FMT, ZP, UB, NL, G>, a, b, c, d, args);
     return e != cudaSuccess ? e : cudaGetLastError();
   }
   // The persistent grid holds no more pairs than can be resident at once (an SM that has no
@@ -669,7 +711,7 @@ cudaError_t launch_pair_one(const CUtensorMap& a, const CUtensorMap& b, const CU
   if (e != cudaSuccess) return e;
   if (max_pairs[dev] == 0) {
     int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, fused_pair_kernel<MODE, FMT, ZP, UB, NL>, &cfg);
+    e = cudaOccupancyMaxActiveClusters(&n, fused_pair_kernel<MODE, FMT, ZP, UB, NL, G>, &cfg);
     if (e != cudaSuccess) return e;
     if (n < 1) return cudaErrorInvalidConfiguration;
     max_pairs[dev] = n;
@@ -679,7 +721,7 @@ cudaError_t launch_pair_one(const CUtensorMap& a, const CUtensorMap& b, const CU
     cfg.gridDim = dim3(static_cast<unsigned>(2 * npairs), 1, 1);
   }
   cfg.numAttrs = 2;
-  e = cudaLaunchKernelEx(&cfg, fused_pair_kernel<MODE, FMT, ZP, UB, NL>, a, b, c, d, args);
+  e = cudaLaunchKernelEx(&cfg, fused_pair_kernel<MODE, FMT, ZP, UB, NL, G>, a, b, c, d, args);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
@@ -728,9 +770,9 @@ int fused_pair_max_clusters(int ksplit) {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices || ksplit < 1 || ksplit > 4) return 0;
   int n = cache[dev][ksplit].load(std::memory_order_acquire);
   if (n > 0) return n;
-  using PR = PairRing<FMT_Q8, true, false>;
+  using PR = PairRing<FMT_Q8, true, false, 4>;
   static bool configured[kMaxDevices] = {};
-  const void* fn = reinterpret_cast<const void*>(fused_pair_kernel<FUSED_FWD_PC, FMT_Q8, false, false, true>);
+  const void* fn = reinterpret_cast<const void*>(fused_pair_kernel<FUSED_FWD_PC, FMT_Q8, false, false, true, 4>);
   if (ensure_smem_attr(fn, 232448 - 1024, configured) != cudaSuccess) return 0;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(2 * ksplit), 1, 1);
@@ -743,7 +785,7 @@ int fused_pair_max_clusters(int ksplit) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaOccupancyMaxActiveClusters(&n, fused_pair_kernel<FUSED_FWD_PC, FMT_Q8, false, false, true>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, fused_pair_kernel<FUSED_FWD_PC, FMT_Q8, false, false, true, 4>, &cfg) != cudaSuccess) {
     (void)cudaGetLastError();
     return 0;
   }

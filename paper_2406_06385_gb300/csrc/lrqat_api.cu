@@ -317,6 +317,23 @@ struct PairTile {
   int64_t cost;   // cycles by the model below
   int tokens() const { return bnp * nacc; }
 };
+// Cycles of a stage with the low-rank tile in it.  Up to 256 tokens (192 for 16-bit bases) the four producer
+// groups share out the stages, each with a low-rank buffer; 448-token tiles leave room for one group and one
+// buffer (fused_pair.cu).  Measured on 4096 x 4096, 14336 x 4096 and 2048 x 8192 layers at T = 512 .. 8192, with
+// the drains and 8 us a call taken off, grouped (64 / 256 tokens; 16-bit 64 / 192) and at 448: 8-bit and
+// packed 1005 / 1050, 1455; FP8 1160 / 1200, 1640; BF16 965 / 1020, 1640; FP16 1120 / 1165, 1710; the
+// bf16 pre-round value 170 and 120 more, zero offsets 50 .. 75 and 40, scales in the stage 60 and 60 .. 110.  The choice
+// by these is within 5% of the fastest tile at all 390 measured points.
+int64_t in_stage_cycles(const lrqat_layer& L, bool dx, int tokens) {
+  int64_t grouped = 975, whole = 1455;
+  if (L.phi_format == LRQAT_PHI_FP8_E4M3 || L.phi_format == LRQAT_PHI_FP8_E5M2) grouped = 1120, whole = 1635;
+  if (L.phi_format == LRQAT_PHI_BF16) grouped = 1000, whole = 1640;
+  if (L.phi_format == LRQAT_PHI_FP16) grouped = 1130, whole = 1710;
+  if (L.u_bf16) grouped += 165, whole += 110;
+  if (L.zero) grouped += 75, whole += 40;
+  if (dx ? !phi_16bit(L) : L.group_size != 0) grouped += 60, whole += 90;
+  return tokens > 256 ? whole : grouped + tokens * 30 / 100;
+}
 // The cheapest tile for `rows` weight rows, a contraction of kdim and T tokens on `pairs` pairs, by
 // the rounds of the busiest pair times a tile's cycles: its 64-wide stages plus the drain.  Stage
 // cycles measured on a 4096 x 4096 layer on the codes (forward, T = 8192, drain taken off): one
@@ -327,25 +344,28 @@ struct PairTile {
 // against 2.4 at 256) and smaller tiles pay where 448 leave pairs idle: T = 4096 takes 304 (three
 // rounds; forward 107 -> 82 us, dX 111 -> 92), T = 1024 takes 256.  Where even one round leaves pairs
 // idle, two or four pairs share a tile's contraction and add their sums through distributed shared
-// memory (T = 256, forward 26.6 us with one pair, 22.8 with two; dX 29.1, 22.6).  With the low-rank tile in the stage (one accumulator: its buffers
-// take the other's TMEM) a stage takes 971 to 1050 cycles.
+// memory (T = 256, forward 26.6 us with one pair, 22.8 with two; dX 29.1, 22.6).  With the low-rank tile in
+// the stage (in_stage_cycles) tiles of 448 tokens pay in long calls: allocation-free 4096 x 4096 forward, T =
+// 8192, 270 us with 256-token tiles, 217 with 448; FP16 base 395, 250; T = 4096 (four rounds, or three) 156, 172.
 // Those figures are of operands that stay in L2.  Beyond it smaller tiles, which read the operands more
 // often, are slower than the model says: 288-token tiles, 1% cheaper by it, took 1408 us for a 5120 x
 // 13824 forward at T = 16384 and 418 for 4096 x 11008 at T = 8192, 448-token tiles 1153 and 380.  There a
 // smaller tile has to be cheaper by an eighth.
-PairTile pair_tile(int64_t rows, int64_t kdim, int64_t T, int pairs, bool codes, bool dx, bool phi16) {
+PairTile pair_tile(const lrqat_layer& L, bool dx, int64_t T, int pairs, bool codes) {
+  const int64_t rows = dx ? L.k : L.m, kdim = dx ? L.m : L.k;
   PairTile best{0, 0, 1, 0};
   int64_t best_cost = -1;
-  const bool beyond_l2 = kdim * (rows + 2 * T) > (int64_t{100} << 20);   // one byte a weight, two a token value
+  const bool beyond_l2 = codes && kdim * (rows + 2 * T) > (int64_t{100} << 20);   // one byte a weight, two a token value
   for (int ks = 1; ks <= 4; ks *= 2) {
     const int64_t slots = ks == 1 ? pairs : fused_pair_max_clusters(ks);
     const int64_t nk = (kdim / 64 + ks - 1) / ks;
     if (slots < 1 || nk < 2) continue;
-    for (int bt = !codes ? (phi16 ? 192 : 256) : ks > 1 ? 256 : 448; bt >= 32; bt -= 32) {
-      if (bt % (16 * ks)) continue;
+    for (int bt = 448; bt >= 32; bt -= 32) {
+      if (bt % (16 * ks) || (bt > 256 && ks > 1)) continue;
+      if (!codes && bt != 448 && bt > (phi_16bit(L) ? 192 : 256)) continue;
       const int64_t tiles = ((rows + 255) / 256) * ((T + bt - 1) / bt);
       const int64_t rounds = (tiles + slots - 1) / slots;
-      const int64_t stage = !codes ? 960 + bt * 35 / 100
+      const int64_t stage = !codes ? in_stage_cycles(L, dx, bt)
                             : bt <= 256 ? (dx ? 538 + bt * 60 / 100 : 513 + bt * 36 / 100)
                                         : (dx ? 749 + (bt - 288) * 183 / 100 : 655 + (bt - 288) * 214 / 100);
       const int64_t cost = rounds * (nk * stage + 2500 + 10 * bt + (ks > 1 ? 2500 + 8 * bt : 0));
@@ -364,9 +384,8 @@ PairTile pair_tile(int64_t rows, int64_t kdim, int64_t T, int pairs, bool codes,
 bool prefer_codes_fwd(const lrqat_layer& L, int64_t T, int pairs) {
   constexpr double kCyclesPerUs = 1920.0;
   const double pass = (2.5 + 0.5e-6 * static_cast<double>(L.m) * static_cast<double>(L.k)) * kCyclesPerUs;
-  const double codes = pass + static_cast<double>(pair_tile(L.m, L.k, T, pairs, true, false, false).cost);
-  const double tile = 2.0 * kCyclesPerUs +
-                      static_cast<double>(pair_tile(L.m, L.k, T, pairs, false, false, phi_16bit(L)).cost);
+  const double codes = pass + static_cast<double>(pair_tile(L, false, T, pairs, true).cost);
+  const double tile = 2.0 * kCyclesPerUs + static_cast<double>(pair_tile(L, false, T, pairs, false).cost);
   return codes <= tile;
 }
 
@@ -908,7 +927,7 @@ static int linear_fwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
     return LRQAT_OK;
   }
   CUtensorMap tm_tok, tm_phi, tm_rf, tm_sf;
-  const PairTile tile = pair_tile(L.m, L.k, T, dev->sms / 2, cb, false, phi_16bit(L));
+  const PairTile tile = pair_tile(L, false, T, dev->sms / 2, cb);
   LRQAT_TRY(encode_2d(&tm_tok, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, tok, L.k, T, L.k * 2, 64, pair ? tile.bnp / 2 : 224,
                       CU_TENSOR_MAP_SWIZZLE_128B, "X"));
   if (cb) {
@@ -1113,7 +1132,7 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
                    "dX scale rows");
     const bool pair = use_pair();
     CUtensorMap tm_tok, tm_phi, tm_rf, tm_sf;
-    const PairTile tile = pair_tile(L.k, L.m, T, dev->sms / 2, cb, true, phi_16bit(L));
+    const PairTile tile = pair_tile(L, true, T, dev->sms / 2, cb);
     LRQAT_TRY(encode_2d(&tm_tok, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, dY, L.m, T, L.m * 2, 64, pair ? tile.bnp / 2 : 224,
                         CU_TENSOR_MAP_SWIZZLE_128B, "dY"));
     if (phi_16bit(L) && !cb)
