@@ -76,9 +76,14 @@ constexpr uint32_t SFH_BYTES = 32 * 128;         // 32 slice rows x up to 64 ran
 
 // Shared-memory rings.  A token slot holds this CTA's half of the stage's tokens (a tile of btp
 // tokens: 64 btp bytes) and its W_hat tile, a factor slot the stored base and, with the low-rank tile
-// (which also has the row factor resident), this CTA's half of the second factor's slice.  As many
-// token slots as the tile leaves room for beside four factor slots, and eight of these where the
-// rest allows (up to eight of each).
+// (which also has the row factor resident), this CTA's half of the second factor's slice.  On the codes
+// eight factor slots where they leave room for five token slots (tiles up to 256 tokens; dX 224) or, with codes
+// that come from HBM (deep), four, then as many token slots as fit (up to eight); else, and with the low-rank
+// tile, whose stages are twice as long, four factor slots first.  Four slots of a short stage do not
+// cover a fetch from HBM: tiles of 64 to 320 tokens took 1.2 to 1.45 times their stages' cycles (14336 x 4096
+// forward at T = 2048: 256-token tiles 183 us with four factor slots, 134 with eight; 288 190, 150).  Where the
+// codes stay in L2 eight slots beside five token slots are up to 25% faster and at most 3% slower, beside four up
+// to 12% slower (1024 x 14336 at T = 1024, 288 tokens).
 // XS: each factor slot also holds the stage's scales (and zero offsets) as bf16, copied by the
 // factor loader, so that the producers read them from shared memory with the base instead of
 // from global memory: for dX the 64 scales of the stage's contraction indices in the CTA's row
@@ -98,24 +103,26 @@ struct PairRing {
   static constexpr uint32_t OFF_TSLOTS = RF;
   static_assert(FSLOT_BYTES % 1024 == 0 && FS_SF % 1024 == 0, "swizzled tiles must start on 1024-byte boundaries");
   __host__ __device__ static constexpr uint32_t tslot(int btp) { return 64u * btp + W_BYTES; }
-  __host__ __device__ static constexpr int nt(int btp) {
+  __host__ __device__ static constexpr int nt(int btp, bool deep) {
     if (G == 1) return 3;
-    const int n = static_cast<int>((RING_BYTES - RF - 4u * FSLOT_BYTES) / tslot(btp));
+    const int n8 = static_cast<int>((RING_BYTES - RF - 8u * FSLOT_BYTES) / tslot(btp));
+    const int n = NL && n8 >= (deep ? 4 : 5) ? n8 : static_cast<int>((RING_BYTES - RF - 4u * FSLOT_BYTES) / tslot(btp));
     return n < NT_MAX ? n : NT_MAX;
   }
   // four or eight, multiples of G: a group then knows that the previous use of a slot it waits for has
   // landed (it was its own), so barrier phases cannot alias; one group: four, or two of 16-bit bases
-  __host__ __device__ static constexpr int nf(int btp) {
+  __host__ __device__ static constexpr int nf(int btp, bool deep) {
     if (G == 1) return fmt_16bit(FMT) ? 2 : 4;
-    return (RING_BYTES - RF - nt(btp) * tslot(btp)) / FSLOT_BYTES >= 8 ? 8 : 4;
+    return (RING_BYTES - RF - nt(btp, deep) * tslot(btp)) / FSLOT_BYTES >= 8 ? 8 : 4;
   }
   // the largest token tile: 448 on the codes and of one group; beside four low-rank buffers 256
   // (16-bit bases: 192)
   static constexpr int MAX_TILE = NL || G == 1 ? 448 : fmt_16bit(FMT) ? 192 : MAX_TILE_L;
-  __host__ __device__ static constexpr uint32_t smem(int btp) {
-    return RF + nt(btp) * tslot(btp) + nf(btp) * FSLOT_BYTES + 1024u;
+  __host__ __device__ static constexpr uint32_t smem(int btp, bool deep) {
+    return RF + nt(btp, deep) * tslot(btp) + nf(btp, deep) * FSLOT_BYTES + 1024u;
   }
-  static_assert(nt(MAX_TILE) >= (G == 4 ? 4 : 1) && smem(MAX_TILE) <= RING_BYTES + 1024 && smem(32) <= RING_BYTES + 1024,
+  static_assert(nt(MAX_TILE, true) >= (G == 4 ? 4 : 1) && smem(MAX_TILE, true) <= RING_BYTES + 1024 &&
+                    smem(32, true) <= RING_BYTES + 1024,
                 "shared memory budget");
 };
 
@@ -197,7 +204,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 
   // the token tile: one accumulator of bnp <= 256 tokens or two of bnp <= 224, half of each per CTA
   const int bnp = G == 1 ? BNP : args.bnp, bnh = bnp / 2, nacc = G == 1 ? NACC : args.nacc, btp = bnp * nacc;
-  const int NT = PR::nt(btp), NF = PR::nf(btp);
+  const int NT = PR::nt(btp, args.deep), NF = PR::nf(btp, args.deep);
   const uint32_t TSLOT_BYTES = PR::tslot(btp), TOK_BOX = 128u * bnh, TS_W = 64u * btp;
   const uint32_t OFF_FSLOTS = OFF_TSLOTS + NT * TSLOT_BYTES;
   // one thread issues both accumulators where the other issuer's warp has the low-rank tiles
@@ -680,7 +687,7 @@ cudaError_t launch_pair_one(const CUtensorMap& a, const CUtensorMap& b, const CU
   using PR = PairRing<FMT, NL, MODE == FUSED_DX || MODE == FUSED_FWD_GROUP, G>;
   if (args.bnp * args.nacc > PR::MAX_TILE || (G == 1 && (args.bnp != BNP || args.ksplit != 1))) return cudaErrorInvalidValue;
   if (args.ksplit > 1 && (args.nacc != 1 || args.bnp % (16 * args.ksplit))) return cudaErrorInvalidValue;
-  const uint32_t smem = PR::smem(args.bnp * args.nacc);
+  const uint32_t smem = PR::smem(args.bnp * args.nacc, args.deep);
   static bool configured[kMaxDevices] = {};
   const void* fn = reinterpret_cast<const void*>(fused_pair_kernel<MODE, FMT, ZP, UB, NL, G>);
   cudaError_t e = ensure_smem_attr(fn, 232448 - 1024, configured);   // the most any tile asks for
@@ -777,7 +784,7 @@ int fused_pair_max_clusters(int ksplit) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(2 * ksplit), 1, 1);
   cfg.blockDim = dim3(NUM_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = PR::smem(256);
+  cfg.dynamicSmemBytes = PR::smem(256, true);
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = static_cast<unsigned>(2 * ksplit);

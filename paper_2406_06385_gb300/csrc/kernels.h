@@ -192,6 +192,8 @@ struct FusedArgs {
   // Pair kernel: pairs that share a tile, each with a part of the contraction (1, 2 or 4; above 1 with
   // one accumulator, bnp a multiple of 16 ksplit, and a cluster per tile)
   int32_t ksplit;
+  // Pair kernel on the codes: eight factor slots rather than a fifth token slot (the codes come from HBM)
+  int32_t deep;
 };
 // s_out[g][i] = bf16(s[i][g]) (s [m] per channel: g = 0 only) and, with z, z_out likewise: the
 // dX GEMM's producers read 16 consecutive of them per stage with two 16-byte loads.

@@ -334,28 +334,38 @@ int64_t in_stage_cycles(const lrqat_layer& L, bool dx, int tokens) {
   if (dx ? !phi_16bit(L) : L.group_size != 0) grouped += 60, whole += 90;
   return tokens > 256 ? whole : grouped + tokens * 30 / 100;
 }
-// The cheapest tile for `rows` weight rows, a contraction of kdim and T tokens on `pairs` pairs, by
-// the rounds of the busiest pair times a tile's cycles: its 64-wide stages plus the drain.  Stage
-// cycles measured on a 4096 x 4096 layer on the codes (forward, T = 8192, drain taken off): one
-// accumulator 524 (32 tokens) to 605 (256), two 655 (288) to 997 (448), linear in between; dX, whose
-// producers also multiply by the scales, 557 to 692 and 749 to 1042; the drain 2500 + 10 per token.
-// Up to 256 tokens the stage is bound by the issue of four MMAs whatever their N, beyond by the
-// operands' shared-memory traffic, so 448 tokens are the cheapest per token (2.2 cycles a stage
-// against 2.4 at 256) and smaller tiles pay where 448 leave pairs idle: T = 4096 takes 304 (three
-// rounds; forward 107 -> 82 us, dX 111 -> 92), T = 1024 takes 256.  Where even one round leaves pairs
-// idle, two or four pairs share a tile's contraction and add their sums through distributed shared
-// memory (T = 256, forward 26.6 us with one pair, 22.8 with two; dX 29.1, 22.6).  With the low-rank tile in
-// the stage (in_stage_cycles) tiles of 448 tokens pay in long calls: allocation-free 4096 x 4096 forward, T =
-// 8192, 270 us with 256-token tiles, 217 with 448; FP16 base 395, 250; T = 4096 (four rounds, or three) 156, 172.
-// Those figures are of operands that stay in L2.  Beyond it smaller tiles, which read the operands more
-// often, are slower than the model says: 288-token tiles, 1% cheaper by it, took 1408 us for a 5120 x
-// 13824 forward at T = 16384 and 418 for 4096 x 11008 at T = 8192, 448-token tiles 1153 and 380.  There a
-// smaller tile has to be cheaper by an eighth.
+// Codes beyond this (bytes) do not stay in L2 beside the tokens and the outputs (fused_pair.cu, PairRing).
+constexpr int64_t kDeepCodes = int64_t{32} << 20;
+// Cycles of a stage on the codes: medians by token tile (32, 64, .. 448) over fifteen shapes from 4096 x 4096 to
+// 14336 x 14336, T = 64 .. 16384, with the drains and 4 us a call taken off.  Up to 256 tokens the stage is
+// bound by the issue of four MMAs whatever their N, beyond by the operands' shared-memory traffic; dX's
+// producers also multiply by the scales, and its 384-token tiles, the first with room for four factor slots only,
+// wait for codes that come from HBM.  Zero offsets in dX and the scales of the group-wise forward make the
+// producers the bound of smaller tiles.
+int64_t codes_stage_cycles(const lrqat_layer& L, bool dx, int tokens) {
+  constexpr int16_t kFwd[] = {485, 497, 505, 513, 523, 535, 545, 567, 663, 703, 754, 811, 877, 943};
+  constexpr int16_t kDx[] = {520, 531, 543, 554, 562, 566, 576, 639, 678, 720, 771, 883, 909, 966};
+  int64_t cycles = (dx ? kDx : kFwd)[tokens / 32 - 1];
+  if (dx && tokens == 384 && L.m * L.k > kDeepCodes) cycles += 75;
+  const int64_t producers = dx ? (L.zero ? 640 : 0) : L.group_size ? (L.zero ? 800 : 740) : 0;
+  return cycles > producers ? cycles : producers;
+}
+// The cheapest tile of a layer's forward or dX at T tokens on `pairs` pairs, by the rounds of the busiest
+// pair times a tile's cycles: its 64-wide stages plus the drain (2500 + 10 per token).  448 tokens are the
+// cheapest per token (2.1 cycles a stage against 2.2 at 256) and smaller tiles pay where 448 leave pairs
+// idle: 4096 x 4096 at T = 4096 takes 288 (three rounds; forward 107 -> 82 us, dX 111 -> 92), T = 1024 takes 256.
+// A forward's codes from HBM are read once per token tile, which decides near-ties (14336 x 4096 at T = 16384: 979 us
+// with 448 tokens, 1034 with 384, 1% cheaper by their cycles).  So the choice on the codes is within 3% of the
+// fastest of twelve tiles at 296 of 298 measured points, 8% at all.
+// Where one round leaves pairs idle, two or four pairs share a tile's contraction and add their sums through
+// distributed shared memory (T = 256, forward 26.6 us with one pair, 22.8 with two; dX 29.1, 22.6).  With
+// the low-rank tile in the stage (in_stage_cycles) tiles of 448 tokens pay in long calls: allocation-free
+// 4096 x 4096 forward, T = 8192, 270 us with 256-token tiles, 217 with 448; FP16 base 395, 250; T = 4096 (four
+// rounds, or three) 156, 172.
 PairTile pair_tile(const lrqat_layer& L, bool dx, int64_t T, int pairs, bool codes) {
   const int64_t rows = dx ? L.k : L.m, kdim = dx ? L.m : L.k;
   PairTile best{0, 0, 1, 0};
   int64_t best_cost = -1;
-  const bool beyond_l2 = codes && kdim * (rows + 2 * T) > (int64_t{100} << 20);   // one byte a weight, two a token value
   for (int ks = 1; ks <= 4; ks *= 2) {
     const int64_t slots = ks == 1 ? pairs : fused_pair_max_clusters(ks);
     const int64_t nk = (kdim / 64 + ks - 1) / ks;
@@ -365,11 +375,10 @@ PairTile pair_tile(const lrqat_layer& L, bool dx, int64_t T, int pairs, bool cod
       if (!codes && bt != 448 && bt > (phi_16bit(L) ? 192 : 256)) continue;
       const int64_t tiles = ((rows + 255) / 256) * ((T + bt - 1) / bt);
       const int64_t rounds = (tiles + slots - 1) / slots;
-      const int64_t stage = !codes ? in_stage_cycles(L, dx, bt)
-                            : bt <= 256 ? (dx ? 538 + bt * 60 / 100 : 513 + bt * 36 / 100)
-                                        : (dx ? 749 + (bt - 288) * 183 / 100 : 655 + (bt - 288) * 214 / 100);
-      const int64_t cost = rounds * (nk * stage + 2500 + 10 * bt + (ks > 1 ? 2500 + 8 * bt : 0));
-      if (best_cost < 0 || (beyond_l2 ? 8 * cost < 7 * best_cost : cost < best_cost)) {
+      const int64_t stage = !codes ? in_stage_cycles(L, dx, bt) : codes_stage_cycles(L, dx, bt);
+      int64_t cost = rounds * (nk * stage + 2500 + 10 * bt + (ks > 1 ? 2500 + 8 * bt : 0));
+      if (codes && !dx && L.m * L.k > kDeepCodes && (T + bt - 1) / bt > (T + 447) / 448) cost += cost / 64;
+      if (best_cost < 0 || cost < best_cost) {
         best_cost = cost;
         best = bt <= 256 ? PairTile{bt, 1, ks, cost} : PairTile{bt / 2, 2, ks, cost};
       }
@@ -379,13 +388,13 @@ PairTile pair_tile(const lrqat_layer& L, bool dx, int64_t T, int pairs, bool cod
 }
 // Whether a forward (rank up to 64) takes the codes pass rather than the in-stage tile: the pass (2.5 us
 // and 0.5 us per million weights; 10.8 us on 4096 x 4096, 34.7 on 13824 x 5120) and its GEMM against the
-// adapter layouts (2 us) and the slower stages.  Measured, codes / tile: 4096 x 4096 at T = 200 28.0 /
+// adapter layouts (2 us; the scale rows of group-wise layers 4 more) and the slower stages.  Measured, codes / tile: 4096 x 4096 at T = 200 28.0 /
 // 26.9 us, at T = 1024 37 / 47; 14336 x 4096 at T = 64 49 / 40 us, at T = 2999 (11008 x 4096) 164 / 216.
 bool prefer_codes_fwd(const lrqat_layer& L, int64_t T, int pairs) {
   constexpr double kCyclesPerUs = 1920.0;
   const double pass = (2.5 + 0.5e-6 * static_cast<double>(L.m) * static_cast<double>(L.k)) * kCyclesPerUs;
   const double codes = pass + static_cast<double>(pair_tile(L, false, T, pairs, true).cost);
-  const double tile = 2.0 * kCyclesPerUs + static_cast<double>(pair_tile(L, false, T, pairs, false).cost);
+  const double tile = (L.group_size ? 6.0 : 2.0) * kCyclesPerUs + static_cast<double>(pair_tile(L, false, T, pairs, false).cost);
   return codes <= tile;
 }
 
@@ -991,6 +1000,7 @@ static int linear_fwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
     a.bnp = tile.bnp;
     a.nacc = tile.nacc;
     a.ksplit = tile.ksplit;
+    a.deep = L.m * L.k > kDeepCodes;
     const int64_t tiles = ((L.m + 255) / 256) * ((T + tile.tokens() - 1) / tile.tokens());
     const int npairs = static_cast<int>(tile.ksplit > 1 || tiles < dev->sms / 2 ? tiles : dev->sms / 2);
     LRQAT_LAUNCH("fused_fwd", 1, stream, launch_fused_pair(fmode, ffmt, tm_tok, tm_phi, tm_rf, tm_sf, a, npairs, stream),
@@ -1185,6 +1195,7 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
       a.bnp = tile.bnp;
       a.nacc = tile.nacc;
       a.ksplit = tile.ksplit;
+      a.deep = L.m * L.k > kDeepCodes;
       const int64_t tiles = ((L.k + 255) / 256) * ((T + tile.tokens() - 1) / tile.tokens());
       const int npairs = static_cast<int>(tile.ksplit > 1 || tiles < dev->sms / 2 ? tiles : dev->sms / 2);
       LRQAT_LAUNCH("fused_dx", 1, stream,

@@ -83,3 +83,31 @@ def test_input_gradient(cid, spec, T, lowrank_path):
     LQ.get_device_status()
     assert t.isnan(dX[T]).all().item()
     assert t.equal(dX[:T], (dY.double() @ w).to(t.bfloat16))
+
+
+@pytest.mark.parametrize("tile", range(32, 449, 32))
+def test_every_tile_on_the_codes(tile, lowrank_path):
+    """Four 256-row blocks and 19 token tiles fill one round of 76 pairs, so each token count here takes
+    another tile; 12 stages, more than any ring holds.  Forward and dX."""
+    t = torch()
+    lowrank_path("codes")
+    T = 19 * tile - 5
+    spec = _spec(1024, 768, 16, group=256, phi=WL.PHI_INT_PACKED)
+    dl, X, w = _layer(spec, T, spec.k)
+    Y = t.full((T + 1, spec.m), float("nan"), dtype=t.bfloat16, device="cuda")
+    ws = t.empty(LQ.fwd_workspace_bytes(dl.layer, T), dtype=t.uint8, device="cuda")
+    LQ.linear_fwd(dl.layer, T, X.to(t.bfloat16), dl.phi0, dl.s, dl.A, dl.B, None, Y, ws)
+    assert t.isnan(Y[T]).all().item()
+    assert t.equal(Y[:T], (X.double() @ w.t()).to(t.bfloat16))
+
+    spec = _spec(768, 1024, 16, bits=2, asym=True)
+    dl, dY, w = _layer(spec, T, spec.m)
+    X = t.zeros((T, spec.k), dtype=t.bfloat16, device="cuda")
+    dX = t.full((T + 1, spec.k), float("nan"), dtype=t.bfloat16, device="cuda")
+    dA, dB = t.empty((spec.m, spec.r), device="cuda"), t.empty((spec.r, spec.k), device="cuda")
+    ws = t.empty(LQ.bwd_workspace_bytes(dl.layer, T), dtype=t.uint8, device="cuda")
+    LQ.linear_bwd(dl.layer, T, dY.to(t.bfloat16), X, dl.phi0, dl.s, dl.A, dl.B, None, dX, dA, dB, t.empty_like(dl.s),
+                  False, ws)
+    LQ.get_device_status()
+    assert t.isnan(dX[T]).all().item()
+    assert t.equal(dX[:T], (dY.double() @ w).to(t.bfloat16))
