@@ -358,14 +358,17 @@ int64_t codes_stage_cycles(const lrqat_layer& L, bool dx, int tokens) {
 // with 448 tokens, 1034 with 384, 1% cheaper by their cycles).  So the choice on the codes is within 3% of the
 // fastest of twelve tiles at 296 of 298 measured points, 8% at all.
 // Where one round leaves pairs idle, two or four pairs share a tile's contraction and add their sums through
-// distributed shared memory (T = 256, forward 26.6 us with one pair, 22.8 with two; dX 29.1, 22.6).  With
-// the low-rank tile in the stage (in_stage_cycles) tiles of 448 tokens pay in long calls: allocation-free
+// distributed shared memory (T = 256, forward 26.6 us with one pair, 22.8 with two; dX 29.1, 22.6).  A
+// cluster has one tile, so another round is another start of its CTAs, about 7 us (11008 x 8192 forward at
+// T = 64, three rounds of four pairs per tile 57 us, one pair per tile 44; allocation-free 4096 x 4096 FP16 base
+// at T = 2048, five rounds of two pairs 145, three of one 127).  With the low-rank tile in the stage (in_stage_cycles) tiles of 448 tokens pay in long calls: allocation-free
 // 4096 x 4096 forward, T = 8192, 270 us with 256-token tiles, 217 with 448; FP16 base 395, 250; T = 4096 (four
 // rounds, or three) 156, 172.
 PairTile pair_tile(const lrqat_layer& L, bool dx, int64_t T, int pairs, bool codes) {
   const int64_t rows = dx ? L.k : L.m, kdim = dx ? L.m : L.k;
   PairTile best{0, 0, 1, 0};
   int64_t best_cost = -1;
+  constexpr int64_t kClusterStart = 13000;   // 7 us
   for (int ks = 1; ks <= 4; ks *= 2) {
     const int64_t slots = ks == 1 ? pairs : fused_pair_max_clusters(ks);
     const int64_t nk = (kdim / 64 + ks - 1) / ks;
@@ -377,6 +380,7 @@ PairTile pair_tile(const lrqat_layer& L, bool dx, int64_t T, int pairs, bool cod
       const int64_t rounds = (tiles + slots - 1) / slots;
       const int64_t stage = !codes ? in_stage_cycles(L, dx, bt) : codes_stage_cycles(L, dx, bt);
       int64_t cost = rounds * (nk * stage + 2500 + 10 * bt + (ks > 1 ? 2500 + 8 * bt : 0));
+      if (ks > 1) cost += (rounds - 1) * kClusterStart;
       if (codes && !dx && L.m * L.k > kDeepCodes && (T + bt - 1) / bt > (T + 447) / 448) cost += cost / 64;
       if (best_cost < 0 || cost < best_cost) {
         best_cost = cost;
