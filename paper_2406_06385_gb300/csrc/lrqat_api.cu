@@ -390,16 +390,32 @@ PairTile pair_tile(const lrqat_layer& L, bool dx, int64_t T, int pairs, bool cod
   }
   return best;
 }
-// Whether a forward (rank up to 64) takes the codes pass rather than the in-stage tile: the pass (2.5 us
-// and 0.5 us per million weights; 10.8 us on 4096 x 4096, 34.7 on 13824 x 5120) and its GEMM against the
-// adapter layouts (2 us; the scale rows of group-wise layers 4 more) and the slower stages.  Measured, codes / tile: 4096 x 4096 at T = 200 28.0 /
-// 26.9 us, at T = 1024 37 / 47; 14336 x 4096 at T = 64 49 / 40 us, at T = 2999 (11008 x 4096) 164 / 216.
+// Microseconds of a forward (rank up to 64) on pairs, from the codes: the pass (2.5 us and 0.5 us per million weights;
+// 10.8 us on 4096 x 4096, 34.7 on 13824 x 5120) and its GEMM; with the in-stage tile: the adapter layouts
+// (2 us; the scale rows of group-wise layers 4 more) and the slower stages.
+constexpr double kCyclesPerUs = 1920.0;
+double codes_pass_us(const lrqat_layer& L) { return 2.5 + 0.5e-6 * static_cast<double>(L.m) * static_cast<double>(L.k); }
+double codes_fwd_us(const lrqat_layer& L, int64_t T, int pairs) {
+  return codes_pass_us(L) + static_cast<double>(pair_tile(L, false, T, pairs, true).cost) / kCyclesPerUs;
+}
+double tile_fwd_us(const lrqat_layer& L, int64_t T, int pairs) {
+  return (L.group_size ? 6.0 : 2.0) + static_cast<double>(pair_tile(L, false, T, pairs, false).cost) / kCyclesPerUs;
+}
+// Whether such a forward takes the codes pass rather than the in-stage tile.  Measured, codes / tile: 4096 x 4096 at
+// T = 200 28.0 / 26.9 us, at T = 1024 37 / 47; 14336 x 4096 at T = 64 49 / 40 us, at T = 2999 (11008 x 4096)
+// 164 / 216.
 bool prefer_codes_fwd(const lrqat_layer& L, int64_t T, int pairs) {
-  constexpr double kCyclesPerUs = 1920.0;
-  const double pass = (2.5 + 0.5e-6 * static_cast<double>(L.m) * static_cast<double>(L.k)) * kCyclesPerUs;
-  const double codes = pass + static_cast<double>(pair_tile(L, false, T, pairs, true).cost);
-  const double tile = (L.group_size ? 6.0 : 2.0) * kCyclesPerUs + static_cast<double>(pair_tile(L, false, T, pairs, false).cost);
-  return codes <= tile;
+  return codes_fwd_us(L, T, pairs) <= tile_fwd_us(L, T, pairs);
+}
+// The same on one SM (lrqat_set_gemm_variant 1), whose stage computes the low-rank tile beside the main product at
+// little cost: 4096 x 4096 at T = 1024 72 us with the tile, 85 with the codes, at T = 2048 127 and 135; 256 x 256
+// 12.4 and 18.4.  Decoding 16-bit bases takes 0.22 us more a stage than the codes (1664 x 13184 at T = 64 234 us
+// with the tile, 211 with the codes; 4096 x 4096 at T = 512 78 and 84, at T = 2048 143 and 135).
+bool prefer_codes_fwd_one_sm(const lrqat_layer& L, int64_t T, int sms) {
+  if (T >= 3072) return true;
+  if (!phi_16bit(L)) return false;
+  const int64_t rounds = (L.m / 128 * ((T + 447) / 448) + sms - 1) / sms;
+  return 0.22 * static_cast<double>(rounds * (L.k / 64)) > (T <= 64 ? 1.0 : 1.3) * codes_pass_us(L);
 }
 
 constexpr int kDwPairTokensPerStage = 64;   // the pair dW kernel's stage (dw_pair.cu)
@@ -875,15 +891,15 @@ static int linear_fwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
   FwdWs ws;
   fwd_ws_layout(L, T, allow_codes, workspace, &ws);
   const int r16 = round16(L.r);
+  const bool pair = use_pair();
+  const int path = g_lowrank_path.load(std::memory_order_relaxed);
   // A few tokens: their own kernel (ranks up to 64, unless a setting asks for a path).  Per call against
   // the faster of the codes and the in-stage tile, r = 32: 4096 x 4096 at T = 16 15.1 / 25.1 us,
   // 14336 x 4096 38 / 40, 256 x 256 7.0 / 9.6; its tile for 32 tokens spilled and lost (27 us).
-  const bool few = L.r <= 64 && T <= kFewTokens && g_gemm_variant.load(std::memory_order_relaxed) == 0 &&
-                   g_lowrank_path.load(std::memory_order_relaxed) == 0;
-  const bool pair = use_pair();
-  const int path = g_lowrank_path.load(std::memory_order_relaxed);
+  const bool few = L.r <= 64 && T <= kFewTokens && g_gemm_variant.load(std::memory_order_relaxed) == 0 && path == 0;
   const bool cb = L.r > 64 || (!few && allow_codes && path != 1 &&
-                               (path == 2 || !pair || prefer_codes_fwd(L, T, dev->sms / 2)));
+                               (path == 2 || (pair ? prefer_codes_fwd(L, T, dev->sms / 2)
+                                                   : prefer_codes_fwd_one_sm(L, T, dev->sms))));
   // the pair kernel reads K-major factor slices, so it takes B^T from the padded copy
   const bool direct = !cb && !few && !pair && direct_factors(L, A, B);
   if (cb) {
