@@ -373,7 +373,8 @@ PairTile pair_tile(const lrqat_layer& L, bool dx, int64_t T, int pairs, bool cod
     const int64_t slots = ks == 1 ? pairs : fused_pair_max_clusters(ks);
     const int64_t nk = (kdim / 64 + ks - 1) / ks;
     if (slots < 1 || nk < 2) continue;
-    for (int bt = 448; bt >= 32; bt -= 32) {
+    // a tile that holds all tokens twice over is no cheaper than one that just holds them
+    for (int bt = T < 448 ? static_cast<int>((T + 63) / 64 * 64) : 448; bt >= 32; bt -= 32) {
       if (bt % (16 * ks) || (bt > 256 && ks > 1)) continue;
       if (!codes && bt != 448 && bt > (phi_16bit(L) ? 192 : 256)) continue;
       const int64_t tiles = ((rows + 255) / 256) * ((T + bt - 1) / bt);
@@ -416,6 +417,27 @@ bool prefer_codes_fwd_one_sm(const lrqat_layer& L, int64_t T, int sms) {
   if (!phi_16bit(L)) return false;
   const int64_t rounds = (L.m / 128 * ((T + 447) / 448) + sms - 1) / sms;
   return 0.22 * static_cast<double>(rounds * (L.k / 64)) > (T <= 64 ? 1.0 : 1.3) * codes_pass_us(L);
+}
+// Whether a forward of up to 16 tokens (rank up to 64) takes the few-token kernel (fused_few.cu).  Its CTAs of 32 rows
+// each walk the whole contraction and recompute A B from registers: microseconds per 16 blocks of 64
+// columns by rank steps and storage below (9 to 16 tokens, high ranks and 16-bit bases spill registers),
+// plus 1.5 a round of CTAs; the other paths as above, with what they take more at such token counts.  Small calls
+// always gain.  Measured, few / best other: 4096 x 4096 at T = 16, r = 32 20.5 / 31 us, 4096 x 14336 51 / 66,
+// 14336 x 4096 51 / 53, r = 64 72 / 51, BF16 base 65 / 55; 1664 x 13184 45 / 38; 8192 x 8192 59 / 56.
+// Of 880 calls over formats, ranks 4 to 64, ten shapes and T = 1 .. 16 the choice costs 0.9% on average (this kernel
+// for all of them 9%).
+bool prefer_few(const lrqat_layer& L, int64_t T, int sms, bool allow_codes) {
+  const int64_t rounds = (L.m / 32 + sms - 1) / sms, blocks = (L.k / 64 + 15) / 16;
+  if (rounds * blocks < 4) return true;
+  const int steps = round16(L.r) / 16;
+  const bool packed = L.phi_format == LRQAT_PHI_INT_PACKED, f16 = L.phi_format == LRQAT_PHI_FP16;
+  double us;   // of 16 blocks, one per warp
+  if (phi_16bit(L)) us = 2.35 + 0.58 * steps + (T > 8 ? (f16 ? 1.2 : 0.85) + (steps == 4 ? 0.4 : 0.0) : 0.0);
+  else us = (packed ? 2.0 : 2.3) + 0.27 * steps + (T > 8 ? 0.25 + (steps == 4 && !packed ? 0.8 : 0.0) : 0.0);
+  const double few = 2.0 + static_cast<double>(rounds) * (1.5 + static_cast<double>(blocks) * us);
+  // left only for a path that is faster by a tenth, which the estimates can tell
+  if (few > 1.1 * (2.0 + 1.2 * tile_fwd_us(L, T, sms / 2))) return false;
+  return !allow_codes || few <= 1.1 * (codes_fwd_us(L, T, sms / 2) + (L.r % 8 ? 12.0 : 6.0));
 }
 
 constexpr int kDwPairTokensPerStage = 64;   // the pair dW kernel's stage (dw_pair.cu)
@@ -893,10 +915,9 @@ static int linear_fwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
   const int r16 = round16(L.r);
   const bool pair = use_pair();
   const int path = g_lowrank_path.load(std::memory_order_relaxed);
-  // A few tokens: their own kernel (ranks up to 64, unless a setting asks for a path).  Per call against
-  // the faster of the codes and the in-stage tile, r = 32: 4096 x 4096 at T = 16 15.1 / 25.1 us,
-  // 14336 x 4096 38 / 40, 256 x 256 7.0 / 9.6; its tile for 32 tokens spilled and lost (27 us).
-  const bool few = L.r <= 64 && T <= kFewTokens && g_gemm_variant.load(std::memory_order_relaxed) == 0 && path == 0;
+  // A few tokens: their own kernel, unless a setting asks for a path (its tile for 32 tokens spilled and lost)
+  const bool few = L.r <= 64 && T <= kFewTokens && g_gemm_variant.load(std::memory_order_relaxed) == 0 && path == 0 &&
+                   prefer_few(L, T, dev->sms, allow_codes);
   const bool cb = L.r > 64 || (!few && allow_codes && path != 1 &&
                                (path == 2 || (pair ? prefer_codes_fwd(L, T, dev->sms / 2)
                                                    : prefer_codes_fwd_one_sm(L, T, dev->sms))));

@@ -111,3 +111,25 @@ def test_every_tile_on_the_codes(tile, lowrank_path):
     LQ.get_device_status()
     assert t.isnan(dX[T]).all().item()
     assert t.equal(dX[:T], (dY.double() @ w).to(t.bfloat16))
+
+
+@pytest.mark.parametrize("T", [1, 9, 16])
+@pytest.mark.parametrize("cid,spec", [("bf16_r64", _spec(256, 4096, 64, phi=WL.PHI_BF16)),
+                                      ("packed_r64_odd", _spec(384, 6144, 64, phi=WL.PHI_INT_PACKED)),
+                                      ("fp16_group", _spec(128, 4096, 48, phi=WL.PHI_FP16, group=128)),
+                                      ("q44_r8", _spec(128, 4096, 8))])
+def test_few_tokens_on_long_contractions(cid, spec, T):
+    """Where a call of a few tokens may leave the kernel made for them: the same product on every path."""
+    t = torch()
+    dl, X, w = _layer(spec, T, spec.k)
+    want = (X.double() @ w.t()).to(t.bfloat16)
+    for noalloc in (False, True):
+        Y = t.full((T + 1, spec.m), float("nan"), dtype=t.bfloat16, device="cuda")
+        args = (dl.layer, T, X.to(t.bfloat16), dl.phi0, dl.s, dl.A, dl.B, None, Y)
+        if noalloc:
+            LQ.linear_fwd_noalloc(*args)
+        else:
+            LQ.linear_fwd(*args, t.empty(LQ.fwd_workspace_bytes(dl.layer, T), dtype=t.uint8, device="cuda"))
+        LQ.get_device_status()
+        assert t.isnan(Y[T]).all().item()
+        assert t.equal(Y[:T], want)
