@@ -204,7 +204,7 @@ int lrqat_linear_fwd_noalloc(const lrqat_layer* layer, int64_t T, const uint16_t
                              uint16_t* Y, lrqat_stream_t stream);
 
 /* Bytes of workspace lrqat_linear_bwd needs for T tokens (covers every setting of
- * lrqat_set_lowrank_path). */
+ * lrqat_set_lowrank_path, for ranks above 64 also of lrqat_set_gemm_variant). */
 size_t lrqat_bwd_workspace_bytes(const lrqat_layer* layer, int64_t T);
 
 /* Backward of the LR-QAT layer for the upstream gradient dY, with W_hat

@@ -443,10 +443,11 @@ bool prefer_few(const lrqat_layer& L, int64_t T, int sms, bool allow_codes) {
 constexpr int kDwPairTokensPerStage = 64;   // the pair dW kernel's stage (dw_pair.cu)
 // dW on CTA pairs (dw_pair.cu): 256 x 256 tiles, ranks up to 64, by the same setting as the
 // forward and dX GEMMs (lrqat_set_gemm_variant: not with 1, the one-SM kernels).
-bool pair_dw_shape(const lrqat_layer& L) {
-  return L.m % 256 == 0 && L.k % 256 == 0 && g_gemm_variant.load(std::memory_order_relaxed) != 1;
+bool pair_dw_shape(const lrqat_layer& L) { return L.m % 256 == 0 && L.k % 256 == 0; }
+bool pair_dw(const lrqat_layer& L) {
+  return pair_dw_shape(L) && g_gemm_variant.load(std::memory_order_relaxed) != 1;
 }
-bool use_pair_dw(const lrqat_layer& L) { return pair_dw_shape(L) && L.r <= 64; }
+bool use_pair_dw(const lrqat_layer& L) { return pair_dw(L) && L.r <= 64; }
 
 struct DwPlan {
   int nchunks, ni, nj, nsplit, tchunk, units;
@@ -528,10 +529,10 @@ DwPlan plan_dw(const lrqat_layer& L, int64_t T, int sms, bool pair) {
 // epilogue runs beside the next main loop, so pairs are taken when their busiest one has no more
 // tokens to pass than the busiest SM (4096 x 4096 at T = 8192, r = 256: 4 tiles against 7 of a quarter the
 // size; dW 552 -> 290 us).
-DwPlan plan_layer_dw(const lrqat_layer& L, int64_t T, int sms, int pairs) {
-  if (use_pair_dw(L)) return plan_dw(L, T, pairs, true);
+DwPlan plan_layer_dw(const lrqat_layer& L, int64_t T, int sms, int pairs, bool on_pairs) {
+  if (on_pairs && L.r <= 64) return plan_dw(L, T, pairs, true);
   const DwPlan one = plan_dw(L, T, sms, false);
-  if (L.r <= 64 || !pair_dw_shape(L) || pairs < 1) return one;
+  if (L.r <= 64 || !on_pairs || pairs < 1) return one;
   DwPlan p = one;
   p.pair = true;
   p.nchunks = 2;
@@ -1073,7 +1074,11 @@ size_t lrqat_bwd_workspace_bytes(const lrqat_layer* layer, int64_t T) {
   if (device_info(&dev) == LRQAT_OK) sms = dev->sms;
   const int pairs = dev ? dw_pair_max_pairs() : sms / 2;
   if (pairs < 1 && use_pair_dw(*layer)) return 0;
-  return bwd_ws_layout(*layer, T, plan_layer_dw(*layer, T, sms, pairs), nullptr, nullptr);
+  const size_t need = bwd_ws_layout(*layer, T, plan_layer_dw(*layer, T, sms, pairs, pair_dw(*layer)), nullptr, nullptr);
+  if (layer->r <= 64 || !pair_dw_shape(*layer)) return need;
+  // ranks above 64: the size of either kernel's plan, whatever lrqat_set_gemm_variant is at the call
+  const size_t other = bwd_ws_layout(*layer, T, plan_layer_dw(*layer, T, sms, pairs, !pair_dw(*layer)), nullptr, nullptr);
+  return need > other ? need : other;
 }
 
 // quantized: X is already the activation quantizer's output (as for linear_fwd_impl) and
@@ -1112,7 +1117,7 @@ static int linear_bwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
   LRQAT_TRY(device_info(&dev));
   const int dw_pairs = dw_pair_max_pairs();
   if (dw_pairs < 1 && use_pair_dw(L)) return fail(LRQAT_ERR_CUDA, "no cluster of two fits the dW kernel");
-  const DwPlan plan = plan_layer_dw(L, T, dev->sms, dw_pairs);
+  const DwPlan plan = plan_layer_dw(L, T, dev->sms, dw_pairs, pair_dw(L));
   const size_t need = bwd_ws_layout(L, T, plan, nullptr, nullptr);
   if (!workspace || workspace_bytes < need)
     return fail(LRQAT_ERR_WORKSPACE, "backward workspace of %zu bytes required, %zu given", need,
