@@ -402,11 +402,27 @@ double codes_fwd_us(const lrqat_layer& L, int64_t T, int pairs) {
 double tile_fwd_us(const lrqat_layer& L, int64_t T, int pairs) {
   return (L.group_size ? 6.0 : 2.0) + static_cast<double>(pair_tile(L, false, T, pairs, false).cost) / kCyclesPerUs;
 }
-// Whether such a forward takes the codes pass rather than the in-stage tile.  Measured, codes / tile: 4096 x 4096 at
-// T = 200 28.0 / 26.9 us, at T = 1024 37 / 47; 14336 x 4096 at T = 64 49 / 40 us, at T = 2999 (11008 x 4096)
-// 164 / 216.
-bool prefer_codes_fwd(const lrqat_layer& L, int64_t T, int pairs) {
-  return codes_fwd_us(L, T, pairs) <= tile_fwd_us(L, T, pairs);
+// The same with the in-stage tile on one SM, for a layer whose last pair of row blocks would be half empty: 1650 cycles
+// a stage (16-bit bases 2150) and 5000 a tile, but no launch in front of it where the GEMM reads A and B
+// themselves, and no scale rows.  Small layers take it: allocation-free forward of 640 x 384 at T = 1024 16.4
+// us (on pairs 18.4, group-wise 20.5), 384 x 640 group-wise at T = 16384 20.5 (28.7).
+double one_sm_fwd_us(const lrqat_layer& L, int64_t T, int sms, bool direct) {
+  const int64_t rounds = (L.m / 128 * ((T + 447) / 448) + sms - 1) / sms;
+  const int64_t cycles = rounds * (L.k / 64 * (phi_16bit(L) ? 2150 : 1650) + 5000);
+  return static_cast<double>(cycles) / kCyclesPerUs + (direct ? 0.0 : 2.0);
+}
+bool odd_blocks(const lrqat_layer& L) {
+  return L.m % 256 != 0 && g_gemm_variant.load(std::memory_order_relaxed) == 0;
+}
+// Whether such a forward takes the codes pass rather than the in-stage tile, by these and what the measured times
+// have beyond them: the second kernel's launch, the layouts that the pass needs where A and B cannot be read
+// directly, codes from HBM.  Measured, codes / tile: 4096 x 4096 at T = 200 30.7 / 30.7 us, at T = 1024 37 / 47;
+// 4096 x 14336 at T = 64 65 / 75, 1024 x 1024 at T = 200 18.4 / 16.4.  Of 810 calls (ten formats, nine shapes, T = 17 ..
+// 2048) the choice costs 0.3% on average, 13% at most.
+bool prefer_codes_fwd(const lrqat_layer& L, int64_t T, int sms, bool direct) {
+  const double codes = codes_fwd_us(L, T, sms / 2) + (direct ? 1.0 : 6.0);
+  if (odd_blocks(L) && codes + (L.act_bits == 8 ? 2.0 : 0.0) > one_sm_fwd_us(L, T, sms, direct)) return false;
+  return codes <= tile_fwd_us(L, T, sms / 2) + (L.group_size ? 1.0 : 0.0) + (L.m * L.k > kDeepCodes ? 5.0 : 0.0);
 }
 // The same on one SM (lrqat_set_gemm_variant 1), whose stage computes the low-rank tile beside the main product at
 // little cost: 4096 x 4096 at T = 1024 72 us with the tile, 85 with the codes, at T = 2048 127 and 135; 256 x 256
@@ -914,19 +930,21 @@ static int linear_fwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
   FwdWs ws;
   fwd_ws_layout(L, T, allow_codes, workspace, &ws);
   const int r16 = round16(L.r);
-  const bool pair = use_pair();
+  const bool direct_ab = direct_factors(L, A, B);
   const int path = g_lowrank_path.load(std::memory_order_relaxed);
   // A few tokens: their own kernel, unless a setting asks for a path (its tile for 32 tokens spilled and lost)
   const bool few = L.r <= 64 && T <= kFewTokens && g_gemm_variant.load(std::memory_order_relaxed) == 0 && path == 0 &&
                    prefer_few(L, T, dev->sms, allow_codes);
   const bool cb = L.r > 64 || (!few && allow_codes && path != 1 &&
-                               (path == 2 || (pair ? prefer_codes_fwd(L, T, dev->sms / 2)
-                                                   : prefer_codes_fwd_one_sm(L, T, dev->sms))));
+                               (path == 2 || (use_pair() ? prefer_codes_fwd(L, T, dev->sms, direct_ab)
+                                                         : prefer_codes_fwd_one_sm(L, T, dev->sms))));
+  const bool pair = use_pair() && (cb || !odd_blocks(L) ||
+                                   one_sm_fwd_us(L, T, dev->sms, direct_ab) > tile_fwd_us(L, T, dev->sms / 2));
   // the pair kernel reads K-major factor slices, so it takes B^T from the padded copy
-  const bool direct = !cb && !few && !pair && direct_factors(L, A, B);
+  const bool direct = !cb && !few && !pair && direct_ab;
   if (cb) {
     // the codes of every weight, once per call (from A and B themselves when the factors are direct)
-    if (!direct_factors(L, A, B))
+    if (!direct_ab)
       LRQAT_LAUNCH("adapter_layouts", 1, stream,
                    launch_adapter_layouts(A, B, L.m, L.k, L.r, r16, nullptr, nullptr, ws.at, ws.b_pad, stream),
                    "adapter layouts");
