@@ -318,7 +318,8 @@ int lrqat_set_dw_schedule(int schedule);
  * CTA pairs run tcgen05 MMAs of 256 rows across the two SMs of a cluster, each SM holding
  * half of the token operand (256 weight rows x up to 448 tokens per pair); dW on pairs needs m and
  * k multiples of 256 (256 x 256 tiles).  The one-SM kernels take 128 rows per SM.  0 (the default) =
- * pairs wherever they were measured faster, which is wherever the shapes allow; 1 = the
+ * pairs wherever they were measured faster, which is wherever the shapes allow but for forwards of a few
+ * tokens and of small layers with m an odd multiple of 128; 1 = the
  * one-SM kernels always; 2 = pairs wherever the shapes allow.  All give the same codes;
  * outputs agree up to fp32 summation order.  Process-wide; the environment variable LRQAT_GEMM_VARIANT ("auto",
  * "single" or "pair") gives the start value, read once when the library is loaded.
@@ -334,7 +335,7 @@ int lrqat_set_gemm_variant(int variant);
  * = codes in the backward, and in the forward by a cost model (the pass costs two bytes of HBM
  * traffic per weight, the tile a low-rank MMA chain per stage); never in the allocation-free forward,
  * whose scratch does not hold them.  Up to 16 tokens the forward takes a kernel of its own that forms
- * the codes in registers (unless this or lrqat_set_gemm_variant is set).  Ranks above 64
+ * the codes in registers, where an estimate finds no faster path (unless this or lrqat_set_gemm_variant is set).  Ranks above 64
  * always take the codes pass.  dW reads the codes where
  * the pair kernels take it (m and k multiples of 256, up to 7 bits) and computes its own
  * low-rank tile elsewhere.  All settings give the same codes up to
