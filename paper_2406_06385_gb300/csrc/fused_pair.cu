@@ -13,22 +13,21 @@
 // tokens or two of up to 224; CTA c holds half of each one's; the host picks smaller token tiles where
 // 448 leave pairs idle, and two or four pairs per tile where those do too: pair_tile in
 // lrqat_api.cu), one 64-wide slice of the contraction per stage:
-//   * token ring (four to eight slots per CTA; three beside the low-rank tile of 448 tokens): loader warps bring this CTA's token halves
-//     (SW128) with TMA whose completion lands on the leader's barrier; each slot also holds this
-//     CTA's W_hat tile of the stage;
-//   * factor ring (four or eight slots; two for 16-bit bases beside the low-rank tile of 448 tokens): the stored base of this CTA's rows (completion
-//     on its own barrier; only its own producers read it), with it the stage's scales (and zero
-//     offsets) where the producers apply them (dX, group-wise forward), and with the low-rank tile
-//     this CTA's half (32 rows) of the second factor's slice (completion on the leader's
-//     barrier: the low-rank MMA reads both halves);
+//   * token ring (four to eight slots per CTA; three with the low-rank tile in 448-token tiles): loader
+//     warps bring this CTA's token halves (SW128) with TMA whose completion lands on the leader's
+//     barrier; each slot also holds this CTA's W_hat tile of the stage;
+//   * factor ring (four or eight slots; two for 16-bit bases with the low-rank tile in 448-token tiles):
+//     the stored base of this CTA's rows (completion on its own barrier; only its own producers read
+//     it), with it the stage's scales (and zero offsets) where the producers apply them (dX, group-wise
+//     forward), and with the low-rank tile this CTA's half (32 rows) of the second factor's slice
+//     (completion on the leader's barrier: the low-rank MMA reads both halves);
 //   * in the leader, one thread per accumulator issues its main product (M = 256, 4 MMAs per stage)
 //     and, with the low-rank tile in the stage, another the tile L = RF SF^T (M = 256, N = 64) into one of
 //     four TMEM buffers after one accumulator or the one buffer after two (which one thread issues
 //     then), so that neither waits behind the other's barriers; every commit is multicast to both CTAs;
-//   * sixteen producer warps per CTA, in four groups that take every fourth stage each (one group
-//     beside the low-rank tile of 448 tokens), build this CTA's W_hat tile exactly as the one-SM kernel
-//     does, and drain this CTA's 128 rows of the
-//     accumulators in the epilogue.
+//   * sixteen producer warps per CTA, in four groups that take every fourth stage each (one group with
+//     the low-rank tile in 448-token tiles), build this CTA's W_hat tile exactly as the one-SM kernel
+//     does, and drain this CTA's 128 rows of the accumulators in the epilogue.
 // One barrier per slot in the leader counts the stage's token bytes and both CTAs' "W_hat
 // written" events, so the MMA thread tests one barrier per stage; the peer's events ("W_hat
 // written", "L read", "accumulators drained") travel as 16-byte copies into the leader's shared

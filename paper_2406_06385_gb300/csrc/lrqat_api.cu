@@ -301,8 +301,8 @@ std::atomic<int> g_dw_schedule{dw_schedule_from_env()};
 // wherever they were measured faster, which is every GEMM (an odd number of 128-row blocks leaves half
 // a pair without rows in the last one; 1664 x 13184 at T = 512, both odd, forward + backward 415 us on
 // one SM, 246 on pairs), but for a few tokens (prefer_few) and for forwards of small layers with such a block
-// (one_sm_fwd_us); 1 = the one-SM kernel (fused_gemm.cu) always; 2 = pairs always.  LRQAT_GEMM_VARIANT ("auto" / "single" / "pair") sets the start value
-// once, when the library is loaded.
+// (one_sm_fwd_us); 1 = the one-SM kernel (fused_gemm.cu) always; 2 = pairs always.  LRQAT_GEMM_VARIANT
+// ("auto" / "single" / "pair") sets the start value once, when the library is loaded.
 int gemm_variant_from_env() {
   const char* v = std::getenv("LRQAT_GEMM_VARIANT");
   if (v && std::strcmp(v, "single") == 0) return 1;
