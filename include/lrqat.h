@@ -335,9 +335,9 @@ int lrqat_set_gemm_variant(int variant);
  * = codes in the backward, and in the forward by a cost model (the pass costs two bytes of HBM
  * traffic per weight, the tile a low-rank MMA chain per stage); never in the allocation-free forward,
  * whose scratch does not hold them.  Up to 16 tokens the forward takes a kernel of its own that forms
- * the codes in registers, where an estimate finds no faster path (unless this or lrqat_set_gemm_variant is set).  Ranks above 64
- * always take the codes pass.  dW reads the codes where
- * the pair kernels take it (m and k multiples of 256, up to 7 bits) and computes its own
+ * the codes in registers, where an estimate finds no faster path (unless this or
+ * lrqat_set_gemm_variant is set).  Ranks above 64 always take the codes pass.  dW reads the codes
+ * where the pair kernels take it (m and k multiples of 256, up to 7 bits) and computes its own
  * low-rank tile elsewhere.  All settings give the same codes up to
  * fp32 summation order of A B.  Process-wide; the environment variable LRQAT_LOWRANK_PATH
  * ("auto", "tile" or "codes") gives the start value, read once when the library is loaded.

@@ -484,8 +484,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       const int row_g = row_block(rb2) + row;
       const bool has_rows = rb2 * 2 * BM + static_cast<int>(rank) * BM < args.rows;
       const uint32_t z_row = MODE == FUSED_FWD_PC && ZP ? pack_rn_bf16x2(args.zero[row_g], args.zero[row_g]) : 0u;
-      // Group c's stages of the tile (gg % 4 == c; one group: every stage).  A ready barrier costs a test of ~110 cycles and the
-      // proxy fence and reports ~100 more, whatever the warp does between them: with all sixteen warps in
+      // Group c's stages of the tile (gg % 4 == c; one group: every stage).  A ready barrier costs a test of
+      // ~110 cycles and the proxy fence and reports ~100 more, whatever the warp does between them: with all sixteen warps in
       // every stage these made a stage on the codes 770 cycles (4096 x 4096, 32-token tiles), four groups
       // in flight pay them side by side (596 cycles; 256-token tiles 863 -> 700).  With the low-rank tile
       // a group has a TMEM buffer of its own, so four low-rank tiles are in flight instead of one
@@ -684,7 +684,8 @@ cudaError_t launch_pair_one(const CUtensorMap& a, const CUtensorMap& b, const CU
   if constexpr (!NL && G == 4)   // beside the low-rank tile, two accumulators take one producer group
     if (args.nacc == 2) return launch_pair_one<MODE, FMT, ZP, UB, NL, 1>(a, b, c, d, args, npairs, stream);
   using PR = PairRing<FMT, NL, MODE == FUSED_DX || MODE == FUSED_FWD_GROUP, G>;
-  if (args.bnp * args.nacc > PR::MAX_TILE || (G == 1 && (args.bnp != BNP || args.ksplit != 1))) return cudaErrorInvalidValue;
+  if (args.bnp * args.nacc > PR::MAX_TILE) return cudaErrorInvalidValue;
+  if (G == 1 && (args.bnp != BNP || args.ksplit != 1)) return cudaErrorInvalidValue;
   if (args.ksplit > 1 && (args.nacc != 1 || args.bnp % (16 * args.ksplit))) return cudaErrorInvalidValue;
   const uint32_t smem = PR::smem(args.bnp * args.nacc, args.deep);
   static bool configured[kMaxDevices] = {};

@@ -361,7 +361,8 @@ int64_t codes_stage_cycles(const lrqat_layer& L, bool dx, int tokens) {
 // distributed shared memory (T = 256, forward 26.6 us with one pair, 22.8 with two; dX 29.1, 22.6).  A
 // cluster has one tile, so another round is another start of its CTAs, about 7 us (11008 x 8192 forward at
 // T = 64, three rounds of four pairs per tile 57 us, one pair per tile 44; allocation-free 4096 x 4096 FP16 base
-// at T = 2048, five rounds of two pairs 145, three of one 127).  With the low-rank tile in the stage (in_stage_cycles) tiles of 448 tokens pay in long calls: allocation-free
+// at T = 2048, five rounds of two pairs 145, three of one 127).
+// With the low-rank tile in the stage (in_stage_cycles) tiles of 448 tokens pay in long calls: allocation-free
 // 4096 x 4096 forward, T = 8192, 270 us with 256-token tiles, 217 with 448; FP16 base 395, 250; T = 4096 (four
 // rounds, or three) 156, 172.
 PairTile pair_tile(const lrqat_layer& L, bool dx, int64_t T, int pairs, bool codes) {
