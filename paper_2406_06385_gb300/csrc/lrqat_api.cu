@@ -404,16 +404,22 @@ double tile_fwd_us(const lrqat_layer& L, int64_t T, int pairs) {
   return (L.group_size ? 6.0 : 2.0) + static_cast<double>(pair_tile(L, false, T, pairs, false).cost) / kCyclesPerUs;
 }
 // The same with the in-stage tile on one SM, for a layer whose last pair of row blocks would be half empty: 1650 cycles
-// a stage (16-bit bases 2150) and 5000 a tile, but no launch in front of it where the GEMM reads A and B
+// a stage (16-bit bases 1950, group scales 100 more) and 5000 a tile, but no launch in front of it where the GEMM reads A and B
 // themselves, and no scale rows.  Small layers take it: allocation-free forward of 640 x 384 at T = 1024 16.4
 // us (on pairs 18.4, group-wise 20.5), 384 x 640 group-wise at T = 16384 20.5 (28.7).
 double one_sm_fwd_us(const lrqat_layer& L, int64_t T, int sms, bool direct) {
   const int64_t rounds = (L.m / 128 * ((T + 447) / 448) + sms - 1) / sms;
-  const int64_t cycles = rounds * (L.k / 64 * (phi_16bit(L) ? 2150 : 1650) + 5000);
+  const int64_t stage = (phi_16bit(L) ? 1950 : 1650) + (L.group_size ? 100 : 0);
+  const int64_t cycles = rounds * (L.k / 64 * stage + 5000);
   return static_cast<double>(cycles) / kCyclesPerUs + (direct ? 0.0 : 2.0);
 }
-bool odd_blocks(const lrqat_layer& L) {
-  return L.m % 256 != 0 && g_gemm_variant.load(std::memory_order_relaxed) == 0;
+// What the launches of the pair path's scale rows and of the quantizer between its kernels (no dependent launches
+// across it) take beyond its estimate.
+double launch_us(const lrqat_layer& L) { return (L.group_size ? 1.0 : 0.0) + (L.act_bits == 8 ? 2.0 : 0.0); }
+// Whether that is a choice.  Fewer than 64 tokens on many rows are not (11136 x 1024 group-wise at T = 17 37 us on
+// one SM, 27 on pairs; at T = 64 25 and 27).
+bool odd_blocks(const lrqat_layer& L, int64_t T) {
+  return L.m % 256 != 0 && (T >= 64 || L.m <= 2048) && g_gemm_variant.load(std::memory_order_relaxed) == 0;
 }
 // Whether such a forward takes the codes pass rather than the in-stage tile, by these and what the measured times
 // have beyond them: the second kernel's launch, the layouts that the pass needs where A and B cannot be read
@@ -422,7 +428,7 @@ bool odd_blocks(const lrqat_layer& L) {
 // 2048) the choice costs 0.3% on average, 13% at most.
 bool prefer_codes_fwd(const lrqat_layer& L, int64_t T, int sms, bool direct) {
   const double codes = codes_fwd_us(L, T, sms / 2) + (direct ? 1.0 : 6.0);
-  if (odd_blocks(L) && codes + (L.act_bits == 8 ? 2.0 : 0.0) > one_sm_fwd_us(L, T, sms, direct)) return false;
+  if (odd_blocks(L, T) && codes + (L.act_bits == 8 ? 2.0 : 0.0) > one_sm_fwd_us(L, T, sms, direct)) return false;
   return codes <= tile_fwd_us(L, T, sms / 2) + (L.group_size ? 1.0 : 0.0) + (L.m * L.k > kDeepCodes ? 5.0 : 0.0);
 }
 // The same on one SM (lrqat_set_gemm_variant 1), whose stage computes the low-rank tile beside the main product at
@@ -939,8 +945,8 @@ static int linear_fwd_impl(const lrqat_layer* layer, int64_t T, const uint16_t* 
   const bool cb = L.r > 64 || (!few && allow_codes && path != 1 &&
                                (path == 2 || (use_pair() ? prefer_codes_fwd(L, T, dev->sms, direct_ab)
                                                          : prefer_codes_fwd_one_sm(L, T, dev->sms))));
-  const bool pair = use_pair() && (cb || !odd_blocks(L) ||
-                                   one_sm_fwd_us(L, T, dev->sms, direct_ab) > tile_fwd_us(L, T, dev->sms / 2));
+  const bool pair = use_pair() && (cb || !odd_blocks(L, T) || one_sm_fwd_us(L, T, dev->sms, direct_ab) >
+                                                               tile_fwd_us(L, T, dev->sms / 2) + launch_us(L));
   // the pair kernel reads K-major factor slices, so it takes B^T from the padded copy
   const bool direct = !cb && !few && !pair && direct_ab;
   if (cb) {
