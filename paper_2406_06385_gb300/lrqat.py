@@ -137,9 +137,10 @@ def _stream(stream) -> Optional[int]:
     # The raw handle, where this PyTorch has it: a Stream object took 2.9 us of a call's host time, this 0.2 us
     # (a few-token forward alone, to the end of its kernels: 31.5 -> 30.0 us).
     if torch.cuda.is_initialized():
-        raw, device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
-        if raw is not None and device is not None:
-            return raw(device())
+        try:
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        except AttributeError:
+            pass
     return torch.cuda.current_stream().cuda_stream
 
 
